@@ -82,9 +82,9 @@ typedef struct {
   int32_t fused_step_min_tokens; /* fl_server_backward_step applies AdamW inside the weight-
                              * gradient GEMMs when the pending call has at least this many
                              * tokens, else it runs the backward and then fl_server_step;
-                             * 0 -> 4608 (the crossover measured on GB300: with fewer tokens
-                             * the weight-gradient main loop is too short to hide the 26 B per
-                             * parameter of the fused update); 1 -> always fused */
+                             * 0 -> the library's choice (fused at every token count where a
+                             * block holds 2^24 matrix weights or more, as measured on GB300);
+                             * 1 -> always fused */
   int32_t n_replicas;       /* server-hierarchical strategy (§3.3) on one GPU: 0 or 1 = one
                              * server; 2..4 = that many replicas in one handle, each with its
                              * own parameters, gradients and Adam state (arena of replica r at
@@ -155,8 +155,8 @@ int fl_server_step(fl_server_t h, float lr);
  * matrices of every block runs in the epilogue of their weight-gradient GEMMs: the fp32
  * matrix gradients are never written to memory, and the update's traffic overlaps the
  * tensor-core work.  The bias and LayerNorm vectors get one AdamW launch at the end.
- * Otherwise (gradients accumulated by earlier backward calls, or fewer tokens in the
- * pending call than cfg.fused_step_min_tokens) it runs the two calls as they are.
+ * Otherwise (gradients accumulated by earlier backward calls, or a call that
+ * cfg.fused_step_min_tokens leaves unfused) it runs the two calls as they are.
  * Results equal backward + step up to fp32 rounding.  Errors: as fl_server_backward. */
 int fl_server_backward_step(fl_server_t h, const void* const grad_out[], void* const grad_in[], float lr);
 

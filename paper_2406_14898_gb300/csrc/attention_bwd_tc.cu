@@ -130,19 +130,6 @@ FL_DEV uint8_t* stage_chunk(uint8_t* stage, int r, int j) {
   return stage + (j >> 3) * (TB * 128) + r * 128 + (((j & 7) ^ (r & 7)) << 4);
 }
 
-// 2-D tiled store of one box from shared memory to global memory (bulk-group completion).
-FL_DEV void tma_store_2d(const CUtensorMap* m, const void* src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(m)),
-               "r"(smem_u32(src)), "r"(x), "r"(y)
-               : "memory");
-}
-FL_DEV void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// The committed bulk stores have read their shared memory (it may be written again).
-FL_DEV void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// The committed bulk stores are complete.
-FL_DEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // Adds the column sums of a staged tile over its first `rows` rows to out[0..HD); called by
 // all 256 threads.  Warp wp takes the HD/64 16-byte chunks wp*HD/64 ..: LPC = 32*64/HD
 // lanes per chunk, lane l reading rows l % LPC, + LPC, ... (8 consecutive lanes read 8

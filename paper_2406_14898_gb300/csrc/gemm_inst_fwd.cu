@@ -1,6 +1,6 @@
-// Instantiations of the tcgen05 GEMM for the forward (A and B K-major) operand layout.
+// Instantiations of the CTA-pair tcgen05 GEMM for the forward (A and B K-major) operand layout.
 #include "gemm_tc.cuh"
 
 namespace fl_gemm {
-FL_GEMM_INSTANTIATE(false, false)
+FL_GEMM_INSTANTIATE_PAIR(, false, false)
 }  // namespace fl_gemm

@@ -6,56 +6,61 @@
 #include "gemm_tc.cuh"
 
 namespace fl_gemm {
-#define FL_GEMM_EXTERN(AMN, BMN, FAM)                                                                   \
-  extern template int pair_slots<AMN, BMN, FAM>();                                                      \
-  extern template int launch_pair<AMN, BMN, FAM>(const fl_gemm_args*, const Problems&, const Epi&, int*, cudaStream_t);  \
-  extern template int launch<256, AMN, BMN, FAM>(const fl_gemm_args*, const Problems&, const Epi&, int*, cudaStream_t); \
-  extern template int launch<128, AMN, BMN, FAM>(const fl_gemm_args*, const Problems&, const Epi&, int*, cudaStream_t);
-#define FL_GEMM_EXTERN_ALL(AMN, BMN)                                                                   \
-  FL_GEMM_EXTERN(AMN, BMN, FAM_PLAIN) FL_GEMM_EXTERN(AMN, BMN, FAM_GELU) FL_GEMM_EXTERN(AMN, BMN, FAM_RESID) \
-  FL_GEMM_EXTERN(AMN, BMN, FAM_ROPE) FL_GEMM_EXTERN(AMN, BMN, FAM_ADAMW)
-FL_GEMM_EXTERN_ALL(false, false)
-FL_GEMM_EXTERN_ALL(false, true)
-FL_GEMM_EXTERN_ALL(true, true)
+FL_GEMM_INSTANTIATE_PAIR(extern, false, false)
+FL_GEMM_INSTANTIATE_PAIR(extern, false, true)
+FL_GEMM_INSTANTIATE_PAIR(extern, true, true)
+FL_GEMM_INSTANTIATE_LONG(extern)
+FL_GEMM_INSTANTIATE_SINGLE(extern, false, false)
+FL_GEMM_INSTANTIATE_SINGLE(extern, false, true)
+FL_GEMM_INSTANTIATE_SINGLE(extern, true, true)
 
-// Tile shape: 0 = 128 x 128 on one SM, 1 = 128 x 256 on one SM, 2 = 256 x 256 on a CTA pair.
+// Contractions this long take the AdamW epilogue that leaves the operand ring six stages (its
+// own operands in registers, FAM_ADAMW_LONG) instead of the one whose TMA ring takes two of
+// them.  Measured, two 4096 x 16384 weights per launch, ring / registers: 730 / 790 us at K =
+// 2048, 832 / 807 at 3072, 1038 / 878 at 4096, 1381 / 1156 at 6144, 1693 / 1450 at 8192.
+constexpr int ADAMW_LONG_K = 3072;
+
+// Tile shapes: FL_TILE_* - 1.
+enum { SHAPE_128 = 0, SHAPE_256 = 1, SHAPE_PAIR256 = 2 };
+
+template <bool AMN, bool BMN, int FAM>
+int dispatch_shape(int shape, const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cudaStream_t st) {
+  switch (shape) {
+    case SHAPE_PAIR256: return launch_pair<256, AMN, BMN, FAM>(a, pr, e, status, st);
+    case SHAPE_256: return launch<256, AMN, BMN, FAM>(a, pr, e, status, st);
+    default: return launch<128, AMN, BMN, FAM>(a, pr, e, status, st);
+  }
+}
 template <bool AMN, bool BMN>
 int dispatch_layout(int fam, int shape, const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status,
                     cudaStream_t st) {
-  if (shape == 2) {
-    switch (fam) {
-      case FAM_GELU: return launch_pair<AMN, BMN, FAM_GELU>(a, pr, e, status, st);
-      case FAM_RESID: return launch_pair<AMN, BMN, FAM_RESID>(a, pr, e, status, st);
-      case FAM_ROPE: return launch_pair<AMN, BMN, FAM_ROPE>(a, pr, e, status, st);
-      case FAM_ADAMW: return launch_pair<AMN, BMN, FAM_ADAMW>(a, pr, e, status, st);
-      default: return launch_pair<AMN, BMN, FAM_PLAIN>(a, pr, e, status, st);
-    }
-  }
-  const bool wide = shape == 1;
   switch (fam) {
-    case FAM_GELU: return wide ? launch<256, AMN, BMN, FAM_GELU>(a, pr, e, status, st) : launch<128, AMN, BMN, FAM_GELU>(a, pr, e, status, st);
-    case FAM_RESID: return wide ? launch<256, AMN, BMN, FAM_RESID>(a, pr, e, status, st) : launch<128, AMN, BMN, FAM_RESID>(a, pr, e, status, st);
-    case FAM_ROPE: return wide ? launch<256, AMN, BMN, FAM_ROPE>(a, pr, e, status, st) : launch<128, AMN, BMN, FAM_ROPE>(a, pr, e, status, st);
-    case FAM_ADAMW: return wide ? launch<256, AMN, BMN, FAM_ADAMW>(a, pr, e, status, st) : launch<128, AMN, BMN, FAM_ADAMW>(a, pr, e, status, st);
-    default: return wide ? launch<256, AMN, BMN, FAM_PLAIN>(a, pr, e, status, st) : launch<128, AMN, BMN, FAM_PLAIN>(a, pr, e, status, st);
+    case FAM_GELU: return dispatch_shape<AMN, BMN, FAM_GELU>(shape, a, pr, e, status, st);
+    case FAM_RESID: return dispatch_shape<AMN, BMN, FAM_RESID>(shape, a, pr, e, status, st);
+    case FAM_ROPE: return dispatch_shape<AMN, BMN, FAM_ROPE>(shape, a, pr, e, status, st);
+    case FAM_ADAMW: return dispatch_shape<AMN, BMN, FAM_ADAMW>(shape, a, pr, e, status, st);
+    default: return dispatch_shape<AMN, BMN, FAM_PLAIN>(shape, a, pr, e, status, st);
   }
 }
 
 int dispatch_fam(int fam, int shape, bool amn, bool bmn, const fl_gemm_args* a, const Problems& pr, const Epi& e,
                  int* status, cudaStream_t st) {
+  if (fam == FAM_ADAMW && shape == SHAPE_PAIR256 && amn && a->K >= ADAMW_LONG_K)
+    return launch_pair<256, true, true, FAM_ADAMW_LONG>(a, pr, e, status, st);
   if (!amn && !bmn) return dispatch_layout<false, false>(fam, shape, a, pr, e, status, st);
   if (!amn && bmn) return dispatch_layout<false, true>(fam, shape, a, pr, e, status, st);
   return dispatch_layout<true, true>(fam, shape, a, pr, e, status, st);
 }
 
+template <int PBN>
 int pair_slots_for(int fam, bool amn, bool bmn) {
-#define FL_SLOTS(AMN, BMN)                                          \
-  switch (fam) {                                                    \
-    case FAM_GELU: return pair_slots<AMN, BMN, FAM_GELU>();         \
-    case FAM_RESID: return pair_slots<AMN, BMN, FAM_RESID>();       \
-    case FAM_ROPE: return pair_slots<AMN, BMN, FAM_ROPE>();         \
-    case FAM_ADAMW: return pair_slots<AMN, BMN, FAM_ADAMW>();       \
-    default: return pair_slots<AMN, BMN, FAM_PLAIN>();              \
+#define FL_SLOTS(AMN, BMN)                                               \
+  switch (fam) {                                                         \
+    case FAM_GELU: return pair_slots<PBN, AMN, BMN, FAM_GELU>();         \
+    case FAM_RESID: return pair_slots<PBN, AMN, BMN, FAM_RESID>();       \
+    case FAM_ROPE: return pair_slots<PBN, AMN, BMN, FAM_ROPE>();         \
+    case FAM_ADAMW: return pair_slots<PBN, AMN, BMN, FAM_ADAMW>();       \
+    default: return pair_slots<PBN, AMN, BMN, FAM_PLAIN>();              \
   }
   if (!amn && !bmn) { FL_SLOTS(false, false) }
   if (!amn && bmn) { FL_SLOTS(false, true) }
@@ -175,7 +180,7 @@ int run(const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cu
   const bool amn = a->a_mn_major != 0, bmn = a->b_mn_major != 0;
   const int fam = family_of(a->epilogue);
   const int batch = pr.n;
-  if (a->tile == FL_TILE_256x256_PAIR && pair_slots_for(fam, amn, bmn) <= 0)
+  if (a->tile == FL_TILE_256x256_PAIR && pair_slots_for<256>(fam, amn, bmn) <= 0)
     return fl_internal_error(FL_ERR_UNSUPPORTED, "gemm: this device cannot hold the CTA-pair kernel");
   if (a->tile != FL_TILE_AUTO) return dispatch_fam(fam, a->tile - 1, amn, bmn, a, pr, e, status, st);
   // Tile shape: 256 columns (on a CTA pair where the device can hold pairs) unless
@@ -183,12 +188,12 @@ int run(const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cu
   int shape = 0;
   if ((a->N % 256) == 0) {
     const int sms = num_sms();
-    const int pairs = pair_slots_for(fam, amn, bmn);
+    const int pairs = pair_slots_for<256>(fam, amn, bmn);
     const long t128 = (long)batch * ((a->M + BM - 1) / BM) * (a->N / 128);
     const double eff128 = double(t128) / double(((t128 + sms - 1) / sms) * sms);
     double eff_wide;
     if (pairs > 0) {
-      const long tp = (long)batch * ((a->M + PAIR_BM - 1) / PAIR_BM) * (a->N / PAIR_BN);
+      const long tp = (long)batch * ((a->M + PAIR_BM - 1) / PAIR_BM) * (a->N / 256);
       eff_wide = double(tp) / double(((tp + pairs - 1) / pairs) * pairs);
       shape = 2;
     } else {

@@ -108,11 +108,13 @@ cudaError_t fl_func_smem(const void* func, int bytes) {
 
 namespace {
 
-// Tokens from which fl_server_backward_step fuses the AdamW update into the weight-gradient
-// GEMMs (measured on GB300 at H 4096, F 16384: fused / separate step 119.1 / 118.3 ms at
-// 4096 tokens, 159.9 / 164.2 ms at 6144; the crossover depends on the tokens, the length of
-// the weight-gradient main loop, not on the widths).
-constexpr int FL_FUSED_STEP_MIN_TOKENS = 4608;
+// Matrix weights per block from which fl_server_backward_step fuses the AdamW update into the
+// weight-gradient GEMMs (at every token count), unless cfg.fused_step_min_tokens says otherwise.
+// Measured on GB300, one block, fused / separate step: H 4096 (201M weights) 1.45 / 1.61 ms at 128
+// tokens, 1.79 / 2.02 at 1024, 3.21 / 3.58 at 3072; H 2048 (50M) 563 / 590, 673 / 719, 1237 / 1296
+// us; H 1024 (12.6M) 302 / 303, 348 / 350, 567 / 565; H 512 203 / 196; H 256 184 / 170 (a small
+// weight's update costs less than the longer epilogue).
+constexpr int64_t FL_FUSED_STEP_MIN_WEIGHTS = int64_t(1) << 24;
 
 constexpr uint64_t GOLDEN = 0x9E3779B97F4A7C15ull;
 uint64_t mix64_host(uint64_t z) {
@@ -945,10 +947,11 @@ extern "C" int fl_server_backward(fl_server_t h, const void* const grad_out[], v
 extern "C" int fl_server_backward_step(fl_server_t h, const void* const grad_out[], void* const grad_in[], float lr) {
   if (!h) return fl_internal_error(FL_ERR_INVALID_ARG, "backward_step: null handle");
   if (!h->pending) return set_err(h, FL_ERR_STATE, "backward_step: no pending forward");
-  // no fusion while gradients from an earlier backward are pending, nor for calls too
-  // short for the weight-gradient main loop to hide the update
-  const int min_tokens = h->cfg.fused_step_min_tokens > 0 ? h->cfg.fused_step_min_tokens : FL_FUSED_STEP_MIN_TOKENS;
-  if (!h->grads_zero || h->Tr < min_tokens) {
+  // no fusion while gradients from an earlier backward are pending, nor where the separate
+  // update is faster
+  const int min_tokens = h->cfg.fused_step_min_tokens;
+  const bool fused = min_tokens > 0 ? h->Tr >= min_tokens : h->mat_stride >= FL_FUSED_STEP_MIN_WEIGHTS;
+  if (!h->grads_zero || !fused) {
     if (int rc = backward_impl(h, grad_out, grad_in)) return rc;
     return fl_server_step(h, lr);
   }

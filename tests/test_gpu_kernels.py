@@ -490,6 +490,52 @@ def test_gemm_adamw_epilogue(F, M, N, K, mn, tile):
     np.testing.assert_array_equal(bits(wbf), bits(wf.to(torch.bfloat16)))
 
 
+@pytest.mark.parametrize("K", [8, 2048, 3064, 3072, 3080])
+def test_gemm_adamw_epilogue_against_exact(F, K):
+    """The fused update on both sides of the contraction length where its epilogue changes,
+    ragged rows, two problems in one launch: against the update in 64 bits of the very
+    gradient the GEMM makes.  Bound per weight: half an ulp of the result and of the update's
+    last product, and 8 ulps of lr * ratio for the moments, the quotient and the root (each
+    correctly rounded or within one ulp); gradients span the range down to zero."""
+    M, N = 264, 512
+    rng = np.random.default_rng(K)
+    lr, b1, b2, eps, wd, t = 1e-3, 0.9, 0.999, 1e-8, 0.01, 3
+    f = [np.float32(x) for x in (lr, b1, b2, eps, wd)]
+    inv1, inv2 = np.float32(1.0 / np.float32(1.0 - b1 ** t)), np.float32(1.0 / np.float32(1.0 - b2 ** t))
+    A = rnd_bf16_f64(rng, (M, K))
+    A[:8] = 0.0  # rows with a zero gradient
+    A[8:64] *= 2.0 ** -rng.integers(0, 60, (56, 1))
+    dA, lda = _store(A, True)
+    dB, ldb = _store(rnd_bf16_f64(rng, (N, K)), True)
+    w0 = (0.05 * rng.standard_normal((2, M, N))).astype(np.float32)
+    w0[:, :, :64] = 0.0
+    m0 = (0.01 * rng.standard_normal((2, M, N))).astype(np.float32)
+    v0 = (1e-3 * rng.random((2, M, N))).astype(np.float32)
+    m0[:, :8], v0[:, :8] = 0.0, 0.0
+    m0[:, 8:64] = 0.0
+    v0[:, 8:64] = 0.0
+    g = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    F.gemm(M, N, K, dA, lda, 1, dB, ldb, 1, g, N, epilogue=F.FL_EPI_STORE_F32, tile=F.FL_TILE_256x256_PAIR)
+    w, m, v = dev_f32(w0), dev_f32(m0), dev_f32(v0)
+    wb = torch.empty((2, M, N), dtype=torch.bfloat16, device="cuda")
+    F.fl_k_gemm_multi([F.gemm_args(M, N, K, dA, lda, 1, dB, ldb, 1, w[r], N, epilogue=F.FL_EPI_ADAMW, adam_m=m[r], adam_v=v[r],
+                                   aux_out=wb[r], ld_aux_out=N, lr=lr, beta1=b1, beta2=b2, eps=eps, weight_decay=wd,
+                                   inv_bc1=float(inv1), inv_bc2=float(inv2), tile=F.FL_TILE_256x256_PAIR) for r in range(2)])
+    torch.cuda.synchronize()
+    lr, b1, b2, eps, wd = (float(x) for x in f)
+    g = f64(g)
+    me = b1 * m0.astype(np.float64) + (1.0 - b1) * g
+    ve = b2 * v0.astype(np.float64) + (1.0 - b2) * g * g
+    ratio = me * float(inv1) / (np.sqrt(ve * float(inv2)) + eps)
+    we = w0 - lr * (ratio + wd * w0.astype(np.float64))
+    u = 2.0 ** -24
+    # the new first moment is a sum of two terms of either sign: its rounding is relative to them
+    terms = (b1 * np.abs(m0) + (1.0 - b1) * np.abs(g)) * float(inv1) / (np.sqrt(ve * float(inv2)) + eps)
+    bound = u * (1.01 * np.abs(we) + 16.0 * lr * (terms + wd * np.abs(w0))) + 1e-30
+    assert (np.abs(f64(w) - we) <= bound).all()
+    np.testing.assert_array_equal(bits(wb), bits(w.to(torch.bfloat16)))
+
+
 def test_zero_size_calls(F):
     """Degenerate sizes: a GEMM of M = 0 rows, LayerNorm forward and backward over T = 0
     rows, AdamW over 0 parameters, column sums over 0 rows, and attention over one empty
