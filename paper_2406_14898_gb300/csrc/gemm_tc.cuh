@@ -597,6 +597,18 @@ FL_DEV void batch_tile(int tile, int num_m, int num_n, Raster rs, int& r, int& m
   tile_coords(tile - r * per, num_m, num_n, rs, mb, nb);
 }
 
+// Shared-memory descriptor of an operand stage, and its step from one 16-deep MMA to the next:
+// K-major, the next 16 elements are 32 bytes further along the swizzled row; MN-major, the next
+// 16 k-rows 16 * 128 bytes further (the descriptor counts 16-byte units).
+template <bool MN>
+FL_DEV uint64_t stage_desc(uint32_t base) {
+  return MN ? smem_desc_sw128(base, BK * 128, 1024) : smem_desc_sw128(base, 16, 1024);
+}
+template <bool MN>
+__host__ __device__ constexpr uint64_t kstep_desc() {
+  return MN ? 128 : 2;
+}
+
 template <int BN, bool A_MN, bool B_MN, int FAM>
 __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ GemmMaps<FAM> maps, Epi epi, int M, int N, int K, int batch, Raster raster,
@@ -654,30 +666,32 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
   pdl_wait();  // the previous kernel's outputs (operands, epilogue inputs) are complete
   pdl_trigger();
 
+  // The producer and MMA loops are run by whole (converged) warps, one elected lane issuing: the
+  // loop state stays in uniform registers, which the TMA and MMA instructions take directly.
+  // With the loops inside one lane's branch a k-block cost at least 270 ns whatever the tile
+  // (4096 columns, K = 16384, 77 rows on 256 x 128 pairs: 79 us; 63 us this way), and the full
+  // 256 x 256 tiles at 2048 rows ran 5-8% slower (QKV projection 131 -> 123 us).
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------ TMA producer
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t armed = 0, last_par = 0;  // per-stage bit masks for the teardown drain
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        int r, mb, nb;
-        batch_tile(tile, num_m, num_n, raster, r, mb, nb);
-        const CUtensorMap* tmA = &maps.a[r];
-        const CUtensorMap* tmB = &maps.b[r];
-        for (int kb = 0; kb < num_k; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1)) {
-            report_status(status, FL_DEV_TIMEOUT_EMPTY);
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&full[stage], C::STAGE_BYTES);
-          armed |= 1u << stage;
-          last_par = (last_par & ~(1u << stage)) | (phase << stage);
+    // -------------------------------------------------------------- TMA producer
+    int stage = 0, used = 0;  // used: stages armed so far (up to STAGES), for the teardown drain
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      int r, mb, nb;
+      batch_tile(tile, num_m, num_n, raster, r, mb, nb);
+      const CUtensorMap* tmA = &maps.a[r];
+      const CUtensorMap* tmB = &maps.b[r];
+      for (int kb = 0; kb < num_k; ++kb) {
+        if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
+          if (lane == 0) report_status(status, FL_DEV_TIMEOUT_EMPTY);
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           const int k0 = kb * BK;
           uint8_t* a_dst = sA + stage * C::A_BYTES;
           uint8_t* b_dst = sB + stage * C::B_BYTES;
+          mbar_arrive_expect_tx(&full[stage], C::STAGE_BYTES);
           if (!A_MN) {
             tma_load_2d(a_dst, tmA, &full[stage], k0, mb * BM);
           } else {
@@ -690,66 +704,64 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
 #pragma unroll
             for (int j = 0; j < BN / 64; ++j) tma_load_2d(b_dst + j * 64 * BK * 2, tmB, &full[stage], nb * BN + 64 * j, k0);
           }
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+        }
+        __syncwarp();
+        if (used < STAGES) ++used;
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
         }
       }
-      // Drain: every armed stage's copies must have landed before shared memory is released.
-      for (int s = 0; s < STAGES; ++s)
-        if (armed & (1u << s))
-          if (!mbar_wait(&full[s], (last_par >> s) & 1)) report_status(status, FL_DEV_TIMEOUT_DRAIN);
     }
+    // Drain: every armed stage's copies must have landed before shared memory is released.
+    // Stage s was last armed in the phase before the current one, or in it where s < stage.
+    for (int s = 0; s < used; ++s)
+      if (!mbar_wait_warp(&full[s], s < stage ? phase : phase ^ 1))
+        if (lane == 0) report_status(status, FL_DEV_TIMEOUT_DRAIN);
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------ MMA issuer
-      constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, A_MN, B_MN);
-      int stage = 0;
-      uint32_t phase = 0;
-      int local = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++local) {
-        const int acc = local & 1;
-        const uint32_t acc_par = (local >> 1) & 1;
-        if (!mbar_wait(&acc_empty[acc], acc_par ^ 1)) {
-          report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
+    // -------------------------------------------------------------- MMA issuer
+    constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, A_MN, B_MN);
+    int stage = 0;
+    uint32_t phase = 0;
+    int local = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++local) {
+      const int acc = local & 1;
+      const uint32_t acc_par = (local >> 1) & 1;
+      if (!mbar_wait_warp(&acc_empty[acc], acc_par ^ 1)) {
+        if (lane == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + acc * BN;
+      for (int kb = 0; kb < num_k; ++kb) {
+        if (!mbar_wait_warp(&full[stage], phase)) {
+          if (lane == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
-        for (int kb = 0; kb < num_k; ++kb) {
-          if (!mbar_wait(&full[stage], phase)) {
-            report_status(status, FL_DEV_TIMEOUT_FULL);
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a_base = smem_u32(sA + stage * C::A_BYTES);
-          const uint32_t b_base = smem_u32(sB + stage * C::B_BYTES);
+        if (elect_one()) {
+          const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + stage * C::A_BYTES));
+          const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + stage * C::B_BYTES));
 #pragma unroll
-          for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-            // K-major: next 16 elements are 32 bytes further along the swizzled row.
-            // MN-major: next 16 k-rows are 16 * 128 bytes further.
-            const uint64_t adesc = A_MN ? smem_desc_sw128(a_base + kk * 2048, BK * 128, 1024)
-                                        : smem_desc_sw128(a_base + kk * 32, 16, 1024);
-            const uint64_t bdesc = B_MN ? smem_desc_sw128(b_base + kk * 2048, BK * 128, 1024)
-                                        : smem_desc_sw128(b_base + kk * 32, 16, 1024);
-            umma_bf16(d_tmem, adesc, bdesc, IDESC, (kb | kk) != 0 ? 1u : 0u);
-          }
+          for (int kk = 0; kk < BK / UMMA_K; ++kk)
+            umma_bf16(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC, (kb | kk) != 0 ? 1u : 0u);
           umma_commit(&empty[stage]);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+          if (kb == num_k - 1) umma_commit(&acc_full[acc]);
         }
-        if (ok) umma_commit(&acc_full[acc]);
+        __syncwarp();
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
+        }
       }
-      // Drain: all MMAs issued by this thread complete before TMEM is released.
-      umma_commit(drain);
-      if (!mbar_wait(drain, 0)) report_status(status, FL_DEV_TIMEOUT_DRAIN);
     }
+    // Drain: all MMAs issued by this warp complete before TMEM is released.
+    if (elect_one()) umma_commit(drain);
+    __syncwarp();
+    if (!mbar_wait_warp(drain, 0) && lane == 0) report_status(status, FL_DEV_TIMEOUT_DRAIN);
   } else {
     // -------------------------------------------------------------- epilogue warps
     auto place = [&](int tile, TilePos& t) {
@@ -862,28 +874,25 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
   pdl_trigger();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------ TMA producer (both CTAs)
-      const uint32_t full0 = mapa_shared(smem_u32(full), 0);  // the even CTA's full[0]
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t armed = 0, last_par = 0;  // per-stage bit masks for the teardown drain
-      bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += n_pairs) {
-        int r, mb, nb;
-        batch_tile(tile, num_m, num_n, raster, r, mb, nb);
-        const CUtensorMap* tmA = &maps.a[r];
-        const CUtensorMap* tmB = &maps.b[r];
-        const int m0 = mb * PAIR_BM + int(rank) * 128, n0 = nb * PBN + int(rank) * (PBN / 2);
-        for (int kb = 0; kb < num_k; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1)) {
-            report_status(status, FL_DEV_TIMEOUT_EMPTY);
-            ok = false;
-            break;
-          }
+    // -------------------------------------------------------------- TMA producer (both CTAs)
+    const uint32_t full0 = mapa_shared(smem_u32(full), 0);  // the even CTA's full[0]
+    int stage = 0, used = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int tile = pair; tile < num_tiles && ok; tile += n_pairs) {
+      int r, mb, nb;
+      batch_tile(tile, num_m, num_n, raster, r, mb, nb);
+      const CUtensorMap* tmA = &maps.a[r];
+      const CUtensorMap* tmB = &maps.b[r];
+      const int m0 = mb * PAIR_BM + int(rank) * 128, n0 = nb * PBN + int(rank) * (PBN / 2);
+      for (int kb = 0; kb < num_k; ++kb) {
+        if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
+          if (lane == 0) report_status(status, FL_DEV_TIMEOUT_EMPTY);
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           if (leader) mbar_arrive_expect_tx(&full[stage], 2 * C::STAGE_BYTES);
-          armed |= 1u << stage;
-          last_par = (last_par & ~(1u << stage)) | (phase << stage);
           const uint32_t fb = full0 + 8u * stage;
           const int k0 = kb * BK;
           uint8_t* a_dst = sA + stage * C::A_BYTES;
@@ -900,20 +909,22 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
 #pragma unroll
             for (int j = 0; j < PBN / 128; ++j) tma_load_2d_pair(b_dst + j * 64 * BK * 2, tmB, fb, n0 + 64 * j, k0);
           }
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+        }
+        __syncwarp();
+        if (used < STAGES) ++used;
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
         }
       }
-      // Drain: a stage loaded in phase p is released (empty phase p completes) only after
-      // the MMAs that read it, and so after its copies landed.
-      for (int s = 0; s < STAGES; ++s)
-        if (armed & (1u << s))
-          if (!mbar_wait(&empty[s], (last_par >> s) & 1)) report_status(status, FL_DEV_TIMEOUT_DRAIN);
     }
+    // Drain: a stage loaded in phase p is released (empty phase p completes) only after
+    // the MMAs that read it, and so after its copies landed.
+    for (int s = 0; s < used; ++s)
+      if (!mbar_wait_warp(&empty[s], s < stage ? phase : phase ^ 1))
+        if (lane == 0) report_status(status, FL_DEV_TIMEOUT_DRAIN);
   } else if (warp == 1) {
-    if (leader && lane == 0) {
+    if (leader) {
       // ------------------------------------------------------------ MMA issuer (even CTA)
       constexpr uint32_t IDESC = umma_idesc_bf16(PAIR_BM, PBN, A_MN, B_MN);
       int stage = 0;
@@ -923,42 +934,42 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
       for (int tile = pair; tile < num_tiles && ok; tile += n_pairs, ++local) {
         const int acc = local & 1;
         const uint32_t acc_par = (local >> 1) & 1;
-        if (!mbar_wait(&acc_empty[acc], acc_par ^ 1)) {
-          report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
+        if (!mbar_wait_warp(&acc_empty[acc], acc_par ^ 1)) {
+          if (lane == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * PBN;
         for (int kb = 0; kb < num_k; ++kb) {
-          if (!mbar_wait(&full[stage], phase)) {
-            report_status(status, FL_DEV_TIMEOUT_FULL);
+          if (!mbar_wait_warp(&full[stage], phase)) {
+            if (lane == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a_base = smem_u32(sA + stage * C::A_BYTES);
-          const uint32_t b_base = smem_u32(sB + stage * C::B_BYTES);
+          if (elect_one()) {
+            const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + stage * C::A_BYTES));
+            const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + stage * C::B_BYTES));
 #pragma unroll
-          for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-            const uint64_t adesc = A_MN ? smem_desc_sw128(a_base + kk * 2048, BK * 128, 1024)
-                                        : smem_desc_sw128(a_base + kk * 32, 16, 1024);
-            const uint64_t bdesc = B_MN ? smem_desc_sw128(b_base + kk * 2048, BK * 128, 1024)
-                                        : smem_desc_sw128(b_base + kk * 32, 16, 1024);
-            umma_bf16_pair(d_tmem, adesc, bdesc, IDESC, (kb | kk) != 0 ? 1u : 0u);
+            for (int kk = 0; kk < BK / UMMA_K; ++kk)
+              umma_bf16_pair(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC,
+                             (kb | kk) != 0 ? 1u : 0u);
+            umma_commit_pair(&empty[stage], 3);
+            if (kb == num_k - 1) umma_commit_pair(&acc_full[acc], 3);
           }
-          umma_commit_pair(&empty[stage], 3);
+          __syncwarp();
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1;
           }
         }
-        if (ok) umma_commit_pair(&acc_full[acc], 3);
       }
-      // Drain: all MMAs issued by this thread (and their arrivals) complete before the pair
+      // Drain: all MMAs issued by this warp (and their arrivals) complete before the pair
       // releases TMEM and shared memory.
-      umma_commit_pair(drain, 1);
-      if (!mbar_wait(drain, 0)) report_status(status, FL_DEV_TIMEOUT_DRAIN);
+      if (elect_one()) umma_commit_pair(drain, 1);
+      __syncwarp();
+      if (!mbar_wait_warp(drain, 0) && lane == 0) report_status(status, FL_DEV_TIMEOUT_DRAIN);
     }
   } else {
     // -------------------------------------------------------------- epilogue warps (both CTAs)

@@ -6,6 +6,17 @@
 
 FL_DEV uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
+// True on one lane of the (converged) warp, the same one every time.
+FL_DEV bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p)::"memory");
+  return p != 0;
+}
+
 // ------------------------------------------------------------------ mbarrier
 FL_DEV void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -41,6 +52,11 @@ FL_DEV bool mbar_wait(uint64_t* bar, uint32_t parity) {
       if (mbar_try_wait(a, parity)) return true;
     if (globaltimer_ns() - t0 > FL_WAIT_NS) return false;
   }
+}
+
+// mbar_wait by a whole converged warp; every lane returns the same answer.
+FL_DEV bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity)) != 0;
 }
 
 // ------------------------------------------------------------------ TMA
