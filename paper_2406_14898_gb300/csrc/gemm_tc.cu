@@ -20,11 +20,15 @@ FL_GEMM_INSTANTIATE_SINGLE(extern, true, true)
 // 2048, 832 / 807 at 3072, 1038 / 878 at 4096, 1381 / 1156 at 6144, 1693 / 1450 at 8192.
 constexpr int ADAMW_LONG_K = 3072;
 
-// Tile shapes: FL_TILE_* - 1.
-enum { SHAPE_128 = 0, SHAPE_256 = 1, SHAPE_PAIR256 = 2 };
+// Tile shapes: FL_TILE_* - 1, and two narrow ones that only the library picks.
+enum { SHAPE_128 = 0, SHAPE_256 = 1, SHAPE_PAIR256 = 2, SHAPE_64 = 3, SHAPE_PAIR128 = 4 };
 
 template <bool AMN, bool BMN, int FAM>
 int dispatch_shape(int shape, const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cudaStream_t st) {
+  if constexpr (FAM != FAM_ADAMW) {
+    if (shape == SHAPE_PAIR128) return launch_pair<128, AMN, BMN, FAM>(a, pr, e, status, st);
+    if (shape == SHAPE_64) return launch<64, AMN, BMN, FAM>(a, pr, e, status, st);
+  }
   switch (shape) {
     case SHAPE_PAIR256: return launch_pair<256, AMN, BMN, FAM>(a, pr, e, status, st);
     case SHAPE_256: return launch<256, AMN, BMN, FAM>(a, pr, e, status, st);
@@ -175,6 +179,44 @@ bool d_is_f32(const fl_gemm_args* a) {
   return a->d_dtype == FL_DT_F32 || mode == FL_EPI_STORE_F32 || mode == FL_EPI_ACCUM_F32 || mode == FL_EPI_ADAMW;
 }
 
+// The tile shape with the least estimated time: waves of tiles, each as long as its main loop
+// or its epilogue, and the fill and last epilogue.  Measured on GB300 (ns per 64-deep k-block
+// of a CTA or pair with one tile at a time; us for the fixed part): 256 x 256 on a pair 295 and
+// 9.7, 256 x 128 on a pair 230 and 5.4, 128 x 128 262 and 6.1, 128 x 64 180 and 5.0 (the fixed
+// parts of the narrow tiles set so that H 256 steps take 128 x 64: 119 us, 135 on pairs).  So one
+// wave of narrow tiles over all SMs beats a wide tile on a few of them: 4096 columns, K = 16384
+// take 85 / 63 / 73 / 51 us (in that order) at 77 rows, 87 / 65 / 75 / 96 at 512; and wide tiles
+// win once they fill the device: 170 / 224 / 271 / 319 us at 2048 rows.
+int pick_shape(const fl_gemm_args* a, int batch, int fam, int pairs) {
+  struct Shape {
+    int id, bm, bn;
+    double k_us, fixed_us, epi_us;  // per k-block; once; least per tile
+  };
+  static constexpr Shape shapes[] = {{SHAPE_PAIR256, 256, 256, 0.295, 9.7, 4.0},
+                                     {SHAPE_PAIR128, 256, 128, 0.230, 5.4, 2.0},
+                                     {SHAPE_128, 128, 128, 0.262, 6.1, 2.0},
+                                     {SHAPE_64, 128, 64, 0.180, 5.0, 2.0},
+                                     {SHAPE_256, 128, 256, 0.400, 9.7, 4.0}};
+  const int num_k = (a->K + BK - 1) / BK;
+  int best = SHAPE_128;
+  double best_us = 0;
+  for (const Shape& s : shapes) {
+    const bool pair = s.bm == 256, narrow = s.id == SHAPE_PAIR128 || s.id == SHAPE_64;
+    const int slots = pair ? pairs : num_sms();
+    // 128 x 256 stands in for the pair where the device cannot hold it; weight updates have no narrow tiles
+    if (slots <= 0 || a->N % s.bn || (s.id == SHAPE_256 && pairs > 0) || (narrow && fam == FAM_ADAMW)) continue;
+    const long tiles = (long)batch * ((a->M + s.bm - 1) / s.bm) * (a->N / s.bn);
+    const long waves = (tiles + slots - 1) / slots;
+    const double main_us = num_k * s.k_us;
+    const double us = waves * (main_us > s.epi_us ? main_us : s.epi_us) + s.fixed_us;
+    if (best_us == 0 || us < best_us) {
+      best = s.id;
+      best_us = us;
+    }
+  }
+  return best;
+}
+
 // Tile shape for the launch (see fl_k_gemm) and the dispatch.
 int run(const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cudaStream_t st) {
   const bool amn = a->a_mn_major != 0, bmn = a->b_mn_major != 0;
@@ -183,26 +225,7 @@ int run(const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cu
   if (a->tile == FL_TILE_256x256_PAIR && pair_slots_for<256>(fam, amn, bmn) <= 0)
     return fl_internal_error(FL_ERR_UNSUPPORTED, "gemm: this device cannot hold the CTA-pair kernel");
   if (a->tile != FL_TILE_AUTO) return dispatch_fam(fam, a->tile - 1, amn, bmn, a, pr, e, status, st);
-  // Tile shape: 256 columns (on a CTA pair where the device can hold pairs) unless
-  // 128 x 128 tiles give clearly fewer idle SM slots in the last wave.
-  int shape = 0;
-  if ((a->N % 256) == 0) {
-    const int sms = num_sms();
-    const int pairs = pair_slots_for<256>(fam, amn, bmn);
-    const long t128 = (long)batch * ((a->M + BM - 1) / BM) * (a->N / 128);
-    const double eff128 = double(t128) / double(((t128 + sms - 1) / sms) * sms);
-    double eff_wide;
-    if (pairs > 0) {
-      const long tp = (long)batch * ((a->M + PAIR_BM - 1) / PAIR_BM) * (a->N / 256);
-      eff_wide = double(tp) / double(((tp + pairs - 1) / pairs) * pairs);
-      shape = 2;
-    } else {
-      const long t256 = (long)batch * ((a->M + BM - 1) / BM) * (a->N / 256);
-      eff_wide = double(t256) / double(((t256 + sms - 1) / sms) * sms);
-      shape = 1;
-    }
-    if (eff128 > eff_wide * 1.15) shape = 0;
-  }
+  const int shape = pick_shape(a, batch, fam, pair_slots_for<256>(fam, amn, bmn));
   return dispatch_fam(fam, shape, amn, bmn, a, pr, e, status, st);
 }
 

@@ -75,11 +75,11 @@ struct AdamRing {
   static constexpr int BYTES = WARPS * SLOTS * SLOT;
 };
 
-// Epilogue warps of a family and the shared memory they work in: the AdamW ring, or one
-// 32x64 fp32 chunk per warp.
-template <int FAM>
+// Epilogue warps of a family at tile width BN (64 columns give eight warps nothing to share)
+// and the shared memory they work in: the AdamW ring, or one 32x64 fp32 chunk per warp.
+template <int FAM, int BN>
 struct EpiCfg {
-  static constexpr int WARPS = FAM == FAM_ADAMW ? AdamRing::WARPS : FAM == FAM_ADAMW_LONG ? 4 : 8;
+  static constexpr int WARPS = FAM == FAM_ADAMW ? AdamRing::WARPS : FAM == FAM_ADAMW_LONG || BN == 64 ? 4 : 8;
   static constexpr int THREADS = 64 + 32 * WARPS;
   static constexpr int BYTES = FAM == FAM_ADAMW ? AdamRing::BYTES : WARPS * 32 * 64 * 4;
   static constexpr int BARS = FAM == FAM_ADAMW ? WARPS * AdamRing::SLOTS : 0;
@@ -93,15 +93,20 @@ constexpr int ring_stages(int bytes, int epi_bytes) {
   return n < 6 ? n : 6;
 }
 
+// k-blocks per stage: the products of one k-block of a 128 x 64 tile are shorter than a
+// stage's barrier round trip, so a stage of that shape holds two (4096 columns, K = 16384, 77
+// rows: 67 -> 51 us; the 256 x 128 pair tile, left three such stages, would lose: 63 -> 68 us).
+
 template <int BN, int FAM>
 struct Cfg {
+  static constexpr int KSUB = BN == 64 ? 2 : 1;
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = BN * BK * 2;
-  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = ring_stages(STAGE_BYTES, EpiCfg<FAM>::BYTES);
+  static constexpr int STAGE_BYTES = KSUB * (A_BYTES + B_BYTES);
+  static constexpr int STAGES = ring_stages(STAGE_BYTES, EpiCfg<FAM, BN>::BYTES);
   static constexpr int TMEM_COLS = 2 * BN;  // double-buffered accumulator
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EpiCfg<FAM>::BYTES + BAR_BYTES + 1024 /*align*/;
-  static_assert((2 * STAGES + 5 + EpiCfg<FAM>::BARS) * 8 + 4 <= BAR_BYTES, "barriers");
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EpiCfg<FAM, BN>::BYTES + BAR_BYTES + 1024 /*align*/;
+  static_assert((2 * STAGES + 5 + EpiCfg<FAM, BN>::BARS) * 8 + 4 <= BAR_BYTES, "barriers");
 };
 
 struct Epi {
@@ -389,7 +394,7 @@ template <int FAM, int BN, typename Place, typename Release>
 FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int warp, int lane, int t0, int step,
                           int num_tiles, uint64_t* acc_full, int* status, Place place, Release release) {
   constexpr int RB = EpiBatch<FAM>::RB, DEPTH = EpiBatch<FAM>::DEPTH;
-  constexpr int HALVES = EpiCfg<FAM>::WARPS / 4;    // warps per lane quarter
+  constexpr int HALVES = EpiCfg<FAM, BN>::WARPS / 4;    // warps per lane quarter
   constexpr int WCH = BN / (64 * HALVES);           // chunks per warp and tile
   constexpr int NBC = 16 / RB;                      // batches per chunk
   static_assert(NBC % DEPTH == 0, "whole rounds of register sets per chunk");
@@ -610,24 +615,24 @@ __host__ __device__ constexpr uint64_t kstep_desc() {
 }
 
 template <int BN, bool A_MN, bool B_MN, int FAM>
-__global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
+__global__ void __launch_bounds__(EpiCfg<FAM, BN>::THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ GemmMaps<FAM> maps, Epi epi, int M, int N, int K, int batch, Raster raster,
                    int* status) {
   using C = Cfg<BN, FAM>;
-  constexpr int STAGES = C::STAGES;
+  constexpr int STAGES = C::STAGES, KSUB = C::KSUB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + STAGES * C::A_BYTES;
+  uint8_t* sB = smem + STAGES * KSUB * C::A_BYTES;
   uint8_t* epi_smem = smem + STAGES * C::STAGE_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(epi_smem + EpiCfg<FAM>::BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(epi_smem + EpiCfg<FAM, BN>::BYTES);
   uint64_t* full = bars;
   uint64_t* empty = bars + STAGES;
   uint64_t* acc_full = bars + 2 * STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
   uint64_t* ring_full = drain + 1;  // the AdamW ring's
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ring_full + EpiCfg<FAM>::BARS);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ring_full + EpiCfg<FAM, BN>::BARS);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -643,10 +648,10 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], EpiCfg<FAM>::WARPS);
+      mbar_init(&acc_empty[a], EpiCfg<FAM, BN>::WARPS);
     }
     mbar_init(drain, 1);
-    for (int i = 0; i < EpiCfg<FAM>::BARS; ++i) mbar_init(&ring_full[i], 1);
+    for (int i = 0; i < EpiCfg<FAM, BN>::BARS; ++i) mbar_init(&ring_full[i], 1);
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -681,28 +686,31 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
       batch_tile(tile, num_m, num_n, raster, r, mb, nb);
       const CUtensorMap* tmA = &maps.a[r];
       const CUtensorMap* tmB = &maps.b[r];
-      for (int kb = 0; kb < num_k; ++kb) {
+      for (int kb = 0; kb < num_k; kb += KSUB) {
         if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
           if (lane == 0) report_status(status, FL_DEV_TIMEOUT_EMPTY);
           ok = false;
           break;
         }
         if (elect_one()) {
-          const int k0 = kb * BK;
-          uint8_t* a_dst = sA + stage * C::A_BYTES;
-          uint8_t* b_dst = sB + stage * C::B_BYTES;
           mbar_arrive_expect_tx(&full[stage], C::STAGE_BYTES);
-          if (!A_MN) {
-            tma_load_2d(a_dst, tmA, &full[stage], k0, mb * BM);
-          } else {
 #pragma unroll
-            for (int j = 0; j < BM / 64; ++j) tma_load_2d(a_dst + j * 64 * BK * 2, tmA, &full[stage], mb * BM + 64 * j, k0);
-          }
-          if (!B_MN) {
-            tma_load_2d(b_dst, tmB, &full[stage], k0, nb * BN);
-          } else {
+          for (int q = 0; q < KSUB; ++q) {  // a k-block past K reads zeros
+            const int k0 = (kb + q) * BK;
+            uint8_t* a_dst = sA + (stage * KSUB + q) * C::A_BYTES;
+            uint8_t* b_dst = sB + (stage * KSUB + q) * C::B_BYTES;
+            if (!A_MN) {
+              tma_load_2d(a_dst, tmA, &full[stage], k0, mb * BM);
+            } else {
 #pragma unroll
-            for (int j = 0; j < BN / 64; ++j) tma_load_2d(b_dst + j * 64 * BK * 2, tmB, &full[stage], nb * BN + 64 * j, k0);
+              for (int j = 0; j < BM / 64; ++j) tma_load_2d(a_dst + j * 64 * BK * 2, tmA, &full[stage], mb * BM + 64 * j, k0);
+            }
+            if (!B_MN) {
+              tma_load_2d(b_dst, tmB, &full[stage], k0, nb * BN);
+            } else {
+#pragma unroll
+              for (int j = 0; j < BN / 64; ++j) tma_load_2d(b_dst + j * 64 * BK * 2, tmB, &full[stage], nb * BN + 64 * j, k0);
+            }
           }
         }
         __syncwarp();
@@ -735,7 +743,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
       }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + acc * BN;
-      for (int kb = 0; kb < num_k; ++kb) {
+      for (int kb = 0; kb < num_k; kb += KSUB) {
         if (!mbar_wait_warp(&full[stage], phase)) {
           if (lane == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
           ok = false;
@@ -743,13 +751,18 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
         }
         tc_fence_after();
         if (elect_one()) {
-          const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + stage * C::A_BYTES));
-          const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + stage * C::B_BYTES));
 #pragma unroll
-          for (int kk = 0; kk < BK / UMMA_K; ++kk)
-            umma_bf16(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC, (kb | kk) != 0 ? 1u : 0u);
+          for (int q = 0; q < KSUB; ++q) {
+            if (KSUB > 1 && kb + q >= num_k) break;
+            const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + (stage * KSUB + q) * C::A_BYTES));
+            const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + (stage * KSUB + q) * C::B_BYTES));
+#pragma unroll
+            for (int kk = 0; kk < BK / UMMA_K; ++kk)
+              umma_bf16(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC,
+                        (kb | q | kk) != 0 ? 1u : 0u);
+          }
           umma_commit(&empty[stage]);
-          if (kb == num_k - 1) umma_commit(&acc_full[acc]);
+          if (kb + KSUB >= num_k) umma_commit(&acc_full[acc]);
         }
         __syncwarp();
         if (++stage == STAGES) {
@@ -804,34 +817,35 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
 constexpr int PAIR_BM = 256;
 template <int PBN, int FAM>
 struct CfgPair {
+  static constexpr int KSUB = 1;
   static constexpr int A_BYTES = 128 * BK * 2;        // this CTA's 128 rows of A
   static constexpr int B_BYTES = (PBN / 2) * BK * 2;  // this CTA's columns of B
-  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = ring_stages(STAGE_BYTES, EpiCfg<FAM>::BYTES);
+  static constexpr int STAGE_BYTES = KSUB * (A_BYTES + B_BYTES);
+  static constexpr int STAGES = ring_stages(STAGE_BYTES, EpiCfg<FAM, PBN>::BYTES);
   static constexpr int TMEM_COLS = 2 * PBN;  // double-buffered accumulator
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EpiCfg<FAM>::BYTES + BAR_BYTES + 1024 /*align*/;
-  static_assert((2 * STAGES + 5 + EpiCfg<FAM>::BARS) * 8 + 4 <= BAR_BYTES, "barriers");
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EpiCfg<FAM, PBN>::BYTES + BAR_BYTES + 1024 /*align*/;
+  static_assert((2 * STAGES + 5 + EpiCfg<FAM, PBN>::BARS) * 8 + 4 <= BAR_BYTES, "barriers");
 };
 
 template <int PBN, bool A_MN, bool B_MN, int FAM>
-__global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
+__global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ GemmMaps<FAM> maps, Epi epi, int M, int N, int K, int batch, Raster raster,
                      int* status) {
   using C = CfgPair<PBN, FAM>;
-  constexpr int STAGES = C::STAGES;
+  constexpr int STAGES = C::STAGES, KSUB = C::KSUB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + STAGES * C::A_BYTES;
+  uint8_t* sB = smem + STAGES * KSUB * C::A_BYTES;
   uint8_t* epi_smem = smem + STAGES * C::STAGE_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(epi_smem + EpiCfg<FAM>::BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(epi_smem + EpiCfg<FAM, PBN>::BYTES);
   uint64_t* full = bars;
   uint64_t* empty = bars + STAGES;
   uint64_t* acc_full = bars + 2 * STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
   uint64_t* ring_full = drain + 1;  // the AdamW ring's
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ring_full + EpiCfg<FAM>::BARS);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ring_full + EpiCfg<FAM, PBN>::BARS);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -850,10 +864,10 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 2 * EpiCfg<FAM>::WARPS);  // the epilogue warps of both CTAs
+      mbar_init(&acc_empty[a], 2 * EpiCfg<FAM, PBN>::WARPS);  // the epilogue warps of both CTAs
     }
     mbar_init(drain, 1);
-    for (int i = 0; i < EpiCfg<FAM>::BARS; ++i) mbar_init(&ring_full[i], 1);
+    for (int i = 0; i < EpiCfg<FAM, PBN>::BARS; ++i) mbar_init(&ring_full[i], 1);
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -885,7 +899,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
       const CUtensorMap* tmA = &maps.a[r];
       const CUtensorMap* tmB = &maps.b[r];
       const int m0 = mb * PAIR_BM + int(rank) * 128, n0 = nb * PBN + int(rank) * (PBN / 2);
-      for (int kb = 0; kb < num_k; ++kb) {
+      for (int kb = 0; kb < num_k; kb += KSUB) {
         if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
           if (lane == 0) report_status(status, FL_DEV_TIMEOUT_EMPTY);
           ok = false;
@@ -894,20 +908,23 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
         if (elect_one()) {
           if (leader) mbar_arrive_expect_tx(&full[stage], 2 * C::STAGE_BYTES);
           const uint32_t fb = full0 + 8u * stage;
-          const int k0 = kb * BK;
-          uint8_t* a_dst = sA + stage * C::A_BYTES;
-          uint8_t* b_dst = sB + stage * C::B_BYTES;
-          if (!A_MN) {
-            tma_load_2d_pair(a_dst, tmA, fb, k0, m0);
-          } else {
-            tma_load_2d_pair(a_dst, tmA, fb, m0, k0);
-            tma_load_2d_pair(a_dst + 64 * BK * 2, tmA, fb, m0 + 64, k0);
-          }
-          if (!B_MN) {
-            tma_load_2d_pair(b_dst, tmB, fb, k0, n0);
-          } else {
 #pragma unroll
-            for (int j = 0; j < PBN / 128; ++j) tma_load_2d_pair(b_dst + j * 64 * BK * 2, tmB, fb, n0 + 64 * j, k0);
+          for (int q = 0; q < KSUB; ++q) {  // a k-block past K reads zeros
+            const int k0 = (kb + q) * BK;
+            uint8_t* a_dst = sA + (stage * KSUB + q) * C::A_BYTES;
+            uint8_t* b_dst = sB + (stage * KSUB + q) * C::B_BYTES;
+            if (!A_MN) {
+              tma_load_2d_pair(a_dst, tmA, fb, k0, m0);
+            } else {
+              tma_load_2d_pair(a_dst, tmA, fb, m0, k0);
+              tma_load_2d_pair(a_dst + 64 * BK * 2, tmA, fb, m0 + 64, k0);
+            }
+            if (!B_MN) {
+              tma_load_2d_pair(b_dst, tmB, fb, k0, n0);
+            } else {
+#pragma unroll
+              for (int j = 0; j < PBN / 128; ++j) tma_load_2d_pair(b_dst + j * 64 * BK * 2, tmB, fb, n0 + 64 * j, k0);
+            }
           }
         }
         __syncwarp();
@@ -941,7 +958,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * PBN;
-        for (int kb = 0; kb < num_k; ++kb) {
+        for (int kb = 0; kb < num_k; kb += KSUB) {
           if (!mbar_wait_warp(&full[stage], phase)) {
             if (lane == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
             ok = false;
@@ -949,14 +966,18 @@ __global__ void __launch_bounds__(EpiCfg<FAM>::THREADS, 1)
           }
           tc_fence_after();
           if (elect_one()) {
-            const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + stage * C::A_BYTES));
-            const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + stage * C::B_BYTES));
 #pragma unroll
-            for (int kk = 0; kk < BK / UMMA_K; ++kk)
-              umma_bf16_pair(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC,
-                             (kb | kk) != 0 ? 1u : 0u);
+            for (int q = 0; q < KSUB; ++q) {
+              if (KSUB > 1 && kb + q >= num_k) break;
+              const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + (stage * KSUB + q) * C::A_BYTES));
+              const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + (stage * KSUB + q) * C::B_BYTES));
+#pragma unroll
+              for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                umma_bf16_pair(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC,
+                               (kb | q | kk) != 0 ? 1u : 0u);
+            }
             umma_commit_pair(&empty[stage], 3);
-            if (kb == num_k - 1) umma_commit_pair(&acc_full[acc], 3);
+            if (kb + KSUB >= num_k) umma_commit_pair(&acc_full[acc], 3);
           }
           __syncwarp();
           if (++stage == STAGES) {
@@ -1108,7 +1129,7 @@ int launch(const fl_gemm_args* a, const Problems& pr, const Epi& epi, int* statu
   const int tiles = batch * num_m * num_n;
   const int grid = tiles < num_sms() ? tiles : num_sms();
   const Raster r = pick_raster(a->M, a->N, a->K, BM, BN);
-  FL_CUDA_TRY(fl_launch(gemm_tc_kernel<BN, A_MN, B_MN, FAM>, dim3(grid), dim3(EpiCfg<FAM>::THREADS), C::SMEM_BYTES, st, maps,
+  FL_CUDA_TRY(fl_launch(gemm_tc_kernel<BN, A_MN, B_MN, FAM>, dim3(grid), dim3(EpiCfg<FAM, BN>::THREADS), C::SMEM_BYTES, st, maps,
                         epi, a->M, a->N, a->K, batch, r, status));
   return FL_OK;
 }
@@ -1139,7 +1160,7 @@ int pair_slots() {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(2 * num_sms());
-    cfg.blockDim = dim3(EpiCfg<FAM>::THREADS);
+    cfg.blockDim = dim3(EpiCfg<FAM, PBN>::THREADS);
     cfg.dynamicSmemBytes = CfgPair<PBN, FAM>::SMEM_BYTES;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -1182,7 +1203,7 @@ int launch_pair(const fl_gemm_args* a, const Problems& pr, const Epi& epi, int* 
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see pdl_wait
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(EpiCfg<FAM>::THREADS);
+  cfg.blockDim = dim3(EpiCfg<FAM, PBN>::THREADS);
   cfg.dynamicSmemBytes = CfgPair<PBN, FAM>::SMEM_BYTES;
   cfg.stream = st;
   cfg.attrs = attr;
@@ -1207,12 +1228,21 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
   X(EXT, W, AMN, BMN, FAM_RESID)          \
   X(EXT, W, AMN, BMN, FAM_ROPE)           \
   X(EXT, W, AMN, BMN, FAM_ADAMW)
+// The narrow tiles (256 x 128 on a pair, 128 x 64) are for outputs of few tiles, which weight
+// updates are not.
+#define FL_GEMM_NARROW_FAMS(X, EXT, W, AMN, BMN) \
+  X(EXT, W, AMN, BMN, FAM_PLAIN)                 \
+  X(EXT, W, AMN, BMN, FAM_GELU)                  \
+  X(EXT, W, AMN, BMN, FAM_RESID)                 \
+  X(EXT, W, AMN, BMN, FAM_ROPE)
 // FAM_ADAMW_LONG: the weight gradients' long contractions on CTA pairs only.
 #define FL_GEMM_INSTANTIATE_LONG(EXT) FL_GEMM_PAIR_FAM(EXT, 256, true, true, FAM_ADAMW_LONG)
 #define FL_GEMM_INSTANTIATE_PAIR(EXT, AMN, BMN)      \
-  FL_GEMM_FAMS(FL_GEMM_PAIR_FAM, EXT, 256, AMN, BMN)
+  FL_GEMM_FAMS(FL_GEMM_PAIR_FAM, EXT, 256, AMN, BMN) \
+  FL_GEMM_NARROW_FAMS(FL_GEMM_PAIR_FAM, EXT, 128, AMN, BMN)
 #define FL_GEMM_INSTANTIATE_SINGLE(EXT, AMN, BMN)      \
   FL_GEMM_FAMS(FL_GEMM_SINGLE_FAM, EXT, 256, AMN, BMN) \
-  FL_GEMM_FAMS(FL_GEMM_SINGLE_FAM, EXT, 128, AMN, BMN)
+  FL_GEMM_FAMS(FL_GEMM_SINGLE_FAM, EXT, 128, AMN, BMN) \
+  FL_GEMM_NARROW_FAMS(FL_GEMM_SINGLE_FAM, EXT, 64, AMN, BMN)
 
 }  // namespace fl_gemm

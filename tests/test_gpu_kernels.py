@@ -490,6 +490,54 @@ def test_gemm_adamw_epilogue(F, M, N, K, mn, tile):
     np.testing.assert_array_equal(bits(wbf), bits(wf.to(torch.bfloat16)))
 
 
+@pytest.mark.parametrize("layout", [(0, 0), (0, 1), (1, 1)], ids=["fwd", "dgrad", "wgrad"])
+@pytest.mark.parametrize("M,N,K", [(8, 128, 8), (72, 4096, 4040), (128, 4096, 4096), (136, 1280, 4168), (264, 4096, 136),
+                                   (304, 4096, 200), (512, 4096, 1024), (520, 2176, 72)])
+def test_gemm_picked_tile_bit_identical(F, M, N, K, layout):
+    """The tile the library picks (narrow ones here: few tiles, ragged rows, odd and ragged
+    counts of k-blocks) gives the bits of the 128 x 128 tile for every epilogue: each output
+    sums over K in the same order whatever the tile, which client-batching relies on."""
+    a_mn, b_mn = layout
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+
+    def rnd(*shape, dt=torch.bfloat16, s=1.0):
+        return (s * torch.randn(shape, generator=g, device="cuda")).to(dt)
+    A = rnd(*((K, M) if a_mn else (M, K)))
+    B = rnd(*((K, N) if b_mn else (N, K)), s=0.05)
+    lda, ldb = (M if a_mn else K), (N if b_mn else K)
+    bias, aux16, aux32 = rnd(N, dt=torch.float32), rnd(M, N), rnd(M, N, dt=torch.float32)
+    mu, rs, ga = rnd(M, dt=torch.float32), rnd(M, dt=torch.float32), rnd(N, dt=torch.float32)
+    pos = torch.arange(M, device="cuda", dtype=torch.int32)
+    tab = rnd(M, 32, 2, dt=torch.float32)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    f32 = dict(aux_dtype=F.FL_DT_F32, d_dtype=F.FL_DT_F32)
+    cases = [(torch.bfloat16, dict(epilogue=F.FL_EPI_STORE, bias=bias)), (torch.float32, dict(epilogue=F.FL_EPI_STORE_F32)),
+             (torch.float32, dict(epilogue=F.FL_EPI_ACCUM_F32)),
+             (torch.bfloat16, dict(epilogue=F.FL_EPI_BIAS_GELU, bias=bias, ld_aux_out=N, aux_out="u")),
+             (torch.bfloat16, dict(epilogue=F.FL_EPI_GELU_BWD, aux=aux16, ld_aux=N, colsum="c")),
+             (torch.float32, dict(epilogue=F.FL_EPI_BIAS_RESID, bias=bias, aux=aux32, ld_aux=N, alpha=7.5, ln_mean=mu,
+                                  ln_rstd=rs, ln_gamma=ga, ln_beta=bias, **f32))]
+    if N % 384 == 0 or N == 4096:
+        cases.append((torch.bfloat16, dict(epilogue=F.FL_EPI_BIAS_ROPE, bias=bias, pos=pos, rope_tab=tab, n_heads=N // 384,
+                                           head_dim=128, rotary_dim=64)))
+    for dt, kw in cases:
+        got = []
+        for tile in (F.FL_TILE_AUTO, F.FL_TILE_128x128):
+            D = torch.ones((M, N), dtype=dt, device="cuda")
+            u, c = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda"), torch.zeros(N, device="cuda")
+            k = {n: {"u": u, "c": c}[v] if isinstance(v, str) else v for n, v in kw.items()}
+            F.gemm(M, N, K, A, lda, a_mn, B, ldb, b_mn, D, N, status=status, tile=tile, **k)
+            got.append((D, u, c))
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        (D0, u0, c0), (D1, u1, c1) = got
+        assert torch.equal(D0.view(torch.int32 if dt == torch.float32 else torch.int16),
+                           D1.view(torch.int32 if dt == torch.float32 else torch.int16)), kw["epilogue"]
+        assert torch.equal(u0.view(torch.int16), u1.view(torch.int16))
+        # column sums: atomic sums of at most M fp32 values in any order
+        assert (c0 - c1).abs().max() <= 2.0 ** -22 * M * max(1.0, float(D1.float().abs().max())) if kw["epilogue"] == F.FL_EPI_GELU_BWD else True
+
+
 @pytest.mark.parametrize("K", [8, 2048, 3064, 3072, 3080])
 def test_gemm_adamw_epilogue_against_exact(F, K):
     """The fused update on both sides of the contraction length where its epilogue changes,
