@@ -76,8 +76,12 @@ struct BwdCfg {
   static constexpr int SMEM = USED > 120 * 1024 ? USED : 120 * 1024;
 };
 
-FL_DEV uint64_t desc_k(uint32_t base, int kk) { return smem_desc_sw128(base + (kk >> 2) * BOX + (kk & 3) * 32, 16, 1024); }
-FL_DEV uint64_t desc_mn(uint32_t base, int kk) { return smem_desc_sw128(base + kk * 2048, BOX, 1024); }
+// Descriptors of k-step 0 of a K-major (MN-major) tile, and the distance to k-step kk in the
+// descriptor's 16-byte units.
+FL_DEV uint64_t desc_k(uint32_t base) { return smem_desc_sw128(base, 16, 1024); }
+FL_DEV constexpr uint64_t step_k(int kk) { return (kk >> 2) * (BOX / 16) + (kk & 3) * 2; }
+FL_DEV uint64_t desc_mn(uint32_t base) { return smem_desc_sw128(base, BOX, 1024); }
+FL_DEV constexpr uint64_t step_mn(int kk) { return kk * 128; }
 
 // TMEM column (relative to the region's start) of the bf16 operand's k-step kk (16
 // columns of the 128-wide product): thread half g = kk / 4 wrote its columns 64 g .. + 63
@@ -273,10 +277,14 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
   BarTrack tkv, tq0, tq1, tm1, tm2;
-  auto issue_q = [&](const Unit& w, int it, int b) {  // one elected thread: Q_it, dO_it into pair b
+  // Copies and products are issued by warp 0 as a whole, one elected lane at work: the
+  // instructions' operands stay in uniform registers.
+  auto issue_q = [&](const Unit& w, int it, int b) {  // Q_it, dO_it into pair b
     int row0, qpos0, valid;
     qtile(w, it, row0, qpos0, valid);
     (b ? tq1 : tq0).pend = true;
+    __syncwarp();
+    if (!elect_one()) return;
     mbar_arrive_expect_tx(bar_q + b, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
@@ -284,8 +292,10 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       tma_load_2d(sdO + b * TILE + x * BOX, &tm_do, bar_q + b, w.h * HD + 64 * x, row0);
     }
   };
-  auto issue_kv = [&](const Unit& w) {  // one elected thread: the unit's K and V
+  auto issue_kv = [&](const Unit& w) {  // the unit's K and V
     tkv.pend = true;
+    __syncwarp();
+    if (!elect_one()) return;
     mbar_arrive_expect_tx(bar_kv, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
@@ -315,7 +325,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   };
   float pf = (u < n_units && w.it0 < w.it_end) ? stat_of(w, w.it0) : 0.f;
   RopeRow<HD> rrow;
-  if (tid == 0 && u < n_units && w.it0 < w.it_end) {
+  if (warp == 0 && u < n_units && w.it0 < w.it_end) {
     issue_kv(w);
     issue_q(w, w.it0, 0);
     if (w.it0 + 1 < w.it_end) issue_q(w, w.it0 + 1, 1);
@@ -352,16 +362,20 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       }
       // ---- S^T = K Q^T, dP^T = V dO^T (the previous dV / dK products, which read these
       // columns, have completed)
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
-        const uint32_t ak = smem_u32(sK), av = smem_u32(sV), bq = smem_u32(sQ + b * TILE),
-                       bo = smem_u32(sdO + b * TILE);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, desc_k(ak, kk), desc_k(bq, kk), IDESC_S, kk > 0);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, desc_k(av, kk), desc_k(bo, kk), IDESC_S, kk > 0);
         tm1.pend = true;
-        umma_commit(bar_mma1);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t ak = desc_k(smem_u32(sK)), av = desc_k(smem_u32(sV)), bq = desc_k(smem_u32(sQ + b * TILE)),
+                         bo = desc_k(smem_u32(sdO + b * TILE));
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, ak + step_k(kk), bq + step_k(kk), IDESC_S, kk > 0);
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, av + step_k(kk), bo + step_k(kk), IDESC_S, kk > 0);
+          umma_commit(bar_mma1);
+        }
+        __syncwarp();
       }
       // while the products run: the next tile's statistics, the unit after next
       if (it + 1 < w.it_end) pf = stat_of(w, it + 1);
@@ -373,7 +387,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         break;
       }
       tc_fence_after();
-      if (tid == 0 && next && it + 1 == w.it_end) issue_kv(wn);
+      if (warp == 0 && next && it + 1 == w.it_end) issue_kv(wn);
       // ---- P^T and dS^T of key row r for queries qh * 64 .. + 63, in two groups of 32,
       // each written (bf16 pairs) into the 16 columns at 64 qh + 16 hf it has just read
       {
@@ -427,18 +441,22 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       __syncthreads();
       // ---- dV += P^T dO, dK += dS^T Q (A from TMEM); then the tile after next into this
       // buffer pair once both products have read it
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
-        const uint32_t bq = smem_u32(sQ + b * TILE), bo = smem_u32(sdO + b * TILE);
-        const bool acc = it > w.it0;
-#pragma unroll
-        for (int kk = 0; kk < TB / 16; ++kk)
-          umma_bf16_ts(tmem + 256, tmem + a_col(kk), desc_mn(bo, kk), IDESC_G, (acc || kk > 0) ? 1u : 0u);
-#pragma unroll
-        for (int kk = 0; kk < TB / 16; ++kk)
-          umma_bf16_ts(tmem + 256 + HD, tmem + 128 + a_col(kk), desc_mn(bq, kk), IDESC_G, (acc || kk > 0) ? 1u : 0u);
         tm2.pend = true;
-        umma_commit(bar_mma2);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t bq = desc_mn(smem_u32(sQ + b * TILE)), bo = desc_mn(smem_u32(sdO + b * TILE));
+          const bool acc = it > w.it0;
+#pragma unroll
+          for (int kk = 0; kk < TB / 16; ++kk)
+            umma_bf16_ts(tmem + 256, tmem + a_col(kk), bo + step_mn(kk), IDESC_G, (acc || kk > 0) ? 1u : 0u);
+#pragma unroll
+          for (int kk = 0; kk < TB / 16; ++kk)
+            umma_bf16_ts(tmem + 256 + HD, tmem + 128 + a_col(kk), bq + step_mn(kk), IDESC_G, (acc || kk > 0) ? 1u : 0u);
+          umma_commit(bar_mma2);
+        }
+        __syncwarp();
       }
       if (it == w.it0 && un + (int)gridDim.x < n_units) wnn = unit_t(un + gridDim.x, tnn);
       if (!PREFIX && it + 1 == w.it_end && qh < nreg && key_ok) {  // the key's rotary row, for the epilogue
@@ -451,7 +469,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         break;
       }
       tc_fence_after();
-      if (tid == 0) {
+      if (warp == 0) {
         if (it + 2 < w.it_end) {
           issue_q(w, it + 2, b);
         } else if (next) {  // pair b's last use in this unit: the next unit's tile of pair b
@@ -464,7 +482,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
 
     // ---- every product of the unit is complete: its dK / dV leave while the next unit's
     // tiles load
-    if (tid == 0 && next && !work) {
+    if (warp == 0 && next && !work) {
       issue_kv(wn);
       issue_q(wn, wn.it0, 0);
       if (wn.it0 + 1 < wn.it_end) issue_q(wn, wn.it0 + 1, 1);
@@ -642,8 +660,11 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
   BarTrack tqdo, tkv0, tkv1, tm1, tm2;
-  auto issue_kv = [&](const Unit& w, int j, int b) {  // one elected thread: K_j, V_j into pair b
+  // Copies and products are issued by warp 0 as a whole, as in the dK / dV kernel.
+  auto issue_kv = [&](const Unit& w, int j, int b) {  // K_j, V_j into pair b
     (b ? tkv1 : tkv0).pend = true;
+    __syncwarp();
+    if (!elect_one()) return;
     mbar_arrive_expect_tx(bar_kv + b, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
@@ -657,8 +678,10 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
       }
     }
   };
-  auto issue_qdo = [&](const Unit& w) {  // one elected thread: the unit's Q and dO
+  auto issue_qdo = [&](const Unit& w) {  // the unit's Q and dO
     tqdo.pend = true;
+    __syncwarp();
+    if (!elect_one()) return;
     mbar_arrive_expect_tx(bar_qdo, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
@@ -675,7 +698,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   float lse2 = 0.f, dl = 0.f;
   if (u < n_units) row_stats(w, lse2, dl);
   RopeRow<HD> rrow;
-  if (tid == 0 && u < n_units) {
+  if (warp == 0 && u < n_units) {
     issue_qdo(w);
     issue_kv(w, 0, 0);
     if (w.n_kv > 1) issue_kv(w, 1, 1);
@@ -704,16 +727,20 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
       }
       // ---- S = Q K_j^T, dP = dO V_j^T (the previous dQ product, which read these
       // columns, has completed)
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
-        const uint32_t aq = smem_u32(sQ), ao = smem_u32(sdO), bk = smem_u32(sK + b * TILE),
-                       bv = smem_u32(sV + b * TILE);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, desc_k(aq, kk), desc_k(bk, kk), IDESC_S, kk > 0);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, desc_k(ao, kk), desc_k(bv, kk), IDESC_S, kk > 0);
         tm1.pend = true;
-        umma_commit(bar_mma1);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t aq = desc_k(smem_u32(sQ)), ao = desc_k(smem_u32(sdO)), bk = desc_k(smem_u32(sK + b * TILE)),
+                         bv = desc_k(smem_u32(sV + b * TILE));
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, aq + step_k(kk), bk + step_k(kk), IDESC_S, kk > 0);
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, ao + step_k(kk), bv + step_k(kk), IDESC_S, kk > 0);
+          umma_commit(bar_mma1);
+        }
+        __syncwarp();
       }
       if (!track_wait_all(bar_mma1, tm1)) {
         if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
@@ -721,7 +748,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
         break;
       }
       tc_fence_after();
-      if (tid == 0 && next && j + 1 == w.n_kv) issue_qdo(wn);
+      if (warp == 0 && next && j + 1 == w.n_kv) issue_qdo(wn);
       // ---- dS of query row r for keys kh * 64 .. + 63 of the tile, in two groups of 32,
       // each written (bf16 pairs) into the 16 S columns at 64 kh + 16 hf it has just read
       {
@@ -755,14 +782,18 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
       __syncthreads();
       // ---- dQ += dS K_j (A from TMEM); then the tile after next into this buffer pair
       // once both products have read it
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
-        const uint32_t bk = smem_u32(sK + b * TILE);
-#pragma unroll
-        for (int kk = 0; kk < TB / 16; ++kk)
-          umma_bf16_ts(tmem + 256, tmem + a_col(kk), desc_mn(bk, kk), IDESC_G, (j > 0 || kk > 0) ? 1u : 0u);
         tm2.pend = true;
-        umma_commit(bar_mma2);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t bk = desc_mn(smem_u32(sK + b * TILE));
+#pragma unroll
+          for (int kk = 0; kk < TB / 16; ++kk)
+            umma_bf16_ts(tmem + 256, tmem + a_col(kk), bk + step_mn(kk), IDESC_G, (j > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(bar_mma2);
+        }
+        __syncwarp();
       }
       if (j + 1 == w.n_kv && kh < nreg && q_ok) {  // the query's rotary row, for the epilogue
         const int32_t* gp = kh == 0 ? gpos : gpos2;
@@ -774,7 +805,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
         break;
       }
       tc_fence_after();
-      if (tid == 0) {
+      if (warp == 0) {
         if (j + 2 < w.n_kv) {
           issue_kv(w, j + 2, b);
         } else if (next) {  // pair b's last use in this unit: the next unit's tile of pair b

@@ -48,12 +48,13 @@ struct FwdCfg {
   static constexpr int SMEM = USED > 80 * 1024 ? USED : 80 * 1024;
 };
 
-// K-major operand (rows x HD columns in 64-column swizzled boxes): descriptor of k-step kk.
-FL_DEV uint64_t desc_kmajor(uint32_t base, int kk) {
-  return smem_desc_sw128(base + (kk >> 2) * BOX + (kk & 3) * 32, 16, 1024);
-}
-// MN-major operand (K = the tile's 128 rows, N = its HD columns): descriptor of k-step kk.
-FL_DEV uint64_t desc_mnmajor(uint32_t base, int kk) { return smem_desc_sw128(base + kk * 2048, BOX, 1024); }
+// K-major operand (rows x HD columns in 64-column swizzled boxes): descriptor of k-step 0 and
+// the distance to k-step kk (in the descriptor's 16-byte units).
+FL_DEV uint64_t desc_kmajor(uint32_t base) { return smem_desc_sw128(base, 16, 1024); }
+FL_DEV constexpr uint64_t step_kmajor(int kk) { return (kk >> 2) * (BOX / 16) + (kk & 3) * 2; }
+// MN-major operand (K = the tile's 128 rows, N = its HD columns).
+FL_DEV uint64_t desc_mnmajor(uint32_t base) { return smem_desc_sw128(base, BOX, 1024); }
+FL_DEV constexpr uint64_t step_mnmajor(int kk) { return kk * 128; }
 
 template <int HD>
 __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
@@ -114,11 +115,15 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   const uint32_t t_s = t_lane, t_o = t_lane + 128;
 
   BarTrack tq, tk, tv, ts, tpv;
-  // one elected thread: the key (part 0) or value (part 1) tile j of unit w into its buffer
+  // Copies and products are issued by warp 0 as a whole, one elected lane at work: the
+  // instructions' operands stay in uniform registers.
+  // the key (part 0) or value (part 1) tile j of unit w into its buffer
   auto issue = [&](const Unit& w, int j, int part) {
     uint8_t* dst = part ? sV : sK;
     uint64_t* bar = part ? bar_v : bar_k;
     (part ? tv : tk).pend = true;
+    __syncwarp();
+    if (!elect_one()) return;
     mbar_arrive_expect_tx(bar, TILE);
     if (j < npt) {
       const CUtensorMap* m = part ? &tm_pv : &tm_pk;
@@ -133,9 +138,12 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   };
   auto issue_unit = [&](const Unit& w) {  // Q and the first key / value tiles of a unit
     tq.pend = true;
-    mbar_arrive_expect_tx(bar_q, TILE);
+    __syncwarp();
+    if (elect_one()) {
+      mbar_arrive_expect_tx(bar_q, TILE);
 #pragma unroll
-    for (int b = 0; b < NB; ++b) tma_load_2d(sQ + b * BOX, &tm_qkv, bar_q, w.h * HD + 64 * b, w.seg0 + w.q0);
+      for (int b = 0; b < NB; ++b) tma_load_2d(sQ + b * BOX, &tm_qkv, bar_q, w.h * HD + 64 * b, w.seg0 + w.q0);
+    }
     issue(w, 0, 0);
     issue(w, 0, 1);
   };
@@ -146,7 +154,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   int u = blockIdx.x;
   Unit w = u < n_units ? unit(u) : Unit{};
   Unit wn = u + (int)gridDim.x < n_units ? unit(u + gridDim.x) : Unit{};
-  if (tid == 0 && u < n_units) issue_unit(w);
+  if (warp == 0 && u < n_units) issue_unit(w);
   while (u < n_units && ok) {
     const int q = w.q0 + tid;  // this thread's query row (inside the segment)
     const int un = u + gridDim.x, unn = un + gridDim.x;
@@ -167,14 +175,18 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
         break;
       }
       // ---- S = Q K_j^T (the previous P V, which read the S columns, has completed)
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
-        const uint32_t aq = smem_u32(sQ), bk = smem_u32(sK);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk)
-          umma_bf16(tmem, desc_kmajor(aq, kk), desc_kmajor(bk, kk), IDESC_S, kk > 0);
         ts.pend = true;
-        umma_commit(bar_s);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t aq = desc_kmajor(smem_u32(sQ)), bk = desc_kmajor(smem_u32(sK));
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk)
+            umma_bf16(tmem, aq + step_kmajor(kk), bk + step_kmajor(kk), IDESC_S, kk > 0);
+          umma_commit(bar_s);
+        }
+        __syncwarp();
       }
       if (j == 0 && unn < n_units) tnn = tiles[unn / n_heads];
       if (!track_wait_all(bar_s, ts)) {
@@ -183,7 +195,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
         break;
       }
       tc_fence_after();
-      if (tid == 0 && j + 1 < w.n_kv) issue(w, j + 1, 0);  // K_j has been read
+      if (warp == 0 && j + 1 < w.n_kv) issue(w, j + 1, 0);  // K_j has been read
       // ---- the thread's S row, read once (4 x 32 columns, one wait)
       const bool prefix = j < npt;
       const int kb = prefix ? 0 : (j - npt) * TB;  // first key of the tile inside its sequence
@@ -241,14 +253,18 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
         break;
       }
       // ---- O += P V_j
-      if (tid == 0) {
+      if (warp == 0) {
         tc_fence_after();
-        const uint32_t bv = smem_u32(sV);
-#pragma unroll
-        for (int kk = 0; kk < TB / 16; ++kk)
-          umma_bf16_ts(tmem + 128, tmem + kk * 8, desc_mnmajor(bv, kk), IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u);
         tpv.pend = true;
-        umma_commit(bar_pv);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t bv = desc_mnmajor(smem_u32(sV));
+#pragma unroll
+          for (int kk = 0; kk < TB / 16; ++kk)
+            umma_bf16_ts(tmem + 128, tmem + kk * 8, bv + step_mnmajor(kk), IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(bar_pv);
+        }
+        __syncwarp();
       }
       if (j == 0 && unn < n_units) wnn = unit_t(unn, tnn);
       if (!track_wait_all(bar_pv, tpv)) {
@@ -257,12 +273,12 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
         break;
       }
       tc_fence_after();
-      if (tid == 0 && j + 1 < w.n_kv) issue(w, j + 1, 1);  // V_j has been read
+      if (warp == 0 && j + 1 < w.n_kv) issue(w, j + 1, 1);  // V_j has been read
     }
     if (!ok) break;
     // ---- every product of the unit is complete and Q / K / V are free: the next unit's
     // first tiles load while this one's O leaves
-    if (tid == 0 && un < n_units) issue_unit(wn);
+    if (warp == 0 && un < n_units) issue_unit(wn);
     // ---- O / l and the log-sum-exp (every lane reads TMEM, all of the row at once; rows
     // past the segment end store nothing)
     const bool valid = q < w.L;
