@@ -49,6 +49,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "../../include/flglm_kernels.h"
 #include "common.cuh"
@@ -201,8 +202,9 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   uint64_t* bars = reinterpret_cast<uint64_t*>(sD + TB);
   uint64_t* bar_kv = bars;
   uint64_t* bar_q = bars + 1;  // [2]
-  uint64_t* bar_mma1 = bars + 3;
-  uint64_t* bar_mma2 = bars + 4;
+  uint64_t* bar_s = bars + 3;
+  uint64_t* bar_dp = bars + 4;
+  uint64_t* bar_mma2 = bars + 5;
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
 
   const int nh = H / HD;
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   };
 
   if (tid == 0) {
-    for (int i = 0; i < 5; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < 6; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
     tma_prefetch_desc(&tm_do);
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
-  BarTrack tkv, tq0, tq1, tm1, tm2;
+  BarTrack tkv, tq0, tq1, ts, tdp, tm2;
   // Copies and products are issued by warp 0 as a whole, one elected lane at work: the
   // instructions' operands stay in uniform registers.
   auto issue_q = [&](const Unit& w, int it, int b) {  // Q_it, dO_it into pair b
@@ -346,8 +348,34 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       ok = false;
       break;
     }
+    auto scores = [&](int b) {  // warp 0: S^T = K Q^T and dP^T = V dO^T of the tile in pair b
+      ts.pend = tdp.pend = true;
+      if (elect_one()) {
+        const uint64_t ak = desc_k(smem_u32(sK)), av = desc_k(smem_u32(sV)), bq = desc_k(smem_u32(sQ + b * TILE)),
+                       bo = desc_k(smem_u32(sdO + b * TILE));
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, ak + step_k(kk), bq + step_k(kk), IDESC_S, kk > 0);
+        umma_commit(bar_s);
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, av + step_k(kk), bo + step_k(kk), IDESC_S, kk > 0);
+        umma_commit(bar_dp);
+      }
+      __syncwarp();
+    };
+    if (work) {
+      if (!track_wait_all(bar_q, tq0)) {
+        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+        ok = false;
+        break;
+      }
+      if (warp == 0) {
+        tc_fence_after();
+        scores(0);
+      }
+    }
     for (int it = w.it0; it < w.it_end && ok; ++it) {
       const int b = (it - w.it0) & 1;
+      const bool last = it + 1 == w.it_end;
       int row0, qpos0, valid;
       qtile(w, it, row0, qpos0, valid);
       {  // lse and delta of the query tile (rows past its segment are never visible)
@@ -355,127 +383,146 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         if (tid < TB) sL[c] = pf * LOG2E_B;  // the previous tile's readers passed a barrier since
         else sD[c] = pf;
       }
-      if (!track_wait_all(bar_q + b, b ? tq1 : tq0)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
-      // ---- S^T = K Q^T, dP^T = V dO^T (the previous dV / dK products, which read these
-      // columns, have completed)
-      if (warp == 0) {
-        tc_fence_after();
-        tm1.pend = true;
-        __syncwarp();
-        if (elect_one()) {
-          const uint64_t ak = desc_k(smem_u32(sK)), av = desc_k(smem_u32(sV)), bq = desc_k(smem_u32(sQ + b * TILE)),
-                         bo = desc_k(smem_u32(sdO + b * TILE));
-#pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, ak + step_k(kk), bq + step_k(kk), IDESC_S, kk > 0);
-#pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, av + step_k(kk), bo + step_k(kk), IDESC_S, kk > 0);
-          umma_commit(bar_mma1);
-        }
-        __syncwarp();
-      }
       // while the products run: the next tile's statistics, the unit after next
-      if (it + 1 < w.it_end) pf = stat_of(w, it + 1);
+      if (!last) pf = stat_of(w, it + 1);
       else if (next) pf = stat_of(wn, wn.it0);
       if (it == w.it0 && un + (int)gridDim.x < n_units) tnn = tile_word(un + gridDim.x);
-      if (!track_wait_all(bar_mma1, tm1)) {
+      if (!track_wait_all(bar_s, ts)) {
         if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
         ok = false;
         break;
       }
       tc_fence_after();
-      if (warp == 0 && next && it + 1 == w.it_end) issue_kv(wn);
-      // ---- P^T and dS^T of key row r for queries qh * 64 .. + 63, in two groups of 32,
-      // each written (bf16 pairs) into the 16 columns at 64 qh + 16 hf it has just read
-      {
-        const int q0 = qpos0 + qh * 64;
-        // key k is visible to queries [qfirst, qlim) of the tile's segment
-        int qlim, qfirst;
-        if constexpr (PREFIX) {
-          qlim = key_ok ? qpos0 + valid : q0;
-          qfirst = q0;
-        } else {
-          qlim = key_ok ? min(w.L, q0 + 64) : q0;
-          qfirst = k <= w.clast ? q0 : max(q0, k);
+      // S^T is complete and so is every product issued before it: the other buffer pair is free
+      // for the next tile (the second tile of a unit was loaded at the end of the unit before)
+      if (warp == 0) {
+        if (!last) {
+          if (it > w.it0) issue_q(w, it + 1, 1 - b);
+        } else if (next && wn.it0 + (1 - b) < wn.it_end) {
+          issue_q(wn, wn.it0 + (1 - b), 1 - b);
         }
-        const float* Lb = sL;
-        const float* Db = sD;
-#pragma unroll 1
+      }
+      const int q0 = qpos0 + qh * 64;
+      // key k is visible to queries [qfirst, qlim) of the tile's segment
+      int qlim, qfirst;
+      if constexpr (PREFIX) {
+        qlim = key_ok ? qpos0 + valid : q0;
+        qfirst = q0;
+      } else {
+        qlim = key_ok ? min(w.L, q0 + 64) : q0;
+        qfirst = k <= w.clast ? q0 : max(q0, k);
+      }
+      // every key of the warp visible to all 64 queries: no masks
+      const bool open = __all_sync(0xffffffffu, qfirst <= q0 && qlim >= q0 + 64);
+      // ---- P^T of key row r for queries qh * 64 .. + 63, in two groups of 32, kept in registers
+      // and written (bf16 pairs) into the 16 columns at 64 qh + 16 hf of the S^T just read
+      float p[64];
+      auto probs = [&](auto masked) {
+#pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
-          uint32_t sr[32], dr[32];
+          uint32_t sr[32];
           tmem_ld32(t_lane + qh * 64 + 32 * hf, sr);
-          tmem_ld32(t_lane + 128 + qh * 64 + 32 * hf, dr);
           tmem_ld_wait();
-          const float4* L4 = reinterpret_cast<const float4*>(Lb + qh * 64 + 32 * hf);
-          const float4* D4 = reinterpret_cast<const float4*>(Db + qh * 64 + 32 * hf);
-          uint32_t pp[16], dd[16];
+          const float4* L4 = reinterpret_cast<const float4*>(sL + qh * 64 + 32 * hf);
+          uint32_t pp[16];
 #pragma unroll
-          for (int c8 = 0; c8 < 4; ++c8) {
-            const float4 la = L4[2 * c8], lb = L4[2 * c8 + 1], da = D4[2 * c8], db = D4[2 * c8 + 1];
-            const float lq[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
-            const float dq[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
-            float p[8], ds[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int c = 8 * c8 + e, q = q0 + 32 * hf + c;
-              const bool vis = q >= qfirst && q < qlim;
-              const float pv = vis ? exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lq[e])) : 0.f;
-              p[e] = pv;
-              ds[e] = pv * (__uint_as_float(dr[c]) - dq[e]);
-            }
+          for (int c4 = 0; c4 < 8; ++c4) {
+            const float4 l4 = L4[c4];
+            const float lq[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              pp[4 * c8 + e] = pack_bf16x2(p[2 * e], p[2 * e + 1]);
-              dd[4 * c8 + e] = pack_bf16x2(ds[2 * e], ds[2 * e + 1]);
+              const int c = 4 * c4 + e, q = q0 + 32 * hf + c;
+              const float pv = exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lq[e]));
+              p[32 * hf + c] = !masked.value || (q >= qfirst && q < qlim) ? pv : 0.f;
             }
+            pp[2 * c4] = pack_bf16x2(p[32 * hf + 4 * c4], p[32 * hf + 4 * c4 + 1]);
+            pp[2 * c4 + 1] = pack_bf16x2(p[32 * hf + 4 * c4 + 2], p[32 * hf + 4 * c4 + 3]);
           }
           tmem_st16(t_lane + qh * 64 + 16 * hf, pp);
-          tmem_st16(t_lane + 128 + qh * 64 + 16 * hf, dd);
         }
-      }
+      };
+      if (open) probs(std::false_type{});
+      else probs(std::true_type{});
+      if (it == w.it0 && un + (int)gridDim.x < n_units) wnn = unit_t(un + gridDim.x, tnn);
       tmem_st_wait();
       tc_fence_before();
-      __syncthreads();
-      // ---- dV += P^T dO, dK += dS^T Q (A from TMEM); then the tile after next into this
-      // buffer pair once both products have read it
-      if (warp == 0) {
-        tc_fence_after();
-        tm2.pend = true;
-        __syncwarp();
-        if (elect_one()) {
-          const uint64_t bq = desc_mn(smem_u32(sQ + b * TILE)), bo = desc_mn(smem_u32(sdO + b * TILE));
-          const bool acc = it > w.it0;
-#pragma unroll
-          for (int kk = 0; kk < TB / 16; ++kk)
-            umma_bf16_ts(tmem + 256, tmem + a_col(kk), bo + step_mn(kk), IDESC_G, (acc || kk > 0) ? 1u : 0u);
-#pragma unroll
-          for (int kk = 0; kk < TB / 16; ++kk)
-            umma_bf16_ts(tmem + 256 + HD, tmem + 128 + a_col(kk), bq + step_mn(kk), IDESC_G, (acc || kk > 0) ? 1u : 0u);
-          umma_commit(bar_mma2);
-        }
-        __syncwarp();
-      }
-      if (it == w.it0 && un + (int)gridDim.x < n_units) wnn = unit_t(un + gridDim.x, tnn);
-      if (!PREFIX && it + 1 == w.it_end && qh < nreg && key_ok) {  // the key's rotary row, for the epilogue
-        const int32_t* gp = qh == 0 ? gpos : gpos2;
-        rope_load<HD>(rrow, rope_tab + (int64_t)(gp ? __ldg(gp + w.seg0 + k) : k) * E);
-      }
-      if (!track_wait_all(bar_mma2, tm2)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
+      if (!track_wait_all(bar_dp, tdp)) {
+        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
         ok = false;
         break;
       }
       tc_fence_after();
+      // ---- dV += P^T dO (A from TMEM) while dS^T is made; the unit's last reader of K and V is done
       if (warp == 0) {
-        if (it + 2 < w.it_end) {
-          issue_q(w, it + 2, b);
-        } else if (next) {  // pair b's last use in this unit: the next unit's tile of pair b
-          if (wn.it0 + b < wn.it_end) issue_q(wn, wn.it0 + b, b);
-          if (w.it0 + 1 == w.it_end && wn.it0 + 1 < wn.it_end) issue_q(wn, wn.it0 + 1, 1);  // pair 1 unused here
+        if (last && next) issue_kv(wn);
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t bo = desc_mn(smem_u32(sdO + b * TILE));
+#pragma unroll
+          for (int kk = 0; kk < TB / 16; ++kk)
+            umma_bf16_ts(tmem + 256, tmem + a_col(kk), bo + step_mn(kk), IDESC_G, (it > w.it0 || kk > 0) ? 1u : 0u);
         }
+        __syncwarp();
+      }
+      // ---- dS^T, written the same way over dP^T
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        uint32_t dr[32];
+        tmem_ld32(t_lane + 128 + qh * 64 + 32 * hf, dr);
+        tmem_ld_wait();
+        const float4* D4 = reinterpret_cast<const float4*>(sD + qh * 64 + 32 * hf);
+        uint32_t dd[16];
+#pragma unroll
+        for (int c4 = 0; c4 < 8; ++c4) {
+          const float4 d4 = D4[c4];
+          const float dq[4] = {d4.x, d4.y, d4.z, d4.w};
+          float ds[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ds[e] = p[32 * hf + 4 * c4 + e] * (__uint_as_float(dr[4 * c4 + e]) - dq[e]);
+          dd[2 * c4] = pack_bf16x2(ds[0], ds[1]);
+          dd[2 * c4 + 1] = pack_bf16x2(ds[2], ds[3]);
+        }
+        tmem_st16(t_lane + 128 + qh * 64 + 16 * hf, dd);
+      }
+      tmem_st_wait();
+      tc_fence_before();
+      // the next tile's Q and dO have landed (and every thread has written its dS^T)
+      if (last) {
+        __syncthreads();
+      } else if (!track_wait_all(bar_q + 1 - b, b ? tq0 : tq1)) {
+        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+        ok = false;
+        break;
+      }
+      // ---- dK += dS^T Q, and the next tile's scores behind it (they overwrite P^T and dS^T, which
+      // the products before them in the tensor pipe have read)
+      if (warp == 0) {
+        tc_fence_after();
+        if (last) tm2.pend = true;
+        __syncwarp();
+        if (elect_one()) {
+          const uint64_t bq = desc_mn(smem_u32(sQ + b * TILE));
+#pragma unroll
+          for (int kk = 0; kk < TB / 16; ++kk)
+            umma_bf16_ts(tmem + 256 + HD, tmem + 128 + a_col(kk), bq + step_mn(kk), IDESC_G, (it > w.it0 || kk > 0) ? 1u : 0u);
+          if (last) umma_commit(bar_mma2);
+        }
+        __syncwarp();
+        if (!last) scores(1 - b);
+      }
+      if (last) {
+        if (!PREFIX && qh < nreg && key_ok) {  // the key's rotary row, for the epilogue
+          const int32_t* gp = qh == 0 ? gpos : gpos2;
+          rope_load<HD>(rrow, rope_tab + (int64_t)(gp ? __ldg(gp + w.seg0 + k) : k) * E);
+        }
+        if (!track_wait_all(bar_mma2, tm2)) {
+          if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        // this pair's last use in the unit: the next unit's tile of the pair
+        if (warp == 0 && next && wn.it0 + b < wn.it_end) issue_q(wn, wn.it0 + b, b);
       }
     }
     if (!ok) break;
@@ -572,7 +619,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     track_drain(bar_kv, tkv);
     track_drain(bar_q, tq0);
     track_drain(bar_q + 1, tq1);
-    track_drain(bar_mma1, tm1);
+    track_drain(bar_s, ts);
+    track_drain(bar_dp, tdp);
     track_drain(bar_mma2, tm2);
   }
   tc_fence_before();
@@ -606,8 +654,9 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 7 * TILE + 2 * TB * 4);
   uint64_t* bar_qdo = bars;
   uint64_t* bar_kv = bars + 1;  // [2]
-  uint64_t* bar_mma1 = bars + 3;
-  uint64_t* bar_mma2 = bars + 4;
+  uint64_t* bar_s = bars + 3;
+  uint64_t* bar_dp = bars + 4;
+  uint64_t* bar_mma2 = bars + 5;
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
 
   const int nh = H / HD;
@@ -644,7 +693,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   };
 
   if (tid == 0) {
-    for (int i = 0; i < 5; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < 6; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
     tma_prefetch_desc(&tm_do);
@@ -659,7 +708,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
-  BarTrack tqdo, tkv0, tkv1, tm1, tm2;
+  BarTrack tqdo, tkv0, tkv1, ts, tdp, tm2;
   // Copies and products are issued by warp 0 as a whole, as in the dK / dV kernel.
   auto issue_kv = [&](const Unit& w, int j, int b) {  // K_j, V_j into pair b
     (b ? tkv1 : tkv0).pend = true;
@@ -718,100 +767,128 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
       ok = false;
       break;
     }
+    auto scores = [&](int b) {  // warp 0: S = Q K^T and dP = dO V^T of the tile in pair b
+      ts.pend = tdp.pend = true;
+      if (elect_one()) {
+        const uint64_t aq = desc_k(smem_u32(sQ)), ao = desc_k(smem_u32(sdO)), bk = desc_k(smem_u32(sK + b * TILE)),
+                       bv = desc_k(smem_u32(sV + b * TILE));
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, aq + step_k(kk), bk + step_k(kk), IDESC_S, kk > 0);
+        umma_commit(bar_s);
+#pragma unroll
+        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, ao + step_k(kk), bv + step_k(kk), IDESC_S, kk > 0);
+        umma_commit(bar_dp);
+      }
+      __syncwarp();
+    };
+    if (!track_wait_all(bar_kv, tkv0)) {
+      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+      ok = false;
+      break;
+    }
+    if (warp == 0) {
+      tc_fence_after();
+      scores(0);
+    }
     for (int j = 0; j < w.n_kv && ok; ++j) {
       const int b = j & 1;
-      if (!track_wait_all(bar_kv + b, b ? tkv1 : tkv0)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
-      // ---- S = Q K_j^T, dP = dO V_j^T (the previous dQ product, which read these
-      // columns, has completed)
-      if (warp == 0) {
-        tc_fence_after();
-        tm1.pend = true;
-        __syncwarp();
-        if (elect_one()) {
-          const uint64_t aq = desc_k(smem_u32(sQ)), ao = desc_k(smem_u32(sdO)), bk = desc_k(smem_u32(sK + b * TILE)),
-                         bv = desc_k(smem_u32(sV + b * TILE));
-#pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, aq + step_k(kk), bk + step_k(kk), IDESC_S, kk > 0);
-#pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, ao + step_k(kk), bv + step_k(kk), IDESC_S, kk > 0);
-          umma_commit(bar_mma1);
-        }
-        __syncwarp();
-      }
-      if (!track_wait_all(bar_mma1, tm1)) {
+      const bool last = j + 1 == w.n_kv;
+      if (!track_wait_all(bar_s, ts)) {
         if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
         ok = false;
         break;
       }
       tc_fence_after();
-      if (warp == 0 && next && j + 1 == w.n_kv) issue_qdo(wn);
-      // ---- dS of query row r for keys kh * 64 .. + 63 of the tile, in two groups of 32,
-      // each written (bf16 pairs) into the 16 S columns at 64 kh + 16 hf it has just read
-      {
-        const bool prefix = j < npt;
-        const int u0 = (prefix ? 0 : (j - npt) * TB) + kh * 64;  // first key of the half
-        const int uend = prefix ? (q_ok ? Lp : 0) : ulim + 1;    // keys [u0, uend) are visible
-#pragma unroll 1
-        for (int hf = 0; hf < 2; ++hf) {
-          uint32_t sr[32], dr[32];
-          tmem_ld32(t_lane + kh * 64 + 32 * hf, sr);
-          tmem_ld32(t_lane + 128 + kh * 64 + 32 * hf, dr);
-          tmem_ld_wait();
-          uint32_t dd[16];
-#pragma unroll
-          for (int c2 = 0; c2 < 16; ++c2) {
-            float ds[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const int c = 2 * c2 + e;
-              const bool vis = u0 + 32 * hf + c < uend;
-              const float pv = vis ? exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lse2)) : 0.f;
-              ds[e] = pv * (__uint_as_float(dr[c]) - dl);
-            }
-            dd[c2] = pack_bf16x2(ds[0], ds[1]);
-          }
-          tmem_st16(t_lane + kh * 64 + 16 * hf, dd);
+      // S is complete and so is every product issued before it: the other buffer pair is free for
+      // the next tile (the second tile of a unit was loaded at the end of the unit before)
+      if (warp == 0) {
+        if (!last) {
+          if (j > 0) issue_kv(w, j + 1, 1 - b);
+        } else if (next && 1 - b < wn.n_kv) {
+          issue_kv(wn, 1 - b, 1 - b);
         }
+      }
+      const bool prefix = j < npt;
+      const int u0 = (prefix ? 0 : (j - npt) * TB) + kh * 64;  // first key of the half
+      const int uend = prefix ? (q_ok ? Lp : 0) : ulim + 1;    // keys [u0, uend) are visible
+      const bool open = __all_sync(0xffffffffu, uend >= u0 + 64);
+      // ---- P of query row r for keys kh * 64 .. + 63 of the tile, kept in registers
+      float p[64];
+      auto probs = [&](auto masked) {
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t sr[32];
+          tmem_ld32(t_lane + kh * 64 + 32 * hf, sr);
+          tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 32; ++c) {
+            const float pv = exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lse2));
+            p[32 * hf + c] = !masked.value || u0 + 32 * hf + c < uend ? pv : 0.f;
+          }
+        }
+      };
+      if (open) probs(std::false_type{});
+      else probs(std::true_type{});
+      tc_fence_before();
+      if (!track_wait_all(bar_dp, tdp)) {
+        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      if (warp == 0 && next && last) issue_qdo(wn);
+      // ---- dS, written (bf16 pairs) into the 16 S columns at 64 kh + 16 hf
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        uint32_t dr[32];
+        tmem_ld32(t_lane + 128 + kh * 64 + 32 * hf, dr);
+        tmem_ld_wait();
+        uint32_t dd[16];
+#pragma unroll
+        for (int c2 = 0; c2 < 16; ++c2)
+          dd[c2] = pack_bf16x2(p[32 * hf + 2 * c2] * (__uint_as_float(dr[2 * c2]) - dl),
+                               p[32 * hf + 2 * c2 + 1] * (__uint_as_float(dr[2 * c2 + 1]) - dl));
+        tmem_st16(t_lane + kh * 64 + 16 * hf, dd);
       }
       tmem_st_wait();
       tc_fence_before();
-      __syncthreads();
-      // ---- dQ += dS K_j (A from TMEM); then the tile after next into this buffer pair
-      // once both products have read it
+      // the next tile's K and V have landed (and every thread has written its dS)
+      if (last) {
+        __syncthreads();
+      } else if (!track_wait_all(bar_kv + 1 - b, b ? tkv0 : tkv1)) {
+        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+        ok = false;
+        break;
+      }
+      // ---- dQ += dS K_j (A from TMEM), and the next tile's scores behind it (they overwrite dS,
+      // which the product before them in the tensor pipe has read)
       if (warp == 0) {
         tc_fence_after();
-        tm2.pend = true;
+        if (last) tm2.pend = true;
         __syncwarp();
         if (elect_one()) {
           const uint64_t bk = desc_mn(smem_u32(sK + b * TILE));
 #pragma unroll
           for (int kk = 0; kk < TB / 16; ++kk)
             umma_bf16_ts(tmem + 256, tmem + a_col(kk), bk + step_mn(kk), IDESC_G, (j > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(bar_mma2);
+          if (last) umma_commit(bar_mma2);
         }
         __syncwarp();
+        if (!last) scores(1 - b);
       }
-      if (j + 1 == w.n_kv && kh < nreg && q_ok) {  // the query's rotary row, for the epilogue
-        const int32_t* gp = kh == 0 ? gpos : gpos2;
-        rope_load<HD>(rrow, rope_tab + (int64_t)(gp ? __ldg(gp + w.seg0 + q) : q) * E);
-      }
-      if (!track_wait_all(bar_mma2, tm2)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      if (warp == 0) {
-        if (j + 2 < w.n_kv) {
-          issue_kv(w, j + 2, b);
-        } else if (next) {  // pair b's last use in this unit: the next unit's tile of pair b
-          if (b < wn.n_kv) issue_kv(wn, b, b);
-          if (w.n_kv == 1 && wn.n_kv > 1) issue_kv(wn, 1, 1);  // pair 1 unused here
+      if (last) {
+        if (kh < nreg && q_ok) {  // the query's rotary row, for the epilogue
+          const int32_t* gp = kh == 0 ? gpos : gpos2;
+          rope_load<HD>(rrow, rope_tab + (int64_t)(gp ? __ldg(gp + w.seg0 + q) : q) * E);
         }
+        if (!track_wait_all(bar_mma2, tm2)) {
+          if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        // this pair's last use in the unit: the next unit's tile of the pair
+        if (warp == 0 && next && b < wn.n_kv) issue_kv(wn, b, b);
       }
     }
     if (!ok) break;
@@ -876,7 +953,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     track_drain(bar_qdo, tqdo);
     track_drain(bar_kv, tkv0);
     track_drain(bar_kv + 1, tkv1);
-    track_drain(bar_mma1, tm1);
+    track_drain(bar_s, ts);
+    track_drain(bar_dp, tdp);
     track_drain(bar_mma2, tm2);
   }
   tc_fence_before();
