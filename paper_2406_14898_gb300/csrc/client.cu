@@ -7,9 +7,9 @@
 // zero rows, final LayerNorm gamma/beta) live in one flat arena like the server's, so one
 // AdamW launch updates them all.
 //
-// Kernels here: embedding gather (warp per token, 16-byte rows) and its scatter-add
+// Kernels here: embedding gather (CTA per token, 16-byte rows) and its scatter-add
 // backward (fp32 atomics); the target count; the cross-entropy row kernel (one CTA per
-// row: online max / sum-exp over the fp32 logits, then the bf16 logit gradient
+// row, or a cluster for few rows: online max / sum-exp over the fp32 logits, then the bf16 gradient
 // (softmax - onehot) / n_targets, zero on the padded columns); the fixed-order loss sum.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -25,6 +25,7 @@
 #include "../../include/flglm_kernels.h"
 #include "common.cuh"
 #include "kernels.cuh"
+#include "ptx.cuh"
 
 int fl_server_create_keyed(const fl_server_cfg* cfg, uint64_t seed, int purpose, int block0, fl_server_t* out);
 
@@ -39,33 +40,65 @@ constexpr int BLOCK_BOTTOM = 0, BLOCK_TOP = 1, BLOCK_EMBED = 2, BLOCK_HEAD = 3;
 
 // ---------------------------------------------------------------------------- kernels
 
-__global__ void embed_gather_kernel(int T, int H, const int32_t* __restrict__ tokens, const bf16* __restrict__ table,
-                                    int V, bf16* __restrict__ out, int* __restrict__ status) {
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= T) return;
-  const int tok = tokens[w];
+// One CTA per token: its row copied (or added) in pieces requested together.  A warp per token
+// walked the row 512 bytes at a time (T = 2048, H = 4096: gather 7.0 us, scatter 15.7).
+constexpr int EMB_THREADS = 128;
+
+__global__ void __launch_bounds__(EMB_THREADS) embed_gather_kernel(int H, const int32_t* __restrict__ tokens,
+                                                                   const bf16* __restrict__ table, int V,
+                                                                   bf16* __restrict__ out, int* __restrict__ status) {
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
+  const int64_t t = blockIdx.x;
+  const int tok = tokens[t];
   const bool ok = tok >= 0 && tok < V;
-  if (!ok && lane == 0) atomicOr(status, ST_TOKEN);
+  if (!ok && threadIdx.x == 0) atomicOr(status, ST_TOKEN);
   const uint4* src = reinterpret_cast<const uint4*>(table + (int64_t)(ok ? tok : 0) * H);
-  uint4* dst = reinterpret_cast<uint4*>(out + w * H);
-  for (int i = lane; i < H / 8; i += 32) dst[i] = ok ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
+  uint4* dst = reinterpret_cast<uint4*>(out + t * H);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < H / 8; i += EMB_THREADS) dst[i] = ok ? __ldg(src + i) : make_uint4(0u, 0u, 0u, 0u);
 }
 
-__global__ void embed_scatter_kernel(int T, int H, const int32_t* __restrict__ tokens, int V,
-                                     const bf16* __restrict__ dX, float* __restrict__ dE) {
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= T) return;
-  const int tok = tokens[w];
+// V4: 8-byte pieces of dX and 16-byte vector reductions (H % 4 == 0, dX 8-byte and dE 16-byte
+// aligned); otherwise one reduction per element.
+template <bool V4>
+__global__ void __launch_bounds__(EMB_THREADS) embed_scatter_kernel(int H, const int32_t* __restrict__ tokens, int V,
+                                                                    const bf16* __restrict__ dX,
+                                                                    float* __restrict__ dE) {
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
+  const int64_t t = blockIdx.x;
+  const int tok = tokens[t];
   if (tok < 0 || tok >= V) return;
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(dX + w * H);
   float* dst = dE + (int64_t)tok * H;
-  for (int i = lane; i < H / 2; i += 32) {
-    const float2 v = unpack_bf16x2(src[i]);
-    atomicAdd(dst + 2 * i, v.x);
-    atomicAdd(dst + 2 * i + 1, v.y);
+  if constexpr (V4) {
+    const uint2* src = reinterpret_cast<const uint2*>(dX + t * H);
+#pragma unroll 8
+    for (int i = threadIdx.x; i < H / 4; i += EMB_THREADS) {
+      const uint2 u = __ldg(src + i);
+      const float2 a = unpack_bf16x2(u.x), b = unpack_bf16x2(u.y);
+      red_add_v4(dst + 4 * i, a.x, a.y, b.x, b.y);
+    }
+  } else {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(dX + t * H);
+    for (int i = threadIdx.x; i < H / 2; i += EMB_THREADS) {
+      const float2 v = unpack_bf16x2(src[i]);
+      atomicAdd(dst + 2 * i, v.x);
+      atomicAdd(dst + 2 * i + 1, v.y);
+    }
   }
+}
+
+// Adds the rows of dX to the embedding gradient rows of their tokens.
+cudaError_t launch_embed_scatter(int T, int H, const int32_t* tokens, int V, const void* dX, float* dE, cudaStream_t st) {
+  const bool v4 = H % 4 == 0 && !fl_misaligned(dX, 8) && !fl_misaligned(dE, 16);
+  return v4 ? fl_launch(embed_scatter_kernel<true>, dim3(T), dim3(EMB_THREADS), 0, st, H, tokens, V, (const bf16*)dX, dE)
+            : fl_launch(embed_scatter_kernel<false>, dim3(T), dim3(EMB_THREADS), 0, st, H, tokens, V, (const bf16*)dX, dE);
+}
+cudaError_t launch_embed_gather(int T, int H, const int32_t* tokens, const void* table, int V, void* out, int* status,
+                                cudaStream_t st) {
+  return fl_launch(embed_gather_kernel, dim3(T), dim3(EMB_THREADS), 0, st, H, tokens, (const bf16*)table, V, (bf16*)out,
+                   status);
 }
 
 template <typename T>
@@ -83,6 +116,8 @@ FL_DEV T block_sum(T v, T* red) {
 
 __global__ void __launch_bounds__(RED_THREADS) count_kernel(int T, const int32_t* __restrict__ labels, int V,
                                                             int* __restrict__ count, int* __restrict__ status) {
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
   __shared__ int red[32];
   int c = 0, bad = 0;
   for (int t = threadIdx.x; t < T; t += blockDim.x) {
@@ -103,59 +138,194 @@ FL_DEV void lse_combine(float& m, float& s, float m2, float s2) {
   m = mn;
 }
 
-__global__ void __launch_bounds__(CE_THREADS) ce_kernel(int V, int64_t ld, const float* __restrict__ logits,
-                                                        const int32_t* __restrict__ labels,
-                                                        const int* __restrict__ count, float* __restrict__ row_loss,
-                                                        bf16* __restrict__ dlogits) {
-  __shared__ float rm[CE_THREADS / 32], rs[CE_THREADS / 32];
-  const int row = blockIdx.x;
-  const float* l = logits + (int64_t)row * ld;
-  // pass 1: online max and sum of exponentials
-  float m = -INFINITY, s = 0.f;
-  const int V4 = V / 4;
-  for (int j = threadIdx.x; j < V4; j += blockDim.x) {
-    const float4 x = __ldg(reinterpret_cast<const float4*>(l) + j);
-    const float xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) lse_combine(m, s, xs[q], 1.f);
-  }
-  for (int j = 4 * V4 + threadIdx.x; j < V; j += blockDim.x) lse_combine(m, s, __ldg(l + j), 1.f);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
-    lse_combine(m, s, m2, s2);
-  }
+// Cross-entropy rows, a CTA each: pass 1 the online max and sum of exponentials (CE_NV float4 per
+// thread requested together, one rescale per batch), pass 2 the bf16 gradient of the mean loss,
+// zero on the padded columns.  Persistent, with no more rows at work than L2 holds, so that
+// pass 2 reads the logits there: HBM sees 4 B read and 2 B written per column.  1024 rows of 130528
+// columns: 203 us, 3.9 TB/s (260 with four CTAs per SM and a rescale per element).  Bound by the
+// latency of a batch: a thread requests the next one after it has reduced the last.
+constexpr int CE_NV = 8;
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+    ce_kernel(int T, int V, int64_t ld, const float* __restrict__ logits, const int32_t* __restrict__ labels,
+              const int* __restrict__ count, float* __restrict__ row_loss, bf16* __restrict__ dlogits) {
+  constexpr int W = THREADS / 32;
+  __shared__ float2 red[2][W];  // rows alternate, so that one barrier per row suffices
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    rm[warp] = m;
-    rs[warp] = s;
-  }
-  __syncthreads();
-  m = -INFINITY;
-  s = 0.f;
-  for (int i = 0; i < CE_THREADS / 32; ++i) lse_combine(m, s, rm[i], rs[i]);
-  const float lse = m + __logf(s);
-  const int y = labels[row];
-  const bool valid = y >= 0 && y < V;
-  const float inv = valid ? 1.f / (float)max(*count, 1) : 0.f;
-  if (threadIdx.x == 0) row_loss[row] = valid ? lse - l[y] : 0.f;
-  // pass 2: gradient of the mean loss w.r.t. the logits, 4 columns per thread; the
-  // padded columns [V, ld) get zeros
-  bf16* d = dlogits + (int64_t)row * ld;
-  const int ld4 = (int)(ld / 4);
-  for (int j4 = threadIdx.x; j4 < ld4; j4 += blockDim.x) {
-    float g[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int j = 4 * j4 + q;
-      g[q] = j < V ? (__expf(__ldg(l + j) - lse) - (j == y ? 1.f : 0.f)) * inv : 0.f;
+  const int ld4 = (int)(ld / 4), v4 = (V + 3) / 4;
+  int par = 0;
+  for (int64_t row = blockIdx.x; row < T; row += gridDim.x) {
+    const int y = labels[row];
+    uint2* d = reinterpret_cast<uint2*>(dlogits + row * ld);
+    if (y < 0 || y >= V) {  // no target
+      for (int j = threadIdx.x; j < ld4; j += THREADS) __stcs(d + j, make_uint2(0u, 0u));
+      if (threadIdx.x == 0) row_loss[row] = 0.f;
+      continue;
     }
-    *reinterpret_cast<uint2*>(d + 4 * j4) = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+    const float* l = logits + row * ld;
+    const float4* l4 = reinterpret_cast<const float4*>(l);
+    float m = -INFINITY, s = 0.f;
+    for (int j0 = 0; j0 < v4; j0 += CE_NV * THREADS) {
+      float4 x[CE_NV];
+#pragma unroll
+      for (int k = 0; k < CE_NV; ++k) {
+        const int j = j0 + k * THREADS + threadIdx.x;
+        x[k] = j < v4 ? __ldg(l4 + j) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      }
+      float mt = -INFINITY;
+#pragma unroll
+      for (int k = 0; k < CE_NV; ++k) {
+        const int j = 4 * (j0 + k * THREADS + threadIdx.x);
+        if (j + 1 >= V) x[k].y = -INFINITY;  // columns past the vocabulary
+        if (j + 2 >= V) x[k].z = -INFINITY;
+        if (j + 3 >= V) x[k].w = -INFINITY;
+        mt = fmaxf(mt, fmaxf(fmaxf(x[k].x, x[k].y), fmaxf(x[k].z, x[k].w)));
+      }
+      const float mn = fmaxf(m, mt), mref = mn == -INFINITY ? 0.f : mn;
+      float st = 0.f;
+#pragma unroll
+      for (int k = 0; k < CE_NV; ++k)
+        st += (__expf(x[k].x - mref) + __expf(x[k].y - mref)) + (__expf(x[k].z - mref) + __expf(x[k].w - mref));
+      s = s * __expf(m - mref) + st;  // m = -inf: s is 0 and so is the factor
+      m = mn;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
+      lse_combine(m, s, m2, s2);
+    }
+    if (lane == 0) red[par][warp] = make_float2(m, s);
+    __syncthreads();
+    m = -INFINITY;
+    s = 0.f;
+#pragma unroll
+    for (int i = 0; i < W; ++i) lse_combine(m, s, red[par][i].x, red[par][i].y);
+    par ^= 1;
+    const float lse = m + logf(s);
+    const float inv = 1.f / (float)max(*count, 1);
+    if (threadIdx.x == 0) row_loss[row] = lse - l[y];
+    for (int j0 = 0; j0 < ld4; j0 += CE_NV * THREADS) {
+      float4 x[CE_NV];
+#pragma unroll
+      for (int k = 0; k < CE_NV; ++k) {
+        const int j = j0 + k * THREADS + threadIdx.x;
+        x[k] = j < v4 ? __ldcs(l4 + j) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      }
+#pragma unroll
+      for (int k = 0; k < CE_NV; ++k) {
+        const int j = j0 + k * THREADS + threadIdx.x;
+        const float xs[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+        float g[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          g[q] = 4 * j + q < V ? (__expf(xs[q] - lse) - (4 * j + q == y ? 1.f : 0.f)) * inv : 0.f;
+        if (j < ld4) __stcs(d + j, make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3])));
+      }
+    }
+  }
+}
+
+// Few long rows: a cluster of CE_CLUSTER CTAs holds one in registers, NV float4 per thread; max
+// and sum of exponentials per CTA, combined in rank order through the CTAs' shared memory, then
+// the gradient from the exponentials at hand.  Clusters walk rows cluster, + clusters, ...
+// A row costs its latency (about 6 us; 32 rows of 130528 columns: 10 us, about 24 by a CTA each), which
+// many rows would add up (1024 rows: 275 us, 203 by a CTA each).
+constexpr int CE_CLUSTER = 8;
+
+template <int NV>
+__global__ void __cluster_dims__(CE_CLUSTER, 1, 1) __launch_bounds__(CE_THREADS, 2)
+    ce_cluster_kernel(int T, int V, int64_t ld, const float* __restrict__ logits, const int32_t* __restrict__ labels,
+                      const int* __restrict__ count, float* __restrict__ row_loss, bf16* __restrict__ dlogits) {
+  constexpr int W = CE_THREADS / 32;
+  __shared__ float red[2][W];
+  __shared__ float2 part[2][CE_CLUSTER];  // (max, sum) of each CTA's columns; rows alternate
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
+  const int rank = (int)cluster_ctarank(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int clusters = gridDim.x / CE_CLUSTER;
+  const int ld4 = (int)(ld / 4);
+  int par = 0;
+  for (int row = blockIdx.x / CE_CLUSTER; row < T; row += clusters) {
+    const int y = labels[row];
+    uint2* d = reinterpret_cast<uint2*>(dlogits + (int64_t)row * ld);
+    if (y < 0 || y >= V) {  // no target (the same for the whole cluster)
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        const int j4 = (k * CE_CLUSTER + rank) * CE_THREADS + threadIdx.x;
+        if (j4 < ld4) d[j4] = make_uint2(0u, 0u);
+      }
+      if (rank == 0 && threadIdx.x == 0) row_loss[row] = 0.f;
+      continue;
+    }
+    const float* l = logits + (int64_t)row * ld;
+    float4 x[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int j4 = (k * CE_CLUSTER + rank) * CE_THREADS + threadIdx.x;
+      x[k] = 4 * j4 < V ? __ldg(reinterpret_cast<const float4*>(l) + j4)
+                        : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    }
+    float m = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int j = 4 * ((k * CE_CLUSTER + rank) * CE_THREADS + threadIdx.x);
+      if (j + 1 >= V) x[k].y = -INFINITY;  // columns past the vocabulary
+      if (j + 2 >= V) x[k].z = -INFINITY;
+      if (j + 3 >= V) x[k].w = -INFINITY;
+      m = fmaxf(m, fmaxf(fmaxf(x[k].x, x[k].y), fmaxf(x[k].z, x[k].w)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) red[0][warp] = m;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < W; ++i) m = fmaxf(m, red[0][i]);
+    const float mref = m == -INFINITY ? 0.f : m;
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      x[k] = make_float4(__expf(x[k].x - mref), __expf(x[k].y - mref), __expf(x[k].z - mref), __expf(x[k].w - mref));
+      s += (x[k].x + x[k].y) + (x[k].z + x[k].w);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) red[1][warp] = s;
+    __syncthreads();
+    s = 0.f;
+#pragma unroll
+    for (int i = 0; i < W; ++i) s += red[1][i];
+    if (threadIdx.x < CE_CLUSTER)  // to every CTA of the cluster
+      st_cluster_f2(mapa_shared(smem_u32(&part[par][rank]), threadIdx.x), m, s);
+    cluster_sync();
+    float M = -INFINITY, S = 0.f;
+#pragma unroll
+    for (int i = 0; i < CE_CLUSTER; ++i) {
+      const float2 q = part[par][i];
+      lse_combine(M, S, q.x, q.y);
+    }
+    par ^= 1;
+    const float inv = 1.f / (float)max(*count, 1);
+    const float f = __expf(mref - M) / S;  // exponential at hand -> probability
+    if (rank == 0 && threadIdx.x == 0) row_loss[row] = M + logf(S) - l[y];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int j4 = (k * CE_CLUSTER + rank) * CE_THREADS + threadIdx.x;
+      float g[4] = {x[k].x * f, x[k].y * f, x[k].z * f, x[k].w * f};
+      const int hit = y - 4 * j4;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g[q] = (g[q] - (q == hit ? 1.f : 0.f)) * inv;
+      if (j4 < ld4) d[j4] = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+    }
   }
 }
 
 __global__ void __launch_bounds__(RED_THREADS) loss_kernel(int T, const float* __restrict__ row_loss,
                                                            const int* __restrict__ count, float* __restrict__ loss) {
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
   __shared__ float red[32];
   float s = 0.f;
   for (int t = threadIdx.x; t < T; t += blockDim.x) s += row_loss[t];
@@ -163,7 +333,47 @@ __global__ void __launch_bounds__(RED_THREADS) loss_kernel(int T, const float* _
   if (threadIdx.x == 0) *loss = s / (float)max(*count, 1);
 }
 
-int warps_grid(int64_t rows) { return (int)((rows * 32 + 255) / 256); }
+template <int NV>
+cudaError_t launch_ce_cluster(int T, int V, int64_t ld, const float* logits, const int32_t* labels, const int* count,
+                              float* row_loss, void* dlogits, cudaStream_t st) {
+  int clusters = 2 * fl_sm_count() / CE_CLUSTER;  // two CTAs per SM
+  if (clusters > T) clusters = T;
+  return fl_launch(ce_cluster_kernel<NV>, dim3(clusters * CE_CLUSTER), dim3(CE_THREADS), 0, st, T, V, ld, logits, labels,
+                   count, row_loss, (bf16*)dlogits);
+}
+
+// Target count, rows, loss.
+cudaError_t launch_cross_entropy(int T, int V, int64_t ld, const float* logits, const int32_t* labels, float* row_loss,
+                                 void* dlogits, float* loss, int* count, int* status, cudaStream_t st) {
+  constexpr int64_t PER_NV = (int64_t)CE_CLUSTER * CE_THREADS * 4;
+  cudaError_t e = fl_launch(count_kernel, dim3(1), dim3(RED_THREADS), 0, st, T, labels, V, count, status);
+  if (e != cudaSuccess) return e;
+  // rows longer than one register batch of a CTA, on fewer than half of the SMs: a cluster each
+  const bool few = 2 * T <= fl_sm_count() && ld > PER_NV && ld <= 8 * PER_NV;
+  if (T == 0) {
+    // no rows
+  } else if (few) {
+    e = ld <= 2 * PER_NV   ? launch_ce_cluster<2>(T, V, ld, logits, labels, count, row_loss, dlogits, st)
+        : ld <= 4 * PER_NV ? launch_ce_cluster<4>(T, V, ld, logits, labels, count, row_loss, dlogits, st)
+                           : launch_ce_cluster<8>(T, V, ld, logits, labels, count, row_loss, dlogits, st);
+  } else {
+    // threads and rows per SM by the row's length, the rows at work within the 126 MB L2: 1024 rows
+    // of 16384 columns take 30 us with 256 threads, of 32768 55 with 512 (82 with 1024), of 130528
+    // 203 with 1024 (248 with 512, two rows per SM overflowing L2)
+    const int sms = fl_sm_count();
+    if (ld > 4 * PER_NV)
+      e = fl_launch(ce_kernel<1024>, dim3(T < sms ? T : sms), dim3(1024), 0, st, T, V, ld, logits, labels,
+                    (const int*)count, row_loss, (bf16*)dlogits);
+    else if (ld > PER_NV)
+      e = fl_launch(ce_kernel<512>, dim3(T < 2 * sms ? T : 2 * sms), dim3(512), 0, st, T, V, ld, logits, labels,
+                    (const int*)count, row_loss, (bf16*)dlogits);
+    else
+      e = fl_launch(ce_kernel<256>, dim3(T < 4 * sms ? T : 4 * sms), dim3(256), 0, st, T, V, ld, logits, labels,
+                    (const int*)count, row_loss, (bf16*)dlogits);
+  }
+  if (e != cudaSuccess) return e;
+  return fl_launch(loss_kernel, dim3(1), dim3(RED_THREADS), 0, st, T, (const float*)row_loss, (const int*)count, loss);
+}
 
 }  // namespace
 
@@ -176,9 +386,7 @@ extern "C" int fl_k_embedding_gather(int32_t T, int32_t H, const int32_t* tokens
   if (fl_misaligned(table, 16) || fl_misaligned(out, 16) || fl_misaligned(tokens, 4) || fl_misaligned(status, 4))
     return fl_internal_error(FL_ERR_INVALID_ARG, "embedding gather: table and out must be 16-byte aligned");
   if (T == 0) return FL_OK;
-  embed_gather_kernel<<<warps_grid(T), 256, 0, (cudaStream_t)stream>>>(T, H, tokens, (const bf16*)table, vocab,
-                                                                       (bf16*)out, status);
-  FL_CUDA_TRY(cudaGetLastError());
+  FL_CUDA_TRY(launch_embed_gather(T, H, tokens, table, vocab, out, status, (cudaStream_t)stream));
   return FL_OK;
 }
 
@@ -189,8 +397,7 @@ extern "C" int fl_k_embedding_scatter_add(int32_t T, int32_t H, const int32_t* t
   if (fl_misaligned(dx, 4) || fl_misaligned(dtable, 4) || fl_misaligned(tokens, 4))
     return fl_internal_error(FL_ERR_INVALID_ARG, "embedding scatter: dx, dtable and tokens must be 4-byte aligned");
   if (T == 0) return FL_OK;
-  embed_scatter_kernel<<<warps_grid(T), 256, 0, (cudaStream_t)stream>>>(T, H, tokens, vocab, (const bf16*)dx, dtable);
-  FL_CUDA_TRY(cudaGetLastError());
+  FL_CUDA_TRY(launch_embed_scatter(T, H, tokens, vocab, dx, dtable, (cudaStream_t)stream));
   return FL_OK;
 }
 
@@ -201,11 +408,8 @@ extern "C" int fl_k_cross_entropy(int32_t T, int32_t vocab, int64_t ld, const fl
     return fl_internal_error(FL_ERR_INVALID_ARG, "cross entropy: args");
   if ((reinterpret_cast<uintptr_t>(logits) & 15) || (reinterpret_cast<uintptr_t>(dlogits) & 7))
     return fl_internal_error(FL_ERR_INVALID_ARG, "cross entropy: alignment");
-  cudaStream_t st = (cudaStream_t)stream;
-  count_kernel<<<1, RED_THREADS, 0, st>>>(T, labels, vocab, count, status);
-  if (T > 0) ce_kernel<<<T, CE_THREADS, 0, st>>>(vocab, ld, logits, labels, count, row_loss, (bf16*)dlogits);
-  loss_kernel<<<1, RED_THREADS, 0, st>>>(T, row_loss, count, loss);
-  FL_CUDA_TRY(cudaGetLastError());
+  FL_CUDA_TRY(launch_cross_entropy(T, vocab, ld, logits, labels, row_loss, dlogits, loss, count, status,
+                                   (cudaStream_t)stream));
   return FL_OK;
 }
 
@@ -453,10 +657,9 @@ extern "C" int fl_client_bottom_forward(fl_client_t c, const int32_t* tokens, in
   }
   cudaError_t e = cudaMemcpyAsync(c->tokens, tokens, (size_t)c->T * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream);
   if (e != cudaSuccess) return cl_set(c, FL_ERR_CUDA, "bottom_forward: token copy: %s", cudaGetErrorString(e));
-  embed_gather_kernel<<<warps_grid(c->T), 256, 0, c->stream>>>(c->T, c->H, c->tokens, c->wb + c->off_embed, c->V, c->x0,
-                                                               c->status);
   c->launches += 1;
-  if ((e = cudaGetLastError()) != cudaSuccess) return cl_set(c, FL_ERR_CUDA, "embed gather: %s", cudaGetErrorString(e));
+  e = launch_embed_gather(c->T, c->H, c->tokens, c->wb + c->off_embed, c->V, c->x0, c->status, c->stream);
+  if (e != cudaSuccess) return cl_set(c, FL_ERR_CUDA, "embed gather: %s", cudaGetErrorString(e));
   const void* in[1] = {c->x0};
   void* outp[1] = {h0};
   const int32_t lens[1] = {seq_len};
@@ -495,11 +698,9 @@ extern "C" int fl_client_top_forward_backward(fl_client_t c, const void* h, cons
   a.epilogue = FL_EPI_STORE_F32;
   if ((rc = run_gemm(c, a))) return rc;
   // loss and dloss/dlogits
-  count_kernel<<<1, RED_THREADS, 0, st>>>(T, labels, c->V, c->count, c->status);
-  ce_kernel<<<T, CE_THREADS, 0, st>>>(c->V, c->Vp, c->logits, labels, c->count, c->row_loss, c->dlogits);
-  loss_kernel<<<1, RED_THREADS, 0, st>>>(T, c->row_loss, c->count, loss);
   c->launches += 3;
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_cross_entropy(T, c->V, c->Vp, c->logits, labels, c->row_loss, c->dlogits, loss, c->count,
+                                             c->status, st);
   if (e != cudaSuccess) return cl_set(c, FL_ERR_CUDA, "cross-entropy: %s", cudaGetErrorString(e));
   // head gradient (accumulated), then dz = dlogits W_head
   if (c->train_own) {
@@ -541,10 +742,8 @@ extern "C" int fl_client_bottom_backward(fl_client_t c, const void* grad_h0) {
   void* gi[1] = {c->dx0};
   if (int rc = fl_server_backward(c->bottom, go, gi)) return srv_err(c, c->bottom, rc);
   if (c->train_own) {
-    embed_scatter_kernel<<<warps_grid(c->T), 256, 0, c->stream>>>(c->T, c->H, c->tokens, c->V, c->dx0,
-                                                                  c->g + c->off_embed);
     c->launches += 1;
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_embed_scatter(c->T, c->H, c->tokens, c->V, c->dx0, c->g + c->off_embed, c->stream);
     if (e != cudaSuccess) return cl_set(c, FL_ERR_CUDA, "embed scatter: %s", cudaGetErrorString(e));
   }
   c->phase = 0;

@@ -225,6 +225,10 @@ FL_DEV uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
+// Two floats to a shared::cluster address (8-byte aligned).
+FL_DEV void st_cluster_f2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
 // Arrive on an mbarrier given by its shared::cluster address (this CTA's or the peer's).  CTA
 // scope: what the arrival orders is the thread's TMEM reads (behind tc_fence_before); a
 // cluster-scope release would also wait for every global store the thread has in flight.

@@ -289,6 +289,64 @@ def test_cross_entropy_kernel(F, V, ld):
     assert not got[[0, 9, 30]].any()
 
 
+@pytest.mark.parametrize("V,ld", [(16381, 16384), (16385, 16388), (32766, 32768), (32769, 32776), (65536, 65540),
+                                  (131071, 131072), (131073, 131076)])
+def test_cross_entropy_row_lengths(F, V, ld):
+    """Row lengths on both sides of every change of kernel, more rows than clusters, columns
+    that are masked (-inf, the lowest float) or far apart, a label on the last column; each
+    probability within 8 fp32 ulps plus one bf16 rounding of the result."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    T = 90
+    x = 2.0 * torch.randn((T, ld), generator=g, device="cuda")
+    x[1, : V // 2] = -float("inf")
+    x[2, 3::7] = torch.finfo(torch.float32).min
+    x[3, 5] += 80.0
+    x[4] -= 1000.0
+    x[:, V:] = float("inf")  # padding is not read into the softmax
+    lab = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    lab[0], lab[1], lab[5], lab[89] = V - 1, V - 1, -1, -3
+    row = torch.empty(T, device="cuda")
+    dlog = torch.full((T, ld), 7.0, dtype=torch.bfloat16, device="cuda")
+    loss = torch.empty(1, device="cuda")
+    cnt = torch.empty(1, dtype=torch.int32, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    F.fl_k_cross_entropy(T, V, ld, x, lab, row, dlog, loss, cnt, st)
+    torch.cuda.synchronize()
+    n = T - 2
+    assert int(cnt.item()) == n and int(st.item()) == 0
+    xd, ld_ = x[:, :V].double(), lab.long()
+    lse = torch.logsumexp(xd, 1)
+    keep = ld_ >= 0
+    want_row = torch.where(keep, lse - xd.gather(1, ld_.clamp(min=0)[:, None])[:, 0], torch.zeros_like(lse))
+    # fp32: the exponent's argument is rounded (|x - max| <= 2^11 here), and so is the loss itself
+    assert ((row.double() - want_row).abs() <= 2.0 ** -21 * (1.0 + want_row.abs() + lse.abs())).all()
+    assert abs(loss.item() - want_row.sum().item() / n) <= 2e-6 * max(1.0, want_row.sum().item() / n)
+    p = torch.exp(xd - lse[:, None])
+    p[torch.arange(T, device="cuda"), ld_.clamp(min=0)] -= 1.0
+    want = p * keep[:, None] / n
+    err = (dlog[:, :V].double() - want).abs()
+    assert (err <= 2.0 ** -8 * want.abs() + 2.0 ** -18 / n + 1e-38).all()
+    assert not dlog[:, V:].any() and not dlog[~keep].any()
+
+
+@pytest.mark.parametrize("H,off", [(256, 0), (256, 2), (258, 0), (4096, 4)])
+def test_embedding_scatter_alignment(F, H, off):
+    """Vector and element-wise reductions by the alignment of the gradient and the width."""
+    g = torch.Generator(device="cuda").manual_seed(H + off)
+    V, T = 50, 200
+    tok = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    tok[7] = V
+    buf = torch.randn(T * H + off, generator=g, device="cuda").bfloat16()
+    dx = buf[off:]
+    dE = torch.zeros(V * H + 4, device="cuda")[: V * H]
+    F.fl_k_embedding_scatter_add(T, H, tok, V, dx, dE)
+    torch.cuda.synchronize()
+    ok = tok < V
+    want = torch.zeros((V, H), device="cuda", dtype=torch.float64).index_add_(0, tok[ok].long(), dx.view(T, H)[ok].double())
+    # at most T fp32 additions per element, in any order
+    assert ((dE.view(V, H).double() - want).abs() <= T * 2.0 ** -23 * 6.0).all()
+
+
 def test_embedding_kernels(F):
     rng = np.random.default_rng(5)
     V, H, T = 300, 256, 77
