@@ -120,14 +120,6 @@ FL_DEV void inverse_rope_row(float* v, const RopeRow<HD>& rr) {
   }
 }
 
-// 2^x by the hardware instruction (PTX ex2.approx.ftz.f32): the probabilities it feeds are
-// rounded to bf16 for the tensor cores.
-FL_DEV float exp2_hw(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Staged bf16 tile in the layout of 128-byte-swizzled TMA boxes of 64 columns x 128 rows:
 // 16-byte chunk j of row r in box j / 8, at chunk (j % 8) ^ (r % 8) of the box's row r.
 template <int HD>

@@ -3,21 +3,26 @@
 // keys, causal within the segment or with a bidirectional GLM context; §3.3 segments are
 // never mixed), with both tile contractions on tcgen05 and their accumulators in TMEM.
 //
-// Persistent CTAs (4 warps, two per SM) walk the (128-query tile, head) units; the next
-// unit's Q and first K / V tiles load while a unit's output is written.  Thread i owns
+// Persistent CTAs (4 warps, two per SM) walk the (128-query tile, head) units.  Thread i owns
 // query row i, which is TMEM lane i.  Per 128-key tile j:
 //   TMA: K_j and V_j (128 rows x head_dim, 64-column 128-byte-swizzled boxes; Q once),
 //        each on its own barrier;
-//   S = Q K_j^T     -> TMEM columns [0, 128)   (tcgen05.mma, both operands in shared memory);
-//        K_j's buffer is free once S is complete: K_{j+1} is loaded right away;
+//   S = Q K_j^T     -> TMEM columns [0, 128)   (tcgen05.mma, both operands in shared memory),
+//        issued right behind the P V of the tile before it; once it is complete, so is that
+//        P V, and K_(j+1) (after a unit's last tile the next unit's Q and K) and V_j are loaded;
 //   softmax: the thread's S row (masked max, exp2, row sum); P (bf16, two per 32-bit
 //        column) is stored back into the first 64 columns of S; the O row is rescaled when
 //        the running max moved;
 //   O += P V_j      -> TMEM columns [128, 128 + head_dim) (A = P read from TMEM, V_j as an
-//        MN-major operand); then V_{j+1} is loaded.
+//        MN-major operand).
+// The next unit's first scores run while a unit's output is written.
 // Shared memory: three tiles (96 KB at head_dim 128); 256 TMEM columns: two CTAs per SM
-// overlap each other's copies and softmax.  Every mbarrier wait is bounded (2 s): on
-// expiry the CTA records a status code and leaves its remaining work undone.
+// overlap each other's copies and softmax.  Bound at 256-token segments by HBM (8 H bytes per
+// token), at long ones by the softmax threads: 32 x 256 tokens x
+// 32 heads 72 -> 65 us, 4.2 TB/s; 4 x 2048 tokens 249 -> 196 us, 700 TFLOP/s (before: loads only
+// after a unit's last product, every product waited for, 16-byte stores of half sectors).
+// Every mbarrier wait is bounded (2 s): on expiry the CTA records a status code and leaves its
+// remaining work undone.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -79,6 +84,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int npt = Lp > 0 ? 1 : 0;  // at most one prefix tile (Lp <= 128)
+  const bool o32 = (reinterpret_cast<uintptr_t>(O) & 31) == 0;  // rows in whole 32-byte sectors per lane
 
   // A work unit u is (entry u / n_heads of the 128-row tile list, head u % n_heads): the
   // list's longest segments first, each segment's tiles together (last tile first).
@@ -136,95 +142,100 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
         tma_load_2d(dst + b * BOX, &tm_qkv, bar, (1 + part) * H + w.h * HD + 64 * b, row);
     }
   };
-  auto issue_unit = [&](const Unit& w) {  // Q and the first key / value tiles of a unit
+  auto issue_q = [&](const Unit& w) {
     tq.pend = true;
     __syncwarp();
-    if (elect_one()) {
-      mbar_arrive_expect_tx(bar_q, TILE);
+    if (!elect_one()) return;
+    mbar_arrive_expect_tx(bar_q, TILE);
 #pragma unroll
-      for (int b = 0; b < NB; ++b) tma_load_2d(sQ + b * BOX, &tm_qkv, bar_q, w.h * HD + 64 * b, w.seg0 + w.q0);
-    }
-    issue(w, 0, 0);
-    issue(w, 0, 1);
+    for (int b = 0; b < NB; ++b) tma_load_2d(sQ + b * BOX, &tm_qkv, bar_q, w.h * HD + 64 * b, w.seg0 + w.q0);
   };
 
   constexpr uint32_t IDESC_S = umma_idesc_bf16(TB, TB, false, false);
   constexpr uint32_t IDESC_PV = umma_idesc_bf16(TB, HD, false, true);
+  auto score = [&]() {  // warp 0: S = Q K^T of the tiles in place
+    tc_fence_after();
+    ts.pend = true;
+    __syncwarp();
+    if (elect_one()) {
+      const uint64_t aq = desc_kmajor(smem_u32(sQ)), bk = desc_kmajor(smem_u32(sK));
+#pragma unroll
+      for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, aq + step_kmajor(kk), bk + step_kmajor(kk), IDESC_S, kk > 0);
+      umma_commit(bar_s);
+    }
+    __syncwarp();
+  };
+  // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
+  auto wait_all = [&](uint64_t* bar, BarTrack& t, int code) {
+    const bool good = track_wait_all(bar, t);
+    if (!good && tid == 0) report_status(status, code);
+    return good;
+  };
   bool ok = true;
   int u = blockIdx.x;
   Unit w = u < n_units ? unit(u) : Unit{};
   Unit wn = u + (int)gridDim.x < n_units ? unit(u + gridDim.x) : Unit{};
-  if (warp == 0 && u < n_units) issue_unit(w);
-  while (u < n_units && ok) {
+  if (u < n_units) {
+    if (warp == 0) {
+      issue_q(w);
+      issue(w, 0, 0);
+      issue(w, 0, 1);
+    }
+    ok = wait_all(bar_q, tq, FL_DEV_TIMEOUT_FULL) && wait_all(bar_k, tk, FL_DEV_TIMEOUT_FULL);
+    if (ok && warp == 0) score();
+  }
+  while (u < n_units && ok) {  // the unit's first scores have been issued
     const int q = w.q0 + tid;  // this thread's query row (inside the segment)
     const int un = u + gridDim.x, unn = un + gridDim.x;
+    const bool next = un < n_units;
     // the descriptor of the unit after next, read in two steps while products run
     Unit wnn = Unit{};
     uint32_t tnn = 0;
     float m_run = -INFINITY, l_run = 0.f;
-    // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
-    if (!track_wait_all(bar_q, tq)) {
-      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-      ok = false;
-      break;
-    }
-    for (int j = 0; j < w.n_kv && ok; ++j) {
-      if (!track_wait_all(bar_k, tk)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
-      // ---- S = Q K_j^T (the previous P V, which read the S columns, has completed)
-      if (warp == 0) {
-        tc_fence_after();
-        ts.pend = true;
-        __syncwarp();
-        if (elect_one()) {
-          const uint64_t aq = desc_kmajor(smem_u32(sQ)), bk = desc_kmajor(smem_u32(sK));
-#pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk)
-            umma_bf16(tmem, aq + step_kmajor(kk), bk + step_kmajor(kk), IDESC_S, kk > 0);
-          umma_commit(bar_s);
-        }
-        __syncwarp();
-      }
+    for (int j = 0; j < w.n_kv; ++j) {
+      const bool last = j + 1 == w.n_kv;
       if (j == 0 && unn < n_units) tnn = tiles[unn / n_heads];
-      if (!track_wait_all(bar_s, ts)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
-        ok = false;
-        break;
-      }
+      // ---- S_j is complete, and so is the P V before it: K_j (after the last tile Q too) and
+      // V_(j-1) have been read
+      if (!(ok = wait_all(bar_s, ts, FL_DEV_TIMEOUT_ACC_FULL))) break;
       tc_fence_after();
-      if (warp == 0 && j + 1 < w.n_kv) issue(w, j + 1, 0);  // K_j has been read
+      if (warp == 0) {
+        if (j > 0) issue(w, j, 1);
+        if (!last) {
+          issue(w, j + 1, 0);
+        } else if (next) {
+          issue_q(wn);
+          issue(wn, 0, 0);
+        }
+      }
       // ---- the thread's S row, read once (4 x 32 columns, one wait)
       const bool prefix = j < npt;
       const int kb = prefix ? 0 : (j - npt) * TB;  // first key of the tile inside its sequence
       const int klim = prefix ? Lp - 1 : min(w.L - 1, max(q, w.clast));  // last visible key
-      const bool full = kb + TB - 1 <= klim;       // every key of the tile visible to this row
       uint32_t r[TB];
       tmem_ld32(t_s, *reinterpret_cast<uint32_t(*)[32]>(r));
       tmem_ld32(t_s + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
       tmem_ld32(t_s + 64, *reinterpret_cast<uint32_t(*)[32]>(r + 64));
       tmem_ld32(t_s + 96, *reinterpret_cast<uint32_t(*)[32]>(r + 96));
       tmem_ld_wait();
-      // masked row max; invisible keys become -inf
+      // masked row max; invisible keys become -inf (no masks where the warp's rows see every key)
+      if (!__all_sync(0xffffffffu, kb + TB - 1 <= klim)) {
+#pragma unroll
+        for (int e = 0; e < TB; ++e)
+          if (kb + e > klim) r[e] = 0xff800000u;
+      }
       float mt = -INFINITY;
 #pragma unroll
-      for (int e = 0; e < TB; ++e) {
-        float x = __uint_as_float(r[e]) * scale_log2;
-        if (!full && kb + e > klim) x = -INFINITY;
-        r[e] = __float_as_uint(x);
-        mt = fmaxf(mt, x);
-      }
-      const float m_new = fmaxf(m_run, mt);
+      for (int e = 0; e < TB; ++e) mt = fmaxf(mt, __uint_as_float(r[e]));
+      const float m_new = fmaxf(m_run, mt * scale_log2);
       const float mref = m_new == -INFINITY ? 0.f : m_new;
-      const float corr = exp2f(m_run - mref);  // 0 on the first tile (m_run = -inf)
+      const float corr = exp2_hw(m_run - mref);  // 0 on the first tile (m_run = -inf)
       // ---- P = exp2(S - m), bf16 pairs (keys 2c, 2c + 1 in column c) into S's columns [0, 64)
       float lt = 0.f;
 #pragma unroll
       for (int c = 0; c < TB / 2; ++c) {
-        const float p0 = exp2f(__uint_as_float(r[2 * c]) - mref);
-        const float p1 = exp2f(__uint_as_float(r[2 * c + 1]) - mref);
+        const float p0 = exp2_hw(fmaf(__uint_as_float(r[2 * c]), scale_log2, -mref));
+        const float p1 = exp2_hw(fmaf(__uint_as_float(r[2 * c + 1]), scale_log2, -mref));
         lt += p0 + p1;
         r[c] = pack_bf16x2(p0, p1);
       }
@@ -245,40 +256,35 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
           tmem_st32(t_o + c, o);
         }
       }
+      if (j == 0 && unn < n_units) wnn = unit_t(unn, tnn);
       tmem_st_wait();
       tc_fence_before();
-      if (!track_wait_all(bar_v, tv)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
+      if (!(ok = wait_all(bar_v, tv, FL_DEV_TIMEOUT_FULL))) break;
       // ---- O += P V_j
       if (warp == 0) {
         tc_fence_after();
-        tpv.pend = true;
+        if (last) tpv.pend = true;
         __syncwarp();
         if (elect_one()) {
           const uint64_t bv = desc_mnmajor(smem_u32(sV));
 #pragma unroll
           for (int kk = 0; kk < TB / 16; ++kk)
             umma_bf16_ts(tmem + 128, tmem + kk * 8, bv + step_mnmajor(kk), IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(bar_pv);
+          if (last) umma_commit(bar_pv);
         }
         __syncwarp();
       }
-      if (j == 0 && unn < n_units) wnn = unit_t(unn, tnn);
-      if (!track_wait_all(bar_pv, tpv)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
-        ok = false;
-        break;
+      // ---- the next scores behind it in the tensor pipe (they overwrite P, which it has read):
+      // this unit's next tile, or the next unit's first, whose product runs under this epilogue
+      if (!last || next) {
+        if (last && !(ok = wait_all(bar_q, tq, FL_DEV_TIMEOUT_FULL))) break;
+        if (!(ok = wait_all(bar_k, tk, FL_DEV_TIMEOUT_FULL))) break;
+        if (warp == 0) score();
       }
-      tc_fence_after();
-      if (warp == 0 && j + 1 < w.n_kv) issue(w, j + 1, 1);  // V_j has been read
     }
-    if (!ok) break;
-    // ---- every product of the unit is complete and Q / K / V are free: the next unit's
-    // first tiles load while this one's O leaves
-    if (warp == 0 && un < n_units) issue_unit(wn);
+    if (!ok || !(ok = wait_all(bar_pv, tpv, FL_DEV_TIMEOUT_ACC_EMPTY))) break;
+    tc_fence_after();
+    if (warp == 0 && next) issue(wn, 0, 1);  // the unit's last V has been read
     // ---- O / l and the log-sum-exp (every lane reads TMEM, all of the row at once; rows
     // past the segment end store nothing)
     const bool valid = q < w.L;
@@ -291,12 +297,18 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
       tmem_ld_wait();
       if (valid) {
 #pragma unroll
-        for (int v = 0; v < HD / 8; ++v)
-          *reinterpret_cast<uint4*>(orow + 8 * v) = make_uint4(
-              pack_bf16x2(__uint_as_float(o[8 * v]) * inv, __uint_as_float(o[8 * v + 1]) * inv),
-              pack_bf16x2(__uint_as_float(o[8 * v + 2]) * inv, __uint_as_float(o[8 * v + 3]) * inv),
-              pack_bf16x2(__uint_as_float(o[8 * v + 4]) * inv, __uint_as_float(o[8 * v + 5]) * inv),
-              pack_bf16x2(__uint_as_float(o[8 * v + 6]) * inv, __uint_as_float(o[8 * v + 7]) * inv));
+        for (int v = 0; v < HD / 16; ++v) {
+          uint32_t x[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            x[e] = pack_bf16x2(__uint_as_float(o[16 * v + 2 * e]) * inv, __uint_as_float(o[16 * v + 2 * e + 1]) * inv);
+          if (o32) {
+            st_global_v8(orow + 16 * v, x);
+          } else {
+            *reinterpret_cast<uint4*>(orow + 16 * v) = make_uint4(x[0], x[1], x[2], x[3]);
+            *reinterpret_cast<uint4*>(orow + 16 * v + 8) = make_uint4(x[4], x[5], x[6], x[7]);
+          }
+        }
       }
     }
     if (valid) lse[(int64_t)w.h * T + w.seg0 + q] = (m_run + log2f(l_run)) * LN2_T;

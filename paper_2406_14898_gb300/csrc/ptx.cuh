@@ -282,6 +282,13 @@ FL_DEV void red_add_v4(float* out, float a, float b, float c, float d) {
                : "memory");
 }
 
+// One 32-byte store (32-byte aligned address).
+FL_DEV void st_global_v8(void* p, const uint32_t (&x)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x[0]), "r"(x[1]), "r"(x[2]),
+               "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
+               : "memory");
+}
+
 // ------------------------------------------------------------------ warp-level MMA (attention)
 FL_DEV void ldmatrix_x4(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"

@@ -404,6 +404,25 @@ def test_attention_bwd_many_units(F, hd):
     assert rel_inf(got[:, sel(2 * H)], dvr.reshape(T, n)) < 5e-2
 
 
+@pytest.mark.parametrize("hd", [64, 128])
+def test_attention_forward_output_alignment(F, hd):
+    """An output that is only 16-byte aligned takes the narrower stores: the same bits."""
+    nh, lens = 4, [130, 1, 128, 40]
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    T, H = int(cu[-1]), nh * hd
+    g = torch.Generator(device="cuda").manual_seed(hd)
+    qkv = torch.randn((T, 3 * H), generator=g, device="cuda").bfloat16()
+    tiles = torch.empty(2 * F.fl_k_attention_tiles(cu), dtype=torch.int32, device="cuda")
+    out = []
+    for off in (0, 8):
+        o = torch.zeros(T * H + 16, dtype=torch.bfloat16, device="cuda")[off:off + T * H]
+        lse = torch.empty((nh, T), device="cuda")
+        F.fl_k_attention_fwd(T, nh, hd, qkv, cu, dev_i32(cu), tiles, o, lse)
+        out.append((bits(o), lse))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("hd,Lp", [(64, 16), (128, 100)])
 def test_attention_with_prefix(F, hd, Lp):
     """P-tuning v2 prefix (App. A): every query also sees Lp prefix keys/values (one or two
