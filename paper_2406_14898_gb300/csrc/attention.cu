@@ -85,7 +85,7 @@ int fl_launch_attn_fwd(int T, int nh, int hd, const void* qkv, const int32_t* cu
 }
 
 int fl_launch_attn_bwd(int T, int nh, int hd, const void* qkv, const void* o, const float* lse, const void* dout,
-                       const int32_t* cu, const uint32_t* tiles, int n_tiles, int n_tiles128, float* delta,
+                       const int32_t* cu, const uint32_t* tiles, int n_tiles, int n_tiles128, int max_tiles, float* delta,
                        const float* rope_tab, void* dqkv, const AttnPrefix& pre, const AttnGlm& glm, cudaStream_t st,
                        float* dbias, int* status, int dbias_segs, int64_t dbias_rstride) {
   if (n_tiles <= 0) return FL_OK;
@@ -98,7 +98,7 @@ int fl_launch_attn_bwd(int T, int nh, int hd, const void* qkv, const void* o, co
   else
     FL_CUDA_TRY(fl_launch(attn_delta_kernel<64>, dim3((unsigned)((pairs * 8 + 255) / 256)), dim3(256), 0, st, T, H,
                           nh, (const bf16*)o, (const bf16*)dout, delta));
-  return fl_launch_attn_bwd_tc(T, nh, hd, qkv, dout, lse, delta, cu, tiles + n_tiles, n_tiles128, rope_tab, dqkv, pre,
+  return fl_launch_attn_bwd_tc(T, nh, hd, qkv, dout, lse, delta, cu, tiles + n_tiles, n_tiles128, max_tiles, rope_tab, dqkv, pre,
                                glm, dbias, status, st, dbias_segs, dbias_rstride);
 }
 
@@ -112,7 +112,7 @@ extern "C" int32_t fl_k_attention_tiles(const int32_t* cu_host, int32_t S) {
 }
 
 // The 64-row tile list followed by the 128-row one (at most as long) in tile_ws.
-static int upload_tiles(const int32_t* cu_host, int32_t S, int32_t* tile_ws, int* n_out, int* n128_out) {
+static int upload_tiles(const int32_t* cu_host, int32_t S, int32_t* tile_ws, int* n_out, int* n128_out, int* max_out) {
   const int n = fl_k_attention_tiles(cu_host, S);
   for (int s = 0; s < S; ++s)
     if (cu_host[s + 1] < cu_host[s] || cu_host[s + 1] - cu_host[s] > 65535 * BT)
@@ -125,6 +125,7 @@ static int upload_tiles(const int32_t* cu_host, int32_t S, int32_t* tile_ws, int
   if (n > 0) FL_CUDA_TRY(cudaMemcpy(tile_ws, t.data(), (n + n128) * sizeof(uint32_t), cudaMemcpyHostToDevice));
   *n_out = n;
   *n128_out = n128;
+  *max_out = n128 > 0 ? int(t[n] & 0xFFFFu) + 1 : 0;  // the longest segment's last tile comes first
   return FL_OK;
 }
 
@@ -140,8 +141,8 @@ extern "C" int fl_k_attention_fwd(int32_t T, int32_t n_heads, int32_t head_dim, 
   if (fl_misaligned(qkv, 16) || fl_misaligned(o, 16) || fl_misaligned(lse, 4) || fl_misaligned(cu_seqlens, 4) ||
       fl_misaligned(tile_ws, 4) || fl_misaligned(context_lens, 4))
     return fl_internal_error(FL_ERR_INVALID_ARG, "attention fwd: qkv and o must be 16-byte aligned");
-  int n = 0, n128 = 0;
-  if (int rc = upload_tiles(cu_seqlens_host, S, tile_ws, &n, &n128)) return rc;
+  int n = 0, n128 = 0, max_tiles = 0;
+  if (int rc = upload_tiles(cu_seqlens_host, S, tile_ws, &n, &n128, &max_tiles)) return rc;
   AttnPrefix pre;
   pre.k = prefix_k;
   pre.v = prefix_v;
@@ -176,8 +177,8 @@ extern "C" int fl_k_attention_bwd(int32_t T, int32_t n_heads, int32_t head_dim, 
       fl_misaligned(context_lens, 4) || fl_misaligned(positions, 4) || fl_misaligned(block_positions, 4))
     return fl_internal_error(FL_ERR_INVALID_ARG,
                              "attention bwd: qkv, o, dout, dqkv and the prefix gradients must be 16-byte aligned");
-  int n = 0, n128 = 0;
-  if (int rc = upload_tiles(cu_seqlens_host, S, tile_ws, &n, &n128)) return rc;
+  int n = 0, n128 = 0, max_tiles = 0;
+  if (int rc = upload_tiles(cu_seqlens_host, S, tile_ws, &n, &n128, &max_tiles)) return rc;
   AttnPrefix pre;
   pre.k = prefix_k;
   pre.v = prefix_v;
@@ -189,5 +190,5 @@ extern "C" int fl_k_attention_bwd(int32_t T, int32_t n_heads, int32_t head_dim, 
   glm.pos = positions;
   glm.pos2 = block_positions;
   return fl_launch_attn_bwd(T, n_heads, head_dim, qkv, o, lse, dout, cu_seqlens, (const uint32_t*)tile_ws, n, n128,
-                            delta_ws, rope_tab, dqkv, pre, glm, (cudaStream_t)stream);
+                            max_tiles, delta_ws, rope_tab, dqkv, pre, glm, (cudaStream_t)stream);
 }

@@ -11,7 +11,8 @@
 // previous tile.
 //
 // Both kernels are persistent: one CTA per SM (226 KB of shared memory at head_dim 128,
-// 512 TMEM columns) walks work units u = blockIdx.x, + gridDim.x, ...  Each of the next
+// 512 TMEM columns) walks work units, in a fixed stride or as the hardware hands them out
+// (cluster launch control), see launch_bwd_tc.  Each of the next
 // unit's tiles is loaded as soon as its buffer has had its last use in the current unit,
 // so they arrive while the unit's last products run and its output is staged (in a tile
 // of its own) and written; a whole tile of output rows leaves by bulk tensor stores
@@ -24,10 +25,14 @@
 // query tile.  Per 128-query tile i that sees the key tile:
 //   TMA: Q_i and dO_i into the buffer pair (i % 2), the next tile's while this one works;
 //   S^T = K Q_i^T -> TMEM [0, 128)      dP^T = V dO_i^T -> TMEM [128, 256);
-//   threads: P^T = exp2(S^T scale log2e - lse_q log2e) where key r is visible to query q,
-//            dS^T = P^T (dP^T - delta_q), bf16 over the S^T / dP^T values just read;
-//   dV += P^T dO_i -> TMEM [256, 256 + hd)   dK += dS^T Q_i -> TMEM [256 + hd, 256 + 2 hd)
+//   threads: P^T = exp2(S^T scale log2e - lse_q log2e) where key r is visible to query q, as
+//            soon as S^T is complete; then, while dV += P^T dO_i -> TMEM [256, 256 + hd) runs,
+//            dS^T = P^T (dP^T - delta_q); both bf16 over the S^T / dP^T values just read;
+//   dK += dS^T Q_i -> TMEM [256 + hd, 256 + 2 hd), with S^T and dP^T of tile i + 1 right behind it
 //            (A from TMEM, dO_i and Q_i as MN-major operands).
+// Bound by the latency of that chain, one CTA per SM (cycles of a unit of one tile: loads and
+// scores 2200, P 1100-1800, dS 1200, dK 850, output 4400).  A ninth warp to issue the products
+// (the issuer waits for room in the tensor pipe) left 168 registers a thread and spilled.
 // Epilogue: dK * scale, the inverse rotary rotation(s), bf16 rows of dqkv and the k / v
 // column sums for the QKV bias gradient; the prefix variant (PREFIX: the unit's keys are
 // the prefix of its head, its query tiles a slice of the call's tile list) adds dK * scale
@@ -197,7 +202,9 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   uint64_t* bar_s = bars + 3;
   uint64_t* bar_dp = bars + 4;
   uint64_t* bar_mma2 = bars + 5;
-  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
+  uint64_t* bar_clc = bars + 6;
+  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // the unit taken over
+  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 10);
 
   const int nh = H / HD;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -255,7 +262,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   };
 
   if (tid == 0) {
-    for (int i = 0; i < 6; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < 7; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
     tma_prefetch_desc(&tm_do);
@@ -270,7 +277,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
-  BarTrack tkv, tq0, tq1, ts, tdp, tm2;
+  BarTrack tkv, tq0, tq1, ts, tdp, tm2, tclc;
   // Copies and products are issued by warp 0 as a whole, one elected lane at work: the
   // instructions' operands stay in uniform registers.
   auto issue_q = [&](const Unit& w, int it, int b) {  // Q_it, dO_it into pair b
@@ -306,9 +313,29 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   constexpr uint32_t IDESC_S = umma_idesc_bf16(TB, TB, false, false);
   constexpr uint32_t IDESC_G = umma_idesc_bf16(TB, HD, false, true);
   bool ok = true;
-  int u = blockIdx.x;
-  Unit w = u < n_units ? unit(u) : Unit{};
-  Unit wn = u + (int)gridDim.x < n_units ? unit(u + gridDim.x) : Unit{};
+  // Units: CTA c walks c, + gridDim.x, ..., or, when the grid has one CTA per unit, the hardware
+  // hands them out: the resident CTA takes over the next one that has not started, two units ahead
+  // of its work.
+  const bool handed = (int)gridDim.x == n_units;
+  int u_next = blockIdx.x;
+  auto take = [&]() {
+    if (!handed) return;
+    tclc.pend = true;
+    __syncwarp();
+    if (elect_one()) clc_request(clc, bar_clc);
+  };
+  auto taken = [&](int& x) {  // the unit taken, or -1
+    if (!handed) {
+      u_next += gridDim.x;
+      x = u_next < n_units ? u_next : -1;
+      return true;
+    }
+    ok = track_wait_all(bar_clc, tclc);
+    if (!ok && tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+    x = ok ? clc_answer(clc) : -1;
+    return ok;
+  };
+  Unit w = unit(blockIdx.x), wn = Unit{};
   // the thread's lse (tid < 128) or delta value of the next query tile, loaded a tile early
   auto stat_of = [&](const Unit& x, int it) {
     int row0, qpos0, valid;
@@ -317,23 +344,29 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     const float* src = tid < TB ? lse : delta;
     return c < valid ? __ldg(src + (int64_t)x.h * T + row0 + c) : 0.f;
   };
-  float pf = (u < n_units && w.it0 < w.it_end) ? stat_of(w, w.it0) : 0.f;
+  float pf = w.it0 < w.it_end ? stat_of(w, w.it0) : 0.f;
   RopeRow<HD> rrow;
-  if (warp == 0 && u < n_units && w.it0 < w.it_end) {
-    issue_kv(w);
-    issue_q(w, w.it0, 0);
-    if (w.it0 + 1 < w.it_end) issue_q(w, w.it0 + 1, 1);
+  if (warp == 0) {
+    if (w.it0 < w.it_end) {
+      issue_kv(w);
+      issue_q(w, w.it0, 0);
+      if (w.it0 + 1 < w.it_end) issue_q(w, w.it0 + 1, 1);
+    }
+    take();
   }
-  while (u < n_units && ok) {
+  int un;
+  if (taken(un) && un >= 0) wn = unit(un);
+  while (ok) {
     const int k = w.kb + r;  // the key inside its segment (or the prefix)
     const bool key_ok = PREFIX ? r < Lp : k < w.L;
     const bool work = w.it0 < w.it_end;
     // the next unit: its K / V load once this unit's last S^T / dP^T products have read K
     // and V, its first query tile once buffer pair 0 has had its last use here
-    const int un = u + gridDim.x;
-    const bool next = un < n_units && wn.it0 < wn.it_end;
-    Unit wnn = Unit{};  // the unit after next: its tile word read while the first score
-    uint32_t tnn = 0;   // products run, the rest while the first gradient products run
+    const bool next = un >= 0 && wn.it0 < wn.it_end;
+    Unit wnn = Unit{};  // the unit after next: taken over while the first score products run,
+    int unn = -1;       // read after the first pass
+    uint32_t tnn = 0;
+    if (un >= 0 && warp == 0) take();
     // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
     if (work && !track_wait_all(bar_kv, tkv)) {
       if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
@@ -378,7 +411,6 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       // while the products run: the next tile's statistics, the unit after next
       if (!last) pf = stat_of(w, it + 1);
       else if (next) pf = stat_of(wn, wn.it0);
-      if (it == w.it0 && un + (int)gridDim.x < n_units) tnn = tile_word(un + gridDim.x);
       if (!track_wait_all(bar_s, ts)) {
         if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
         ok = false;
@@ -435,7 +467,10 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       };
       if (open) probs(std::false_type{});
       else probs(std::true_type{});
-      if (it == w.it0 && un + (int)gridDim.x < n_units) wnn = unit_t(un + gridDim.x, tnn);
+      if (it == w.it0 && un >= 0) {
+        if (!taken(unn)) break;
+        if (unn >= 0) tnn = tile_word(unn);
+      }
       tmem_st_wait();
       tc_fence_before();
       if (!track_wait_all(bar_dp, tdp)) {
@@ -502,6 +537,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         __syncwarp();
         if (!last) scores(1 - b);
       }
+      // (its segment: two dependent loads, while the products run)
+      if (it == w.it0 && unn >= 0) wnn = unit_t(unn, tnn);
       if (last) {
         if (!PREFIX && qh < nreg && key_ok) {  // the key's rotary row, for the epilogue
           const int32_t* gp = qh == 0 ? gpos : gpos2;
@@ -558,12 +595,12 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
           const int part = 1 - pi;  // dV, then dK
           uint8_t* stage = sST;
           uint32_t vr[HD / 2];
+          float* v = reinterpret_cast<float*>(vr);
 #pragma unroll
           for (int c = 0; c < HD / 2; c += 32)
             tmem_ld32(t_lane + (part ? 256 : 256 + HD) + qh * (HD / 2) + c,
                       *reinterpret_cast<uint32_t(*)[32]>(vr + c));
           tmem_ld_wait();
-          float* v = reinterpret_cast<float*>(vr);
 #pragma unroll
           for (int c = 0; c < HD / 2; ++c) v[c] = __uint_as_float(vr[c]) * (part ? 1.f : scale);
           if (part == 0 && qh < nreg && key_ok) inverse_rope_row<HD>(v, rrow);  // rotary region qh
@@ -602,9 +639,14 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     // the dK / dV columns are loaded before the next unit's products overwrite them
     tc_fence_before();
     __syncthreads();
-    u = un;
+    if (un < 0) break;
+    if (!work) {  // no first pass to read the answer after
+      if (!taken(unn)) break;
+      if (unn >= 0) wnn = unit(unn);
+    }
     w = wn;
     wn = wnn;
+    un = unn;
   }
   if (tid == 0) bulk_wait_all();  // this CTA's bulk stores are complete before it leaves
   if (!ok && tid == 0) {  // a wait gave up: let what this CTA armed land before leaving
@@ -614,6 +656,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     track_drain(bar_s, ts);
     track_drain(bar_dp, tdp);
     track_drain(bar_mma2, tm2);
+    track_drain(bar_clc, tclc);
   }
   tc_fence_before();
   __syncthreads();
@@ -649,7 +692,9 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   uint64_t* bar_s = bars + 3;
   uint64_t* bar_dp = bars + 4;
   uint64_t* bar_mma2 = bars + 5;
-  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
+  uint64_t* bar_clc = bars + 6;
+  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // the unit taken over
+  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 10);
 
   const int nh = H / HD;
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -664,9 +709,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     int h, seg0, L, q0, clast, n_kv;
     float* db;
   };
-  auto unit = [&](int u) {
+  auto unit_t = [&](int u, uint32_t t) {
     Unit w;
-    const uint32_t t = tiles[u / nh];
     const int s = int(t >> 16), idx = int(t & 0xFFFFu);
     w.h = u % nh;
     w.seg0 = cu[s];
@@ -677,6 +721,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     w.db = dbias ? dbias + (dbias_segs > 0 ? (int64_t)(s / dbias_segs) * dbias_rstride : 0) : nullptr;
     return w;
   };
+  auto unit = [&](int u) { return unit_t(u, tiles[u / nh]); };
   // the thread's row statistics in unit w: lse * log2e and delta
   auto row_stats = [&](const Unit& w, float& lse2, float& dl) {
     const bool q_ok = w.q0 + r < w.L;
@@ -685,7 +730,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   };
 
   if (tid == 0) {
-    for (int i = 0; i < 6; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < 7; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
     tma_prefetch_desc(&tm_do);
@@ -700,7 +745,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
-  BarTrack tqdo, tkv0, tkv1, ts, tdp, tm2;
+  BarTrack tqdo, tkv0, tkv1, ts, tdp, tm2, tclc;
   // Copies and products are issued by warp 0 as a whole, as in the dK / dV kernel.
   auto issue_kv = [&](const Unit& w, int j, int b) {  // K_j, V_j into pair b
     (b ? tkv1 : tkv0).pend = true;
@@ -734,25 +779,51 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   constexpr uint32_t IDESC_S = umma_idesc_bf16(TB, TB, false, false);
   constexpr uint32_t IDESC_G = umma_idesc_bf16(TB, HD, false, true);
   bool ok = true;
-  int u = blockIdx.x;
-  Unit w = u < n_units ? unit(u) : Unit{};
+  // Units: CTA c walks c, + gridDim.x, ..., or, when the grid has one CTA per unit, the hardware
+  // hands them out: the resident CTA takes over the next one that has not started, two units ahead
+  // of its work.
+  const bool handed = (int)gridDim.x == n_units;
+  int u_next = blockIdx.x;
+  auto take = [&]() {
+    if (!handed) return;
+    tclc.pend = true;
+    __syncwarp();
+    if (elect_one()) clc_request(clc, bar_clc);
+  };
+  auto taken = [&](int& x) {  // the unit taken, or -1
+    if (!handed) {
+      u_next += gridDim.x;
+      x = u_next < n_units ? u_next : -1;
+      return true;
+    }
+    ok = track_wait_all(bar_clc, tclc);
+    if (!ok && tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+    x = ok ? clc_answer(clc) : -1;
+    return ok;
+  };
+  Unit w = unit(blockIdx.x), wn = Unit{};
   float lse2 = 0.f, dl = 0.f;
-  if (u < n_units) row_stats(w, lse2, dl);
+  row_stats(w, lse2, dl);
   RopeRow<HD> rrow;
-  if (warp == 0 && u < n_units) {
+  if (warp == 0) {
     issue_qdo(w);
     issue_kv(w, 0, 0);
     if (w.n_kv > 1) issue_kv(w, 1, 1);
+    take();
   }
-  while (u < n_units && ok) {
+  int un;
+  if (taken(un) && un >= 0) wn = unit(un);
+  while (ok) {
     const int q = w.q0 + r;
     const bool q_ok = q < w.L;
     const int ulim = q_ok ? max(q, w.clast) : -1;  // last own key visible to the row
     // the next unit: its Q / dO load once this unit's last S / dP products have read them,
     // its first key / value tile once buffer pair 0 has had its last use here
-    const int un = u + gridDim.x;
-    const Unit wn = un < n_units ? unit(un) : Unit{};
-    const bool next = un < n_units;
+    const bool next = un >= 0;
+    Unit wnn = Unit{};  // the unit after next, as in the dK / dV kernel
+    int unn = -1;
+    uint32_t tnn = 0;
+    if (next && warp == 0) take();
     // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
     if (!track_wait_all(bar_qdo, tqdo)) {
       if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
@@ -821,6 +892,10 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
       };
       if (open) probs(std::false_type{});
       else probs(std::true_type{});
+      if (j == 0 && next) {
+        if (!taken(unn)) break;
+        if (unn >= 0) tnn = tiles[unn / nh];
+      }
       tc_fence_before();
       if (!track_wait_all(bar_dp, tdp)) {
         if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
@@ -868,6 +943,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
         __syncwarp();
         if (!last) scores(1 - b);
       }
+      // (the unit after next's segment: two dependent loads, while the products run)
+      if (j == 0 && unn >= 0) wnn = unit_t(unn, tnn);
       if (last) {
         if (kh < nreg && q_ok) {  // the query's rotary row, for the epilogue
           const int32_t* gp = kh == 0 ? gpos : gpos2;
@@ -895,11 +972,11 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     {
       uint8_t* stage = sST;
       uint32_t vr[HD / 2];
+      float* v = reinterpret_cast<float*>(vr);
 #pragma unroll
       for (int c = 0; c < HD / 2; c += 32)
         tmem_ld32(t_lane + 256 + kh * (HD / 2) + c, *reinterpret_cast<uint32_t(*)[32]>(vr + c));
       tmem_ld_wait();
-      float* v = reinterpret_cast<float*>(vr);
 #pragma unroll
       for (int c = 0; c < HD / 2; ++c) v[c] = __uint_as_float(vr[c]) * scale;
       if (kh < nreg && q_ok) inverse_rope_row<HD>(v, rrow);  // rotary region kh
@@ -935,8 +1012,10 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     // epilogue and products reuse them
     tc_fence_before();
     __syncthreads();
-    u = un;
+    if (!next) break;
     w = wn;
+    wn = wnn;
+    un = unn;
     lse2 = lse2n;
     dl = dln;
   }
@@ -948,6 +1027,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     track_drain(bar_s, ts);
     track_drain(bar_dp, tdp);
     track_drain(bar_mma2, tm2);
+    track_drain(bar_clc, tclc);
   }
   tc_fence_before();
   __syncthreads();
@@ -959,7 +1039,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
 
 template <int HD>
 int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float* lse, const float* delta,
-                  const int32_t* cu, const uint32_t* tiles, int n_tiles, const float* rope_tab, void* dqkv,
+                  const int32_t* cu, const uint32_t* tiles, int n_tiles, int max_tiles, const float* rope_tab, void* dqkv,
                   const AttnPrefix& pre, const AttnGlm& glm, float* dbias, int* status, cudaStream_t st,
                   int dbias_segs, int64_t dbias_rstride) {
   FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dq_tc_kernel<HD>, BwdCfg<HD>::SMEM));
@@ -979,9 +1059,12 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
   }
   const float scale = 1.f / sqrtf((float)HD);
   const float2* tab = reinterpret_cast<const float2*>(rope_tab);
-  // persistent: one CTA per SM (512 TMEM columns each) walks the (tile, head) units
-  const int n_units = n_tiles * nh;
-  const int grid = n_units < fl_sm_count() ? n_units : fl_sm_count();
+  // One CTA is resident per SM (512 TMEM columns).  Units of different cost (segments of three
+  // tiles and more: a unit walks 1 .. that many) are handed out as CTAs finish: segments of 67 to
+  // 2048 tokens 362 -> 331 us, 4 x 512 106 -> 98, 8 x 1024 422 -> 411; a fixed walk is enough for
+  // even ones and spares them the requests: 40 x 190 tokens 262 against 273 us, 64 x 64 181 / 183.
+  const int n_units = n_tiles * nh, sms = fl_sm_count();
+  const int grid = max_tiles >= 3 || n_units < sms ? n_units : sms;
   if (n_units > 0) {
     FL_CUDA_TRY(fl_launch(attn_bwd_dq_tc_kernel<HD>, dim3(grid), dim3(256), BwdCfg<HD>::SMEM, st, tq, tdo, tpk, tpv,
                           tdq, T, H, cu, tiles, n_units, lse, delta, tab, scale, scale * LOG2E_B, pre.len, (bf16*)dqkv,
@@ -1007,14 +1090,14 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
 }  // namespace
 
 int fl_launch_attn_bwd_tc(int T, int nh, int hd, const void* qkv, const void* dout, const float* lse,
-                          const float* delta, const int32_t* cu, const uint32_t* tiles, int n_tiles,
+                          const float* delta, const int32_t* cu, const uint32_t* tiles, int n_tiles, int max_tiles,
                           const float* rope_tab, void* dqkv, const AttnPrefix& pre, const AttnGlm& glm, float* dbias,
                           int* status, cudaStream_t st, int dbias_segs, int64_t dbias_rstride) {
   if (hd == 128)
-    return launch_bwd_tc<128>(T, nh, qkv, dout, lse, delta, cu, tiles, n_tiles, rope_tab, dqkv, pre, glm, dbias,
+    return launch_bwd_tc<128>(T, nh, qkv, dout, lse, delta, cu, tiles, n_tiles, max_tiles, rope_tab, dqkv, pre, glm, dbias,
                               status, st, dbias_segs, dbias_rstride);
   if (hd == 64)
-    return launch_bwd_tc<64>(T, nh, qkv, dout, lse, delta, cu, tiles, n_tiles, rope_tab, dqkv, pre, glm, dbias,
+    return launch_bwd_tc<64>(T, nh, qkv, dout, lse, delta, cu, tiles, n_tiles, max_tiles, rope_tab, dqkv, pre, glm, dbias,
                              status, st, dbias_segs, dbias_rstride);
   return fl_internal_error(FL_ERR_UNSUPPORTED, "attention: head_dim %d", hd);
 }

@@ -206,6 +206,33 @@ FL_DEV void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "
 // tensor core reading an operand written by threads).
 FL_DEV void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// ------------------------------------------------------------------ cluster launch control
+// A running CTA takes over a CTA of its own grid that has not started: the request completes on
+// `bar` (16 bytes) with its answer in `resp` (16-byte aligned shared memory).  One thread; not
+// after an answer was empty.
+FL_DEV void clc_request(void* resp, uint64_t* bar) {
+  fence_proxy_async_smem();  // the previous answer has been read
+  mbar_arrive_expect_tx(bar, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                   smem_u32(resp)),
+               "r"(smem_u32(bar))
+               : "memory");
+}
+// The blockIdx.x taken over, or -1.
+FL_DEV int clc_answer(const void* resp) {
+  int x;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%1];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "mov.s32 %0, -1;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
+      : "=r"(x)
+      : "r"(smem_u32(resp))
+      : "memory");
+  return x;
+}
+
 // ------------------------------------------------------------------ CTA pairs (cluster of 2)
 // tcgen05 with .cta_group::2: the even CTA of a cluster pair issues MMAs that read both
 // CTAs' shared memory and write both CTAs' TMEM.

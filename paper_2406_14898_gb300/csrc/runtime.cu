@@ -191,7 +191,7 @@ struct fl_server {
 
   // pending step
   bool pending = false;
-  int T = 0, S = 0, K = 0, n_tiles = 0, n_tiles128 = 0;
+  int T = 0, S = 0, K = 0, n_tiles = 0, n_tiles128 = 0, max_tiles = 0;  // max_tiles: of the longest segment
   int Tr = 0, Sr = 0;  // tokens and segments of one replica's group (T and S with one replica)
   std::vector<int32_t> seq_lens;
 
@@ -583,7 +583,7 @@ int block_backward(fl_server* h, int b, const __nv_bfloat16* dy, const float* dy
   // attention backward -> dqkv (w.r.t. the un-rotated q, k); dbqkv += colsum(dqkv)
   prof_begin(h, FL_PROF_ATTN, 3);
   TRY(h, fl_launch_attn_bwd(h->T, c.n_heads, c.head_dim, A.qkv, A.o, A.lse, h->d_o, h->cu, h->tiles, h->n_tiles,
-                            h->n_tiles128, h->delta, h->rope_tab, h->dqkv, h->prefix(b, true), h->glm_args(), st,
+                            h->n_tiles128, h->max_tiles, h->delta, h->rope_tab, h->dqkv, h->prefix(b, true), h->glm_args(), st,
                             train_base ? h->gt(b, FL_T_BQKV) : nullptr, h->status, h->R > 1 ? h->Sr : 0,
                             h->n_params));
   prof_end(h);
@@ -874,6 +874,7 @@ static int forward_impl(fl_server_t h, const void* const client_states[], const 
   h->K = K;
   h->n_tiles = nt;
   h->n_tiles128 = nt128;
+  h->max_tiles = nt128 > 0 ? int(meta.tiles[nt] & 0xFFFFu) + 1 : 0;
   h->seq_lens.assign(seq_lens, seq_lens + K);
 
   prof_begin(h, FL_PROF_OTHER);
