@@ -82,7 +82,9 @@ struct EpiCfg {
   static constexpr int WARPS = FAM == FAM_ADAMW ? AdamRing::WARPS : FAM == FAM_ADAMW_LONG || BN == 64 ? 4 : 8;
   static constexpr int THREADS = 64 + 32 * WARPS;
   static constexpr int BYTES = FAM == FAM_ADAMW ? AdamRing::BYTES : WARPS * 32 * 64 * 4;
-  static constexpr int BARS = FAM == FAM_ADAMW ? WARPS * AdamRing::SLOTS : 0;
+  // barriers of its own: the AdamW ring's, or the column sums' (written and read, per column half)
+  static constexpr int BARS = FAM == FAM_ADAMW ? WARPS * AdamRing::SLOTS : FAM == FAM_GELU ? 4 : 0;
+  static constexpr int bar_count(int i) { return FAM == FAM_GELU && i % 2 == 0 ? 4 : 1; }
 };
 // Depth of the operand ring for stages of `bytes`: what fits beside the epilogue's shared
 // memory, six stages at most (deeper gains nothing).
@@ -392,7 +394,7 @@ FL_DEV void epi_apply(const EpiRegs<FAM, RB>& q, const EpiCols& c, const Epi& e,
 // position for this warp, `release` frees accumulator `acc` once the warp has read it.
 template <int FAM, int BN, typename Place, typename Release>
 FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int warp, int lane, int t0, int step,
-                          int num_tiles, uint64_t* acc_full, int* status, Place place, Release release) {
+                          int num_tiles, uint64_t* acc_full, uint64_t* cs_bars, int* status, Place place, Release release) {
   constexpr int RB = EpiBatch<FAM>::RB, DEPTH = EpiBatch<FAM>::DEPTH;
   constexpr int HALVES = EpiCfg<FAM, BN>::WARPS / 4;    // warps per lane quarter
   constexpr int WCH = BN / (64 * HALVES);           // chunks per warp and tile
@@ -413,6 +415,7 @@ FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int wa
 #pragma unroll
   for (int s = 0; s < DEPTH - 1; ++s) epi_load<FAM, RB>(q[s], e, t, n, s * RB, h);
   int local = 0;
+  uint32_t cs_par = 0;  // parity of the column sums' barriers
   for (int tile = t0; tile < num_tiles; tile += step, ++local) {
     const int acc = local & 1;
     if (!mbar_wait(&acc_full[acc], (local >> 1) & 1)) {
@@ -463,10 +466,39 @@ FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int wa
           epi_apply<FAM, RB>(q[s], c, e, t, stage, n, (b0 + s) * RB, h, cs);
         }
       }
-      if (FAM == FAM_GELU && e.colsum != nullptr) {  // the two half-warps hold the same columns for rows of either parity
+      if (FAM == FAM_GELU && e.colsum != nullptr) {
+        // the two half-warps hold the same columns for rows of either parity; the four warps of the
+        // column half meet in their staging and one adds their sum, so that calls of up to two row
+        // blocks sum a bias gradient in one order
 #pragma unroll
         for (int k = 0; k < 4; ++k) cs[k] += __shfl_xor_sync(0xffffffffu, cs[k], 16);
-        if (h == 0 && t.rows > 0) red_add_v4(e.colsum + prob_off(e.o_bias, t.r) + n, cs[0], cs[1], cs[2], cs[3]);
+        __syncwarp();
+        if (h == 0) *reinterpret_cast<float4*>(stage + cl4) = make_float4(cs[0], cs[1], cs[2], cs[3]);
+        __syncwarp();
+        const int wi = (warp - 2) & 3;
+        uint64_t* written = cs_bars + 2 * ((warp - 2) >> 2);
+        if (lane == 0) mbar_arrive(written);
+        if (wi == 0) {
+          if (!mbar_wait(written, cs_par)) {
+            report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+            return;
+          }
+          if (h == 0) {
+            float4 t4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float4 q4 = *reinterpret_cast<const float4*>(stage + i * 32 * 64 + cl4);
+              t4 = make_float4(t4.x + q4.x, t4.y + q4.y, t4.z + q4.z, t4.w + q4.w);
+            }
+            red_add_v4(e.colsum + prob_off(e.o_bias, t.r) + n, t4.x, t4.y, t4.z, t4.w);
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(written + 1);
+        } else if (!mbar_wait(written + 1, cs_par)) {
+          report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+          return;
+        }
+        cs_par ^= 1;
       }
       __syncwarp();  // the chunk has been read
       c = cn;
@@ -631,8 +663,8 @@ __global__ void __launch_bounds__(EpiCfg<FAM, BN>::THREADS, 1)
   uint64_t* acc_full = bars + 2 * STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
-  uint64_t* ring_full = drain + 1;  // the AdamW ring's
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ring_full + EpiCfg<FAM, BN>::BARS);
+  uint64_t* epi_bars = drain + 1;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(epi_bars + EpiCfg<FAM, BN>::BARS);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -651,7 +683,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM, BN>::THREADS, 1)
       mbar_init(&acc_empty[a], EpiCfg<FAM, BN>::WARPS);
     }
     mbar_init(drain, 1);
-    for (int i = 0; i < EpiCfg<FAM, BN>::BARS; ++i) mbar_init(&ring_full[i], 1);
+    for (int i = 0; i < EpiCfg<FAM, BN>::BARS; ++i) mbar_init(&epi_bars[i], EpiCfg<FAM, BN>::bar_count(i));
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -788,11 +820,11 @@ __global__ void __launch_bounds__(EpiCfg<FAM, BN>::THREADS, 1)
       if (lane == 0) mbar_arrive(&acc_empty[acc]);
     };
     if constexpr (FAM == FAM_ADAMW)
-      adamw_epilogue<BN>(epi, maps, epi_smem, ring_full, tmem_base, warp, lane, blockIdx.x, gridDim.x, num_tiles, acc_full,
+      adamw_epilogue<BN>(epi, maps, epi_smem, epi_bars, tmem_base, warp, lane, blockIdx.x, gridDim.x, num_tiles, acc_full,
                          status, place, release);
     else
       epilogue_loop<FAM, BN>(epi, reinterpret_cast<float*>(epi_smem) + (warp - 2) * 32 * 64, tmem_base, warp, lane,
-                             blockIdx.x, gridDim.x, num_tiles, acc_full, status, place, release);
+                             blockIdx.x, gridDim.x, num_tiles, acc_full, epi_bars, status, place, release);
   }
 
   tc_fence_before();
@@ -844,8 +876,8 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
   uint64_t* acc_full = bars + 2 * STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* drain = acc_empty + 2;
-  uint64_t* ring_full = drain + 1;  // the AdamW ring's
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ring_full + EpiCfg<FAM, PBN>::BARS);
+  uint64_t* epi_bars = drain + 1;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(epi_bars + EpiCfg<FAM, PBN>::BARS);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -867,7 +899,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
       mbar_init(&acc_empty[a], 2 * EpiCfg<FAM, PBN>::WARPS);  // the epilogue warps of both CTAs
     }
     mbar_init(drain, 1);
-    for (int i = 0; i < EpiCfg<FAM, PBN>::BARS; ++i) mbar_init(&ring_full[i], 1);
+    for (int i = 0; i < EpiCfg<FAM, PBN>::BARS; ++i) mbar_init(&epi_bars[i], EpiCfg<FAM, PBN>::bar_count(i));
     fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -1006,11 +1038,11 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
       if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8u * acc);
     };
     if constexpr (FAM == FAM_ADAMW)
-      adamw_epilogue<PBN>(epi, maps, epi_smem, ring_full, tmem_base, warp, lane, pair, n_pairs, num_tiles, acc_full, status,
+      adamw_epilogue<PBN>(epi, maps, epi_smem, epi_bars, tmem_base, warp, lane, pair, n_pairs, num_tiles, acc_full, status,
                           place, release);
     else
       epilogue_loop<FAM, PBN>(epi, reinterpret_cast<float*>(epi_smem) + (warp - 2) * 32 * 64, tmem_base, warp, lane, pair,
-                              n_pairs, num_tiles, acc_full, status, place, release);
+                              n_pairs, num_tiles, acc_full, epi_bars, status, place, release);
   }
 
   tc_fence_before();
