@@ -19,6 +19,10 @@ enum CopyMode {
 struct CopyTable {
   int n;
   int mode;
+  // filled with zeros by the same launch: zero[0 .. n_zero), zero_n floats each (a multiple of 4)
+  int n_zero;
+  int64_t zero_n;
+  float* zero[4];
   void* packed_bf16;
   float* packed_f32;
   void* client[FL_MAX_COPY];
@@ -42,7 +46,14 @@ struct MetaArgs {
   int32_t mpos[FL_MAX_SEGS];
 };
 
-int fl_launch_copy_clients(const CopyTable& tab, cudaStream_t st);
+// `meta` (or null): the call's packing metadata, written by the same launch (MetaArgs).
+struct MetaOut {
+  int32_t *cu, *pos;
+  uint32_t* tiles;
+  int32_t *pos2, *ctx;
+};
+int fl_launch_copy_clients(const CopyTable& tab, cudaStream_t st, const MetaArgs* meta = nullptr,
+                           const MetaOut* out = nullptr);
 
 // Replicas averaged together: fp32 master arenas and bf16 copies, same length.
 constexpr int FL_MAX_REPLICAS = 64;
@@ -54,11 +65,9 @@ struct ReplicaTable {
 int fl_launch_average(const ReplicaTable& t, int64_t n, cudaStream_t st);
 // w[i] *= 1/n_replicas (the factor fl_launch_average applies) and wb[i] = bf16(w[i]).
 int fl_launch_mean_finish(int64_t n, int n_replicas, float* w, void* wb, cudaStream_t st);
-// Writes cu_seqlens, the tile list, per-token positions (and, when pos2 != NULL, the GLM
-// block positions and, when ctx != NULL, the per-segment context lengths; both zero
+// A MetaArgs launch writes cu_seqlens, the tile list, per-token positions (and, when pos2 != NULL,
+// the GLM block positions and, when ctx != NULL, the per-segment context lengths; both zero
 // without glm).
-int fl_launch_meta(const MetaArgs& a, int32_t* cu, int32_t* pos, uint32_t* tiles, int32_t* pos2, int32_t* ctx,
-                   cudaStream_t st);
 int fl_launch_normal_init(int64_t n, uint64_t key, double mean, double std_, float* out, cudaStream_t st);
 int fl_launch_fill(int64_t n, float v, float* out, cudaStream_t st);
 int fl_launch_adamw(int64_t n, float* w, float* g, float* m, float* v, void* w_bf16, float lr, float beta1,
@@ -85,7 +94,7 @@ struct AttnGlm {
   const int32_t* pos2 = nullptr;  // [T] block position (inverse rotary of dims [hd/2, hd))
 };
 
-// Attention on a device tile list (built by fl_launch_meta): the 64-row list (n_tiles
+// Attention on a device tile list (written with the packing metadata): the 64-row list (n_tiles
 // entries) followed by the 128-row one (n_tiles128) that the tcgen05 kernels walk.
 // head_dim 64 or 128; `status` (device int or null) receives a code if a bounded wait
 // inside a kernel gave up.

@@ -492,54 +492,80 @@ __global__ void f32_to_bf16_kernel(int64_t n, const float* __restrict__ src, __n
 }
 
 // ------------------------------------------------------------------ pack / unpack
-// blockIdx.y = table entry; each entry moves n8 groups of 8 elements between a client
-// buffer (bf16) and the packed buffer (bf16 or fp32).
-__global__ void copy_clients_kernel(CopyTable tab) {
-  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
-  pdl_trigger();
-  const int e = blockIdx.y;
-  if (e >= tab.n) return;
-  const int64_t n8 = tab.n8[e], off = tab.off8[e];
-  uint4* client = reinterpret_cast<uint4*>(tab.client[e]);
-  uint4* pb = tab.packed_bf16 ? reinterpret_cast<uint4*>(tab.packed_bf16) + off : nullptr;
-  float4* pf = tab.packed_f32 ? reinterpret_cast<float4*>(tab.packed_f32) + 2 * off : nullptr;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
-    switch (tab.mode) {
-      case COPY_GATHER_BF16: pb[i] = client[i]; break;
-      case COPY_SCATTER_BF16: client[i] = pb[i]; break;
-      case COPY_GATHER_F32: {
-        const uint4 w = client[i];
-        if (pb) pb[i] = w;
-        float f[8];
-        unpack8(w, f);
-        pf[2 * i] = make_float4(f[0], f[1], f[2], f[3]);
-        pf[2 * i + 1] = make_float4(f[4], f[5], f[6], f[7]);
-        break;
-      }
-      default: {  // COPY_SCATTER_F32
-        const float4 a = pf[2 * i], b = pf[2 * i + 1];
-        const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        client[i] = pack8(f);
-        break;
-      }
+// One group of 8 elements between a client buffer (bf16) and the packed buffer (bf16 or fp32):
+// MODE's loads into registers, then its stores.
+template <int MODE>
+struct CopyReg {
+  uint4 w;
+  float4 a, b;
+  FL_DEV void load(const CopyTable& t, const uint4* client, int64_t off, int64_t i) {
+    if constexpr (MODE == COPY_GATHER_BF16 || MODE == COPY_GATHER_F32) w = client[i];
+    else if constexpr (MODE == COPY_SCATTER_BF16) w = reinterpret_cast<const uint4*>(t.packed_bf16)[off + i];
+    else {
+      a = reinterpret_cast<const float4*>(t.packed_f32)[2 * (off + i)];
+      b = reinterpret_cast<const float4*>(t.packed_f32)[2 * (off + i) + 1];
     }
   }
+  FL_DEV void store(const CopyTable& t, uint4* client, int64_t off, int64_t i) {
+    if constexpr (MODE == COPY_GATHER_BF16) reinterpret_cast<uint4*>(t.packed_bf16)[off + i] = w;
+    else if constexpr (MODE == COPY_SCATTER_BF16) client[i] = w;
+    else if constexpr (MODE == COPY_GATHER_F32) {
+      if (t.packed_bf16) reinterpret_cast<uint4*>(t.packed_bf16)[off + i] = w;
+      float f[8];
+      unpack8(w, f);
+      float4* pf = reinterpret_cast<float4*>(t.packed_f32) + 2 * (off + i);
+      pf[0] = make_float4(f[0], f[1], f[2], f[3]);
+      pf[1] = make_float4(f[4], f[5], f[6], f[7]);
+    } else {
+      const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+      client[i] = pack8(f);
+    }
+  }
+};
+
+// blockIdx.y = table entry, then one row of blocks for the zeros.  A thread has four groups in
+// flight when it scatters (3072 x 4096 fp32 -> bf16 15.6 -> 11.5 us, bf16 13.5 -> 8.3 on twice the
+// CTAs) and one when it gathers, which its fp32 stores bound (15.6 us against 18 with four).
+constexpr bool copy_scatters(int mode) { return mode == COPY_SCATTER_BF16 || mode == COPY_SCATTER_F32; }
+template <int MODE>
+FL_DEV void copy_clients(const CopyTable& tab) {
+  constexpr int COPY_NV = copy_scatters(MODE) ? 4 : 1;
+  const int e = blockIdx.y;
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+  if (e < tab.n) {
+    const int64_t n8 = tab.n8[e], off = tab.off8[e];
+    uint4* client = reinterpret_cast<uint4*>(tab.client[e]);
+    for (int64_t i0 = tid; i0 < n8; i0 += COPY_NV * nth) {
+      CopyReg<MODE> r[COPY_NV];
+#pragma unroll
+      for (int k = 0; k < COPY_NV; ++k)
+        if (i0 + k * nth < n8) r[k].load(tab, client, off, i0 + k * nth);
+#pragma unroll
+      for (int k = 0; k < COPY_NV; ++k)
+        if (i0 + k * nth < n8) r[k].store(tab, client, off, i0 + k * nth);
+    }
+  } else if (e == tab.n) {
+    for (int z = 0; z < tab.n_zero; ++z)
+      for (int64_t i = tid; i < tab.zero_n / 4; i += nth)
+        reinterpret_cast<float4*>(tab.zero[z])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+template <int MODE>
+__global__ void __launch_bounds__(256) copy_clients_kernel(CopyTable tab) {
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
+  copy_clients<MODE>(tab);
 }
 
 // ------------------------------------------------------------------ packing metadata
 // GLM positions of token i of a segment with context length c and mask position mp:
 // (i, 0) in the context (or in a plain causal segment, c = 0), (mp, i - c + 1) in the span.
-__global__ void meta_kernel(MetaArgs a, int32_t* __restrict__ cu, int32_t* __restrict__ pos,
-                            uint32_t* __restrict__ tiles, int32_t* __restrict__ pos2, int32_t* __restrict__ ctx) {
-  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
-  pdl_trigger();
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+FL_DEV void write_meta(const MetaArgs& a, const MetaOut& o, int64_t tid, int64_t nth) {
   const int T = a.cu[a.S];
-  for (int64_t i = tid; i <= a.S; i += nth) cu[i] = a.cu[i];
-  for (int64_t i = tid; i < a.n_tiles + a.n_tiles128; i += nth) tiles[i] = a.tiles[i];
-  if (ctx)
-    for (int64_t i = tid; i < a.S; i += nth) ctx[i] = a.glm ? a.ctx[i] : 0;
+  for (int64_t i = tid; i <= a.S; i += nth) o.cu[i] = a.cu[i];
+  for (int64_t i = tid; i < a.n_tiles + a.n_tiles128; i += nth) o.tiles[i] = a.tiles[i];
+  if (o.ctx)
+    for (int64_t i = tid; i < a.S; i += nth) o.ctx[i] = a.glm ? a.ctx[i] : 0;
   for (int64_t t = tid; t < T; t += nth) {
     int lo = 0, hi = a.S - 1;  // last segment with cu[s] <= t
     while (lo < hi) {
@@ -553,9 +579,18 @@ __global__ void meta_kernel(MetaArgs a, int32_t* __restrict__ cu, int32_t* __res
       p1 = a.mpos[lo];
       p2 = i - a.ctx[lo] + 1;
     }
-    pos[t] = p1;
-    if (pos2) pos2[t] = p2;
+    o.pos[t] = p1;
+    if (o.pos2) o.pos2[t] = p2;
   }
+}
+// The forward's first launch: the clients' states gathered (blockIdx.y < tab.n) and the call's
+// metadata written (the last row of blocks).
+__global__ void __launch_bounds__(256) gather_meta_kernel(const __grid_constant__ CopyTable tab,
+                                                          const __grid_constant__ MetaArgs a, MetaOut o) {
+  pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
+  pdl_trigger();
+  if (blockIdx.y + 1 < gridDim.y) copy_clients<COPY_GATHER_F32>(tab);
+  else write_meta(a, o, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // ------------------------------------------------------------------ seeded init
@@ -709,23 +744,25 @@ int fl_launch_adamw(int64_t n, float* w, float* g, float* m, float* v, void* w_b
 
 // ====================================================================== internal launchers
 
-int fl_launch_copy_clients(const CopyTable& tab, cudaStream_t st) {
+int fl_launch_copy_clients(const CopyTable& tab, cudaStream_t st, const MetaArgs* meta, const MetaOut* out) {
   if (tab.n <= 0) return FL_OK;
   int64_t maxn = 0;
   for (int e = 0; e < tab.n; ++e) maxn = tab.n8[e] > maxn ? tab.n8[e] : maxn;
   int gx = (int)((maxn + 255) / 256);
-  const int cap = (2 * sm_count() + tab.n - 1) / tab.n + 1;
+  const int cap = ((copy_scatters(tab.mode) ? 4 : 2) * sm_count() + tab.n - 1) / tab.n + 1;
   if (gx > cap) gx = cap;
   if (gx < 1) gx = 1;
-  FL_CUDA_TRY(fl_launch(copy_clients_kernel, dim3(gx, tab.n), dim3(256), 0, st, tab));
-  return FL_OK;
-}
-
-int fl_launch_meta(const MetaArgs& a, int32_t* cu, int32_t* pos, uint32_t* tiles, int32_t* pos2, int32_t* ctx,
-                   cudaStream_t st) {
-  const int T = a.cu[a.S];
-  FL_CUDA_TRY(fl_launch(meta_kernel, dim3(grid_for(T > a.n_tiles ? T : a.n_tiles)), dim3(256), 0, st, a, cu, pos,
-                        tiles, pos2, ctx));
+  if (meta) {  // CopyTable and MetaArgs together stay below the 32 KB of kernel parameters
+    FL_CUDA_TRY(fl_launch(gather_meta_kernel, dim3(gx, tab.n + 1), dim3(256), 0, st, tab, *meta, *out));
+    return FL_OK;
+  }
+  const dim3 grid(gx, tab.n + (tab.n_zero > 0 ? 1 : 0));
+  switch (tab.mode) {
+    case COPY_GATHER_BF16: FL_CUDA_TRY(fl_launch(copy_clients_kernel<COPY_GATHER_BF16>, grid, dim3(256), 0, st, tab)); break;
+    case COPY_SCATTER_BF16: FL_CUDA_TRY(fl_launch(copy_clients_kernel<COPY_SCATTER_BF16>, grid, dim3(256), 0, st, tab)); break;
+    case COPY_GATHER_F32: FL_CUDA_TRY(fl_launch(copy_clients_kernel<COPY_GATHER_F32>, grid, dim3(256), 0, st, tab)); break;
+    default: FL_CUDA_TRY(fl_launch(copy_clients_kernel<COPY_SCATTER_F32>, grid, dim3(256), 0, st, tab)); break;
+  }
   return FL_OK;
 }
 
@@ -799,6 +836,7 @@ extern "C" int fl_k_pack_clients(int32_t K, void* const* clients_host, const int
   int64_t off = 0;
   for (int k0 = 0; k0 < K; k0 += FL_MAX_COPY) {
     CopyTable tab;
+    tab.n_zero = 0;
     tab.n = (K - k0) < FL_MAX_COPY ? (K - k0) : FL_MAX_COPY;
     tab.mode = scatter ? COPY_SCATTER_BF16 : COPY_GATHER_BF16;
     tab.packed_bf16 = packed;

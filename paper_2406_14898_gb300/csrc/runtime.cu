@@ -624,8 +624,11 @@ int block_backward(fl_server* h, int b, const __nv_bfloat16* dy, const float* dy
   return FL_OK;
 }
 
-// Moves the K client tensors to / from the packed buffers (mode: CopyMode).
-int copy_clients(fl_server* h, const void* const* ptrs, int mode, __nv_bfloat16* packed_bf16, float* packed_f32) {
+// Moves the K client tensors to / from the packed buffers (mode: CopyMode).  The first launch also
+// writes `meta` (the forward's gather), or clears the bias, LayerNorm and prefix gradients of every
+// replica (clear_vecs, the backward's gather).
+int copy_clients(fl_server* h, const void* const* ptrs, int mode, __nv_bfloat16* packed_bf16, float* packed_f32,
+                 const MetaArgs* meta = nullptr, bool clear_vecs = false) {
   const int64_t row8 = (int64_t)h->cfg.client_batch * h->cfg.hidden / 8;  // 8-element groups per token
   int64_t off = 0;
   for (int k0 = 0; k0 < h->K; k0 += FL_MAX_COPY) {
@@ -642,8 +645,14 @@ int copy_clients(fl_server* h, const void* const* ptrs, int mode, __nv_bfloat16*
       tab.n8[e] = row8 * h->seq_lens[k];
       off += tab.n8[e];
     }
+    const MetaOut out = {h->cu, h->pos, h->tiles, h->pos2, h->ctx};
+    if (clear_vecs && k0 == 0) {  // their contiguous region, a multiple of 16 floats
+      tab.n_zero = h->R;
+      tab.zero_n = h->n_params - h->vec_base;
+      for (int r = 0; r < h->R; ++r) tab.zero[r] = h->g + r * h->n_params + h->vec_base;
+    }
     prof_begin(h, FL_PROF_OTHER);
-    int rc = fl_launch_copy_clients(tab, h->stream);
+    int rc = fl_launch_copy_clients(tab, h->stream, k0 == 0 ? meta : nullptr, &out);
     prof_end(h);
     if (rc) return fwd_err(h, rc);
   }
@@ -877,12 +886,9 @@ static int forward_impl(fl_server_t h, const void* const client_states[], const 
   h->max_tiles = nt128 > 0 ? int(meta.tiles[nt] & 0xFFFFu) + 1 : 0;
   h->seq_lens.assign(seq_lens, seq_lens + K);
 
-  prof_begin(h, FL_PROF_OTHER);
   h->glm = meta.glm;
-  int rc = fl_launch_meta(meta, h->cu, h->pos, h->tiles, h->pos2, h->ctx, h->stream);
-  prof_end(h);
-  if (rc) return fwd_err(h, rc);
-  if ((rc = copy_clients(h, client_states, COPY_GATHER_F32, nullptr, h->xs[0]))) return rc;
+  int rc = copy_clients(h, client_states, COPY_GATHER_F32, nullptr, h->xs[0], &meta);
+  if (rc) return rc;
   for (int blk = 0; blk < c.n_blocks; ++blk)
     if ((rc = block_forward(h, blk))) return rc;
   if ((rc = copy_clients(h, (const void* const*)out_states, COPY_SCATTER_F32, nullptr, h->xs[c.n_blocks]))) return rc;
@@ -912,16 +918,9 @@ static int backward_impl(fl_server_t h, const void* const grad_out[], void* cons
   if (int rc = check_ptrs(h, grad_out, h->K, "grad_out")) return rc;
   if (int rc = check_ptrs(h, (const void* const*)grad_in, h->K, "grad_in")) return rc;
   int rc;
-  if (h->grads_zero) {
-    // bias and LayerNorm gradients accumulate (+=); one memset of their contiguous region
-    // (per replica)
-    for (int r = 0; r < h->R; ++r) {
-      const cudaError_t e = cudaMemsetAsync(h->g + r * h->n_params + h->vec_base, 0,
-                                            (h->n_params - h->vec_base) * sizeof(float), h->stream);
-      if (e != cudaSuccess) return fwd_err(h, fl_internal_cuda_error(e, "cudaMemsetAsync", __FILE__, __LINE__));
-    }
-  }
-  if ((rc = copy_clients(h, grad_out, COPY_GATHER_F32, h->dy, h->dyf))) return rc;
+  // bias and LayerNorm gradients accumulate (+=): while every gradient is zero by definition they
+  // are cleared here
+  if ((rc = copy_clients(h, grad_out, COPY_GATHER_F32, h->dy, h->dyf, nullptr, h->grads_zero))) return rc;
   __nv_bfloat16* cur = h->dy;
   __nv_bfloat16* nxt = h->dx;
   float* curf = h->dyf;
