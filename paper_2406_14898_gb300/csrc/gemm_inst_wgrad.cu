@@ -3,5 +3,5 @@
 
 namespace fl_gemm {
 FL_GEMM_INSTANTIATE_PAIR(, true, true)
-FL_GEMM_INSTANTIATE_LONG()
+FL_GEMM_INSTANTIATE_WGRAD()
 }  // namespace fl_gemm

@@ -9,7 +9,7 @@ namespace fl_gemm {
 FL_GEMM_INSTANTIATE_PAIR(extern, false, false)
 FL_GEMM_INSTANTIATE_PAIR(extern, false, true)
 FL_GEMM_INSTANTIATE_PAIR(extern, true, true)
-FL_GEMM_INSTANTIATE_LONG(extern)
+FL_GEMM_INSTANTIATE_WGRAD(extern)
 FL_GEMM_INSTANTIATE_SINGLE(extern, false, false)
 FL_GEMM_INSTANTIATE_SINGLE(extern, false, true)
 FL_GEMM_INSTANTIATE_SINGLE(extern, true, true)
@@ -19,6 +19,25 @@ FL_GEMM_INSTANTIATE_SINGLE(extern, true, true)
 // them.  Measured, two 4096 x 16384 weights per launch, ring / registers: 730 / 790 us at K =
 // 2048, 832 / 807 at 3072, 1038 / 878 at 4096, 1381 / 1156 at 6144, 1693 / 1450 at 8192.
 constexpr int ADAMW_LONG_K = 3072;
+
+// fp32 weight gradients on CTA pairs whose epilogue moves by TMA (FAM_F32): added ones always,
+// stored ones below K = 1024.  Measured, two 4096 x 16384 gradients per launch, registers / ring:
+// added 230 / 191 us at K = 77, 236 / 198 at 512, 244 / 220 at 1024, 330 / 327 at 2048; stored 102 /
+// 97, 118 / 122, 181 / 186 and 309 / 306.
+constexpr int F32_SHORT_K = 1024;
+bool f32_ring(const fl_gemm_args* a) {
+  return a->a_mn_major && !a->bias &&
+         (a->epilogue == FL_EPI_ACCUM_F32 || (a->epilogue == FL_EPI_STORE_F32 && a->K < F32_SHORT_K));
+}
+// A short contraction's gradients are bound by their output: past what L2 holds the pair tile
+// with the ring is the fastest whatever pick_shape estimates, two 4096 x 16384 (537 MB) added 225 ->
+// 191 us at K = 77, 230 -> 198 at 512, stored 104 -> 97, 155 -> 122; 12288 x 4096 (201 MB) added 91 ->
+// 81, 95 -> 86.  4096 x 4096 (67 MB, kept in L2) added takes 30 us on narrow tiles, 36 on these.
+constexpr double F32_RING_MIN_BYTES = 128.0 * (1 << 20);
+bool f32_ring_tile(const fl_gemm_args* a, int batch, int pairs) {
+  return pairs > 0 && a->N % 256 == 0 && a->K < F32_SHORT_K && f32_ring(a) &&
+         4.0 * batch * a->M * a->N > F32_RING_MIN_BYTES;
+}
 
 // Tile shapes: FL_TILE_* - 1, and two narrow ones that only the library picks.
 enum { SHAPE_128 = 0, SHAPE_256 = 1, SHAPE_PAIR256 = 2, SHAPE_64 = 3, SHAPE_PAIR128 = 4 };
@@ -51,6 +70,8 @@ int dispatch_fam(int fam, int shape, bool amn, bool bmn, const fl_gemm_args* a, 
                  int* status, cudaStream_t st) {
   if (fam == FAM_ADAMW && shape == SHAPE_PAIR256 && amn && a->K >= ADAMW_LONG_K)
     return launch_pair<256, true, true, FAM_ADAMW_LONG>(a, pr, e, status, st);
+  if (fam == FAM_PLAIN && shape == SHAPE_PAIR256 && f32_ring(a))
+    return launch_pair<256, true, true, FAM_F32>(a, pr, e, status, st);
   if (!amn && !bmn) return dispatch_layout<false, false>(fam, shape, a, pr, e, status, st);
   if (!amn && bmn) return dispatch_layout<false, true>(fam, shape, a, pr, e, status, st);
   return dispatch_layout<true, true>(fam, shape, a, pr, e, status, st);
@@ -225,7 +246,8 @@ int run(const fl_gemm_args* a, const Problems& pr, const Epi& e, int* status, cu
   if (a->tile == FL_TILE_256x256_PAIR && pair_slots_for<256>(fam, amn, bmn) <= 0)
     return fl_internal_error(FL_ERR_UNSUPPORTED, "gemm: this device cannot hold the CTA-pair kernel");
   if (a->tile != FL_TILE_AUTO) return dispatch_fam(fam, a->tile - 1, amn, bmn, a, pr, e, status, st);
-  const int shape = pick_shape(a, batch, fam, pair_slots_for<256>(fam, amn, bmn));
+  const int pairs = pair_slots_for<256>(fam, amn, bmn);
+  const int shape = f32_ring_tile(a, batch, pairs) ? SHAPE_PAIR256 : pick_shape(a, batch, fam, pairs);
   return dispatch_fam(fam, shape, amn, bmn, a, pr, e, status, st);
 }
 

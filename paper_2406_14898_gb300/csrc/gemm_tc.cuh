@@ -46,7 +46,7 @@ constexpr double L2_GROUP_BUDGET_SHORT_K = 32.0 * (1 << 20);
 
 // Epilogue families: each kernel instantiation carries only its family's code, which keeps
 // the kernel small enough for the instruction cache (the MMA-issuing warp shares it).
-enum { FAM_PLAIN = 0, FAM_GELU = 1, FAM_RESID = 2, FAM_ROPE = 3, FAM_ADAMW = 4, FAM_ADAMW_LONG = 5 };
+enum { FAM_PLAIN = 0, FAM_GELU = 1, FAM_RESID = 2, FAM_ROPE = 3, FAM_ADAMW = 4, FAM_ADAMW_LONG = 5, FAM_F32 = 6 };
 __host__ __device__ constexpr int family_of(int mode) {
   return (mode == FL_EPI_BIAS_GELU || mode == FL_EPI_GELU_BWD) ? FAM_GELU
          : (mode == FL_EPI_BIAS_RESID || mode == FL_EPI_RESID) ? FAM_RESID
@@ -75,15 +75,29 @@ struct AdamRing {
   static constexpr int BYTES = WARPS * SLOTS * SLOT;
 };
 
+// The fp32 gradients' epilogue (stored, or added to what is there) the same way, one tensor, chunks of
+// whole 128-byte rows (128-byte swizzle).
+struct F32Ring {
+  static constexpr int CC = 32;
+  static constexpr int SLOTS = 4;
+  static constexpr int WARPS = 4;
+  static constexpr int SLOT = 32 * CC * 4;
+  static constexpr int BYTES = WARPS * SLOTS * SLOT;
+};
+
 // Epilogue warps of a family at tile width BN (64 columns give eight warps nothing to share)
 // and the shared memory they work in: the AdamW ring, or one 32x64 fp32 chunk per warp.
 template <int FAM, int BN>
 struct EpiCfg {
-  static constexpr int WARPS = FAM == FAM_ADAMW ? AdamRing::WARPS : FAM == FAM_ADAMW_LONG || BN == 64 ? 4 : 8;
+  static constexpr int WARPS = FAM == FAM_ADAMW  ? AdamRing::WARPS
+                               : FAM == FAM_F32 ? F32Ring::WARPS
+                               : FAM == FAM_ADAMW_LONG || BN == 64 ? 4 : 8;
   static constexpr int THREADS = 64 + 32 * WARPS;
-  static constexpr int BYTES = FAM == FAM_ADAMW ? AdamRing::BYTES : WARPS * 32 * 64 * 4;
-  // barriers of its own: the AdamW ring's, or the column sums' (written and read, per column half)
-  static constexpr int BARS = FAM == FAM_ADAMW ? WARPS * AdamRing::SLOTS : FAM == FAM_GELU ? 4 : 0;
+  static constexpr int BYTES = FAM == FAM_ADAMW ? AdamRing::BYTES : FAM == FAM_F32 ? F32Ring::BYTES : WARPS * 32 * 64 * 4;
+  // barriers of its own: the rings', or the column sums' (written and read, per column half)
+  static constexpr int BARS = FAM == FAM_ADAMW  ? WARPS * AdamRing::SLOTS
+                              : FAM == FAM_F32  ? WARPS * F32Ring::SLOTS
+                              : FAM == FAM_GELU ? 4 : 0;
   static constexpr int bar_count(int i) { return FAM == FAM_GELU && i % 2 == 0 ? 4 : 1; }
 };
 // Depth of the operand ring for stages of `bytes`: what fits beside the epilogue's shared
@@ -154,6 +168,12 @@ template <int FAM>
 struct GemmMaps {
   CUtensorMap a[FL_GEMM_MAX_BATCH];
   CUtensorMap b[FL_GEMM_MAX_BATCH];
+};
+template <>
+struct GemmMaps<FAM_F32> {
+  CUtensorMap a[FL_GEMM_MAX_BATCH];
+  CUtensorMap b[FL_GEMM_MAX_BATCH];
+  CUtensorMap w[FL_GEMM_MAX_BATCH];
 };
 template <>
 struct GemmMaps<FAM_ADAMW> {
@@ -597,6 +617,88 @@ FL_DEV void adamw_epilogue(const Epi& e, const Maps& maps, uint8_t* ring, uint64
   }
 }
 
+// D = acc or D += acc in fp32, see adamw_epilogue: bound by HBM while the contraction is short.  Two
+// 4096 x 16384 gradients at 77 tokens: added 191 us, 5.6 TB/s (230 from registers on eight warps
+// of the same tile), stored 97 us, 5.5 TB/s (102).  64 KB of ring leave five operand stages.
+template <int BN, typename Maps, typename Place, typename Release>
+FL_DEV void f32_epilogue(const Epi& e, const Maps& maps, uint8_t* ring, uint64_t* ring_full, uint32_t tmem_base,
+                         int warp, int lane, int t0, int step, int num_tiles, uint64_t* acc_full, int* status,
+                         Place place, Release release) {
+  using R = F32Ring;
+  constexpr int CC = R::CC, S = R::SLOTS, CPT = BN / CC;
+  uint8_t* slots = ring + (warp - 2) * S * R::SLOT;
+  uint64_t* full = ring_full + (warp - 2) * S;
+  const bool add = e.mode == FL_EPI_ACCUM_F32;
+  const int total = t0 < num_tiles ? ((num_tiles - t0 + step - 1) / step) * CPT : 0;
+  const uint32_t t_row = tmem_base + (uint32_t((warp & 3) * 32) << 16);
+  TilePos tl, t;  // the tile being loaded (lane 0), the tile at work
+  auto issue = [&](int k) {
+    if (k % CPT == 0) place(t0 + (k / CPT) * step, tl);
+    const int s = k % S;
+    mbar_arrive_expect_tx(full + s, R::SLOT);
+    tma_load_2d(slots + s * R::SLOT, &maps.w[tl.r], full + s, tl.n0 + (k % CPT) * CC, tl.row0);
+  };
+  int issued = 0;
+  if (lane == 0 && add)
+    for (; issued < S - 1 && issued < total; ++issued) issue(issued);
+  int k = 0;
+  for (; k < total; ++k) {
+    const int c = k % CPT, local = k / CPT, acc = local & 1, s = k % S;
+    if (c == 0) {
+      place(t0 + local * step, t);
+      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], (local >> 1) & 1))) {
+        if (lane == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+        break;
+      }
+      tc_fence_after();
+    }
+    if (add) {
+      if (!__all_sync(0xffffffffu, mbar_wait(full + s, (k / S) & 1))) {
+        if (lane == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+        break;
+      }
+    } else {  // the slot's last store has read it
+      if (lane == 0) bulk_wait_read<S - 1>();
+      __syncwarp();
+    }
+    uint32_t g[CC];
+    tmem_ld32(t_row + acc * BN + c * CC, g);
+    tmem_ld_wait();
+    if (c == CPT - 1) {  // the warp's accumulator part is read: the MMA may reuse it
+      tc_fence_before();
+      __syncwarp();
+      release(acc);
+    }
+    uint8_t* p = slots + s * R::SLOT;
+#pragma unroll
+    for (int j = 0; j < CC / 4; ++j) {
+      float4* q = reinterpret_cast<float4*>(p + lane * (CC * 4) + ((j ^ (lane & 7)) << 4));
+      float4 y = make_float4(__uint_as_float(g[4 * j]), __uint_as_float(g[4 * j + 1]), __uint_as_float(g[4 * j + 2]),
+                             __uint_as_float(g[4 * j + 3]));
+      if (add) {
+        const float4 d = *q;
+        y = make_float4(d.x + y.x, d.y + y.y, d.z + y.z, d.w + y.w);
+      }
+      *q = y;
+    }
+    fence_proxy_async_smem();  // the lane's values, visible to the bulk store
+    __syncwarp();
+    if (lane == 0) {
+      if (add) {
+        bulk_wait_read();  // chunk k - 1's store has read its slot: chunk k + S - 1 loads into it
+        if (issued < total) issue(issued++);
+      }
+      if (t.rows > 0) tma_store_2d(&maps.w[t.r], p, t.n0 + c * CC, t.row0);
+      bulk_commit();  // (a group per chunk, empty or not)
+    }
+    __syncwarp();
+  }
+  if (lane == 0) {
+    for (; k < issued; ++k) mbar_wait(full + k % S, (k / S) & 1);  // after a wait gave up: its copies land first
+    bulk_wait_all();  // the stores are complete before the CTA leaves
+  }
+}
+
 // Tile order.  Tiles are taken in groups of `gsz` panels of one operand: along m
 // (gsz m-blocks, m fastest) every group streams B once while its A panels stay in L2;
 // along n the roles swap.  The host picks the side and size that minimise DRAM reads.
@@ -822,6 +924,9 @@ __global__ void __launch_bounds__(EpiCfg<FAM, BN>::THREADS, 1)
     if constexpr (FAM == FAM_ADAMW)
       adamw_epilogue<BN>(epi, maps, epi_smem, epi_bars, tmem_base, warp, lane, blockIdx.x, gridDim.x, num_tiles, acc_full,
                          status, place, release);
+    else if constexpr (FAM == FAM_F32)
+      f32_epilogue<BN>(epi, maps, epi_smem, epi_bars, tmem_base, warp, lane, blockIdx.x, gridDim.x, num_tiles, acc_full,
+                         status, place, release);
     else
       epilogue_loop<FAM, BN>(epi, reinterpret_cast<float*>(epi_smem) + (warp - 2) * 32 * 64, tmem_base, warp, lane,
                              blockIdx.x, gridDim.x, num_tiles, acc_full, epi_bars, status, place, release);
@@ -1040,6 +1145,9 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
     if constexpr (FAM == FAM_ADAMW)
       adamw_epilogue<PBN>(epi, maps, epi_smem, epi_bars, tmem_base, warp, lane, pair, n_pairs, num_tiles, acc_full, status,
                           place, release);
+    else if constexpr (FAM == FAM_F32)
+      f32_epilogue<PBN>(epi, maps, epi_smem, epi_bars, tmem_base, warp, lane, pair, n_pairs, num_tiles, acc_full, status,
+                          place, release);
     else
       epilogue_loop<FAM, PBN>(epi, reinterpret_cast<float*>(epi_smem) + (warp - 2) * 32 * 64, tmem_base, warp, lane, pair,
                               n_pairs, num_tiles, acc_full, epi_bars, status, place, release);
@@ -1091,30 +1199,37 @@ inline int make_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t
   return FL_OK;
 }
 
-// 2-D tensor of the AdamW epilogue: fp32 or bf16 [rows, cols], boxes of AdamRing::CC columns x
-// 32 rows.
-inline int make_adam_map(CUtensorMap* map, const void* base, bool bf16, uint64_t cols, uint64_t rows, int64_t ld) {
+// 2-D tensor of a ring epilogue: fp32 or bf16 [rows, cols], boxes of cc columns x 32 rows, swizzled
+// over the box's row.
+inline int make_ring_map(CUtensorMap* map, const void* base, bool bf16, uint64_t cols, uint64_t rows, int64_t ld,
+                         uint32_t cc) {
   PFN_encodeTiled enc = get_encode_fn();
   if (!enc) return fl_internal_error(FL_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
   cuuint64_t dims[2] = {cols, rows};
   cuuint64_t strides[1] = {cuuint64_t(ld) * (bf16 ? 2 : 4)};
-  cuuint32_t box[2] = {AdamRing::CC, 32};
+  cuuint32_t box[2] = {cc, 32};
+  const uint32_t row = cc * (bf16 ? 2 : 4);
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
                    const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   bf16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   row == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : row == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
-    return fl_internal_error(FL_ERR_INVALID_ARG, "tensor map encode failed (%d): AdamW operand, ld %lld", (int)r, (long long)ld);
+    return fl_internal_error(FL_ERR_INVALID_ARG, "tensor map encode failed (%d): epilogue operand, ld %lld", (int)r, (long long)ld);
   return FL_OK;
 }
-// The AdamW operands' maps of every problem of a launch.
-inline int make_adam_maps(GemmMaps<FAM_ADAMW>& maps, const fl_gemm_args* a, const Problems& pr, const Epi& e) {
+// The ring epilogues' maps of every problem of a launch.
+inline int make_ring_maps(GemmMaps<FAM_F32>& maps, const fl_gemm_args* a, const Problems& pr, const Epi& e) {
+  for (int r = 0; r < pr.n; ++r)
+    if (int rc = make_ring_map(&maps.w[r], static_cast<float*>(e.D) + e.o_d[r], false, a->N, a->M, e.ldd, F32Ring::CC)) return rc;
+  return FL_OK;
+}
+inline int make_ring_maps(GemmMaps<FAM_ADAMW>& maps, const fl_gemm_args* a, const Problems& pr, const Epi& e) {
   for (int r = 0; r < pr.n; ++r) {
-    int rc = make_adam_map(&maps.w[r], static_cast<float*>(e.D) + e.o_d[r], false, a->N, a->M, e.ldd);
-    if (!rc) rc = make_adam_map(&maps.m[r], e.adam_m + e.o_adam[r], false, a->N, a->M, e.ldd);
-    if (!rc) rc = make_adam_map(&maps.v[r], e.adam_v + e.o_adam[r], false, a->N, a->M, e.ldd);
-    if (!rc) rc = make_adam_map(&maps.h[r], e.aux_out + e.o_aux_out[r], true, a->N, a->M, e.ld_aux_out);
+    int rc = make_ring_map(&maps.w[r], static_cast<float*>(e.D) + e.o_d[r], false, a->N, a->M, e.ldd, AdamRing::CC);
+    if (!rc) rc = make_ring_map(&maps.m[r], e.adam_m + e.o_adam[r], false, a->N, a->M, e.ldd, AdamRing::CC);
+    if (!rc) rc = make_ring_map(&maps.v[r], e.adam_v + e.o_adam[r], false, a->N, a->M, e.ldd, AdamRing::CC);
+    if (!rc) rc = make_ring_map(&maps.h[r], e.aux_out + e.o_aux_out[r], true, a->N, a->M, e.ld_aux_out, AdamRing::CC);
     if (rc) return rc;
   }
   return FL_OK;
@@ -1155,8 +1270,8 @@ int launch(const fl_gemm_args* a, const Problems& pr, const Epi& epi, int* statu
     else rc = make_map(&maps.b[r], pr.B[r], a->N, a->K, pr.ldb[r], BK);
     if (rc) return rc;
   }
-  if constexpr (FAM == FAM_ADAMW)
-    if (int rc = make_adam_maps(maps, a, pr, epi)) return rc;
+  if constexpr (FAM == FAM_ADAMW || FAM == FAM_F32)
+    if (int rc = make_ring_maps(maps, a, pr, epi)) return rc;
   const int num_m = (a->M + BM - 1) / BM, num_n = a->N / BN;
   const int tiles = batch * num_m * num_n;
   const int grid = tiles < num_sms() ? tiles : num_sms();
@@ -1221,8 +1336,8 @@ int launch_pair(const fl_gemm_args* a, const Problems& pr, const Epi& epi, int* 
     else rc = make_map(&maps.b[r], pr.B[r], a->N, a->K, pr.ldb[r], BK);
     if (rc) return rc;
   }
-  if constexpr (FAM == FAM_ADAMW)
-    if (int rc = make_adam_maps(maps, a, pr, epi)) return rc;
+  if constexpr (FAM == FAM_ADAMW || FAM == FAM_F32)
+    if (int rc = make_ring_maps(maps, a, pr, epi)) return rc;
   const int tiles = batch * ((a->M + PAIR_BM - 1) / PAIR_BM) * (a->N / PBN);
   const int pairs = tiles < slots ? tiles : slots;
   const Raster r = pick_raster(a->M, a->N, a->K, PAIR_BM, PBN);
@@ -1267,8 +1382,10 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
   X(EXT, W, AMN, BMN, FAM_GELU)                  \
   X(EXT, W, AMN, BMN, FAM_RESID)                 \
   X(EXT, W, AMN, BMN, FAM_ROPE)
-// FAM_ADAMW_LONG: the weight gradients' long contractions on CTA pairs only.
-#define FL_GEMM_INSTANTIATE_LONG(EXT) FL_GEMM_PAIR_FAM(EXT, 256, true, true, FAM_ADAMW_LONG)
+// The weight gradients' families on CTA pairs only: AdamW over long contractions, fp32 gradients.
+#define FL_GEMM_INSTANTIATE_WGRAD(EXT)                  \
+  FL_GEMM_PAIR_FAM(EXT, 256, true, true, FAM_ADAMW_LONG) \
+  FL_GEMM_PAIR_FAM(EXT, 256, true, true, FAM_F32)
 #define FL_GEMM_INSTANTIATE_PAIR(EXT, AMN, BMN)      \
   FL_GEMM_FAMS(FL_GEMM_PAIR_FAM, EXT, 256, AMN, BMN) \
   FL_GEMM_NARROW_FAMS(FL_GEMM_PAIR_FAM, EXT, 128, AMN, BMN)

@@ -81,8 +81,10 @@ FL_DEV void tma_store_2d(const CUtensorMap* m, const void* src, int x, int y) {
                : "memory");
 }
 FL_DEV void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// The committed bulk stores have read their shared memory (it may be written again).
-FL_DEV void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// All but the last N groups of committed bulk stores have read their shared memory (it may be
+// written again).
+template <int N = 0>
+FL_DEV void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 // The committed bulk stores are complete.
 FL_DEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 

@@ -557,6 +557,32 @@ def test_gemm_picked_tile_bit_identical(F, M, N, K, layout):
         assert (c0 - c1).abs().max() <= 2.0 ** -22 * M * max(1.0, float(D1.float().abs().max())) if kw["epilogue"] == F.FL_EPI_GELU_BWD else True
 
 
+@pytest.mark.parametrize("M,N,K", [(8, 256, 8), (264, 512, 1016), (264, 512, 1024), (2056, 4096, 200), (4104, 8192, 72)])
+def test_gemm_fp32_gradient_bit_identical(F, M, N, K):
+    """The pair tile's fp32 gradient epilogue (rows past M, rows longer than the output, one
+    tile to several per pair, one and two problems) gives the bits of the 128 x 128 tile,
+    stored and added, and touches nothing past column N; so does the tile the library picks
+    (outputs past the L2's size among them)."""
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn((K, M), generator=g, device="cuda").bfloat16()
+    B = torch.randn((K, N), generator=g, device="cuda").bfloat16()
+    D0 = torch.randn((2, M, N + 8), generator=g, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for epi in (F.FL_EPI_STORE_F32, F.FL_EPI_ACCUM_F32):
+        for n in (1, 2):
+            got = []
+            for tile in (F.FL_TILE_256x256_PAIR, F.FL_TILE_AUTO, F.FL_TILE_128x128):
+                D = D0.clone()
+                F.fl_k_gemm_multi([F.gemm_args(M, N, K, A, M, 1, B, N, 1, D[r], N + 8, epilogue=epi, tile=tile)
+                                   for r in range(n)], status)
+                got.append(D)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0
+            for D in got[:2]:
+                assert torch.equal(D.view(torch.int32), got[2].view(torch.int32)), (epi, n)
+                assert torch.equal(D[:, :, N:], D0[:, :, N:])
+
+
 @pytest.mark.parametrize("K", [8, 2048, 3064, 3072, 3080])
 def test_gemm_adamw_epilogue_against_exact(F, K):
     """The fused update on both sides of the contraction length where its epilogue changes,
