@@ -405,6 +405,39 @@ def test_attention_bwd_many_units(F, hd):
 
 
 @pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("seqs", [[256] * 10 + [1, 130], [256] * 6 + [1, 300, 130, 700]])
+def test_attention_bwd_unit_order(F, hd, seqs):
+    """Units taken in a fixed stride (two tiles per segment at most) or handed out while the
+    kernel runs (three and more), several per SM: the bits of every segment alone."""
+    nh = 16
+    H, rd = nh * hd, hd // 2
+    g = torch.Generator(device="cuda").manual_seed(hd + len(seqs))
+    T = sum(seqs)
+    qkv = torch.randn((T, 3 * H), generator=g, device="cuda").bfloat16()
+    do = torch.randn((T, H), generator=g, device="cuda").bfloat16()
+    tab = dev_f32(rope_table(max(seqs), rd, 10000.0))
+
+    def backward(lens, qkv, do):
+        cu = np.cumsum([0] + lens).astype(np.int32)
+        T, dcu = int(cu[-1]), dev_i32(cu)
+        tiles = torch.empty(F.fl_k_attention_tiles(cu) * 2, dtype=torch.int32, device="cuda")
+        o = torch.empty((T, H), dtype=torch.bfloat16, device="cuda")
+        lse, delta = torch.empty((2, nh, T), dtype=torch.float32, device="cuda")
+        dq = torch.full((T, 3 * H), float("nan"), dtype=torch.bfloat16, device="cuda")
+        F.fl_k_attention_fwd(T, nh, hd, qkv, cu, dcu, tiles, o, lse)
+        F.fl_k_attention_bwd(T, nh, hd, qkv, o, lse, do, cu, dcu, tiles, delta, tab, rd, dq)
+        torch.cuda.synchronize()
+        return dq
+
+    got, at = backward(seqs, qkv, do), 0
+    for L in seqs:
+        want = backward([L], qkv[at:at + L].clone(), do[at:at + L].clone())
+        assert torch.isfinite(want).all()
+        assert torch.equal(got[at:at + L].view(torch.int16), want.view(torch.int16)), L
+        at += L
+
+
+@pytest.mark.parametrize("hd", [64, 128])
 def test_attention_forward_output_alignment(F, hd):
     """An output that is only 16-byte aligned takes the narrower stores: the same bits."""
     nh, lens = 4, [130, 1, 128, 40]
