@@ -33,6 +33,9 @@
 // Bound by the latency of that chain, one CTA per SM (cycles of a unit of one tile: loads and
 // scores 2200, P 1100-1800, dS 1200, dK 850, output 4400).  A ninth warp to issue the products
 // (the issuer waits for room in the tensor pipe) left 168 registers a thread and spilled.
+// Against both passes in one behind a common barrier: segments of several tiles gain (4 x 2048 tokens
+// 809 -> 646 us), segments of one tile lose, in this kernel alone (64 x 128 tokens 197 -> 205 us for
+// the whole backward, 64 x 64 172 -> 180).
 // Epilogue: dK * scale, the inverse rotary rotation(s), bf16 rows of dqkv and the k / v
 // column sums for the QKV bias gradient; the prefix variant (PREFIX: the unit's keys are
 // the prefix of its head, its query tiles a slice of the call's tile list) adds dK * scale
@@ -479,10 +482,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         break;
       }
       tc_fence_after();
-      // ---- dV += P^T dO (A from TMEM) while dS^T is made; the unit's last reader of K and V is done
-      if (warp == 0) {
-        if (last && next) issue_kv(wn);
-        __syncwarp();
+      auto add_dv = [&]() {
         if (elect_one()) {
           const uint64_t bo = desc_mn(smem_u32(sdO + b * TILE));
 #pragma unroll
@@ -490,6 +490,15 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
             umma_bf16_ts(tmem + 256, tmem + a_col(kk), bo + step_mn(kk), IDESC_G, (it > w.it0 || kk > 0) ? 1u : 0u);
         }
         __syncwarp();
+      };
+      // ---- dV += P^T dO (A from TMEM) while dS^T is made; the unit's last reader of K and V is done.
+      // A unit's last tile has no later products to make room for, and the issuing warp's dS^T would
+      // be what the others wait for: its dV goes with dK.  32 x 256 tokens 234 -> 228 us, 64 x 128 211 ->
+      // 205, 16 x 512 295 -> 288, segments of 67 to 2048 335 -> 329 (late on every tile: 234, 210, 296, 340).
+      if (warp == 0) {
+        if (last && next) issue_kv(wn);
+        __syncwarp();
+        if (!last) add_dv();
       }
       // ---- dS^T, written the same way over dP^T
 #pragma unroll
@@ -527,6 +536,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         tc_fence_after();
         if (last) tm2.pend = true;
         __syncwarp();
+        if (last) add_dv();
         if (elect_one()) {
           const uint64_t bq = desc_mn(smem_u32(sQ + b * TILE));
 #pragma unroll
