@@ -1,5 +1,5 @@
-// Inline-PTX wrappers for sm_103a: mbarrier, TMA tiled loads, tcgen05 (UMMA + TMEM),
-// and the legacy warp-level mma.sync / ldmatrix used by the attention kernels.
+// Inline-PTX wrappers for sm_103a: mbarrier, TMA tiled and bulk copies, tcgen05 (UMMA + TMEM),
+// cluster launch control.
 #pragma once
 #include <cuda.h>
 #include "common.cuh"
@@ -317,31 +317,3 @@ FL_DEV void st_global_v8(void* p, const uint32_t (&x)[8]) {
                "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
                : "memory");
 }
-
-// ------------------------------------------------------------------ warp-level MMA (attention)
-FL_DEV void ldmatrix_x4(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(saddr));
-}
-FL_DEV void ldmatrix_x4_trans(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(saddr));
-}
-// D(16x8 f32) += A(16x16 bf16, row) . B(16x8 bf16, col)
-FL_DEV void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-FL_DEV void cp_async_16(uint32_t saddr, const void* gptr, bool valid) {
-  // src-size 0 zero-fills the 16 destination bytes without reading global memory
-  const int n = valid ? 16 : 0;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr), "l"(gptr), "r"(n) : "memory");
-}
-FL_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-FL_DEV void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }

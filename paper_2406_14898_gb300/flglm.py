@@ -189,7 +189,7 @@ def make_cfg(c, max_tokens: int, max_seq_len: int = 0, recompute: int = 0,
     """fl_server_cfg from a workload description with the attributes of
     ``synthetic.ServerConfig`` (n_blocks, hidden, ... , weight_decay); ``recompute``
     keeps one block's activations and recomputes the rest in the backward;
-    ``fused_step_min_tokens`` as in fl_server_cfg (0: the library's crossover);
+    ``fused_step_min_tokens`` as in fl_server_cfg (0: the library's choice);
     ``n_replicas`` > 1 holds that many server replicas in the handle (§3.3)."""
     cfg = fl_server_cfg()
     lib().fl_server_cfg_default(C.byref(cfg))
