@@ -242,8 +242,10 @@ __global__ void __cluster_dims__(CE_CLUSTER, 1, 1) __launch_bounds__(CE_THREADS,
   constexpr int W = CE_THREADS / 32;
   __shared__ float red[2][W];
   __shared__ float2 part[2][CE_CLUSTER];  // (max, sum) of each CTA's columns; rows alternate
+  cluster_arrive();
   pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
   pdl_trigger();
+  cluster_wait();  // every CTA of the cluster has started: its shared memory may be written
   const int rank = (int)cluster_ctarank(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int clusters = gridDim.x / CE_CLUSTER;
   const int ld4 = (int)(ld / 4);

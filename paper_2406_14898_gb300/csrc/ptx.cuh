@@ -245,8 +245,11 @@ FL_DEV uint32_t cluster_ctarank() {
 }
 // All threads of both CTAs; orders shared-memory and barrier operations across the pair.
 // (Not .aligned: the threads of a warp may arrive from divergent paths.)
+FL_DEV void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+FL_DEV void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 FL_DEV void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 // shared::cluster address of the same shared-memory location in CTA `rank` of the cluster.
 FL_DEV uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {

@@ -289,22 +289,29 @@ def test_cross_entropy_kernel(F, V, ld):
     assert not got[[0, 9, 30]].any()
 
 
+@pytest.mark.parametrize("rows", ["cta", "cluster", "one"])
 @pytest.mark.parametrize("V,ld", [(16381, 16384), (16385, 16388), (32766, 32768), (32769, 32776), (65536, 65540),
                                   (131071, 131072), (131073, 131076)])
-def test_cross_entropy_row_lengths(F, V, ld):
-    """Row lengths on both sides of every change of kernel, more rows than clusters, columns
-    that are masked (-inf, the lowest float) or far apart, a label on the last column; each
-    probability within 8 fp32 ulps plus one bf16 rounding of the result."""
+def test_cross_entropy_row_lengths(F, V, ld, rows):
+    """Row lengths on both sides of every change of kernel, by more rows than half of the SMs (a
+    CTA each), by as many (where long rows take a cluster each, two rows per cluster) and by one;
+    columns that are masked (-inf, the lowest float) or far apart, a label on the last column, rows
+    without a target before and after others of their cluster; each probability within 8 fp32
+    ulps plus one bf16 rounding of the result."""
     g = torch.Generator(device="cuda").manual_seed(V)
-    T = 90
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    T = {"cta": max(90, sms // 2 + 1), "cluster": sms // 2, "one": 1}[rows]
+    assert rows != "cluster" or T > 2 * sms // 8 + 5
     x = 2.0 * torch.randn((T, ld), generator=g, device="cuda")
-    x[1, : V // 2] = -float("inf")
-    x[2, 3::7] = torch.finfo(torch.float32).min
-    x[3, 5] += 80.0
-    x[4] -= 1000.0
     x[:, V:] = float("inf")  # padding is not read into the softmax
     lab = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
-    lab[0], lab[1], lab[5], lab[89] = V - 1, V - 1, -1, -3
+    lab[0] = V - 1
+    if T > 1:
+        x[1, : V // 2] = -float("inf")
+        x[2, 3:V:7] = torch.finfo(torch.float32).min
+        x[3, 5] += 80.0
+        x[4, :V] -= 1000.0
+        lab[1], lab[5], lab[T - 1] = V - 1, -1, -3
     row = torch.empty(T, device="cuda")
     dlog = torch.full((T, ld), 7.0, dtype=torch.bfloat16, device="cuda")
     loss = torch.empty(1, device="cuda")
@@ -312,7 +319,7 @@ def test_cross_entropy_row_lengths(F, V, ld):
     st = torch.zeros(1, dtype=torch.int32, device="cuda")
     F.fl_k_cross_entropy(T, V, ld, x, lab, row, dlog, loss, cnt, st)
     torch.cuda.synchronize()
-    n = T - 2
+    n = T - 2 if T > 1 else 1
     assert int(cnt.item()) == n and int(st.item()) == 0
     xd, ld_ = x[:, :V].double(), lab.long()
     lse = torch.logsumexp(xd, 1)
