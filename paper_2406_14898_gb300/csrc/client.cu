@@ -310,7 +310,8 @@ __global__ void __cluster_dims__(CE_CLUSTER, 1, 1) __launch_bounds__(CE_THREADS,
     }
     par ^= 1;
     const float inv = 1.f / (float)max(*count, 1);
-    const float f = __expf(mref - M) / S;  // exponential at hand -> probability
+    // exponential at hand -> probability (0 in a CTA none of whose columns is live)
+    const float f = __expf((m == -INFINITY ? M : m) - M) / S;
     if (rank == 0 && threadIdx.x == 0) row_loss[row] = M + logf(S) - l[y];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
@@ -320,6 +321,14 @@ __global__ void __cluster_dims__(CE_CLUSTER, 1, 1) __launch_bounds__(CE_THREADS,
 #pragma unroll
       for (int q = 0; q < 4; ++q) g[q] = (g[q] - (q == hit ? 1.f : 0.f)) * inv;
       if (j4 < ld4) d[j4] = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+    }
+    if (S != S) {  // a row that holds a NaN: zeros past the vocabulary all the same
+#pragma unroll 1
+      for (int k = 0; k < NV; ++k)
+        for (int q = 0; q < 4; ++q) {
+          const int j = 4 * ((k * CE_CLUSTER + rank) * CE_THREADS + threadIdx.x) + q;
+          if (j >= V && j < ld) dlogits[row * ld + j] = __float2bfloat16(0.f);
+        }
     }
   }
 }

@@ -336,6 +336,48 @@ def test_cross_entropy_row_lengths(F, V, ld, rows):
     assert not dlog[:, V:].any() and not dlog[~keep].any()
 
 
+@pytest.mark.parametrize("V,ld", [(9000, 16400), (32768, 32768), (60000, 65536), (131072, 131072)])
+@pytest.mark.parametrize("few", [True, False])
+def test_cross_entropy_masked_low_rows(F, V, ld, few):
+    """Rows whose live columns lie in some of a cluster's column ranges only (masked with -inf, or
+    a vocabulary that ends before the last ranges), their maximum far below zero or above: no
+    range without a live column turns into NaN; the lowest logits give probability 0."""
+    g = torch.Generator(device="cuda").manual_seed(V)
+    T = 6 if few else torch.cuda.get_device_properties(0).multi_processor_count
+    x = 2.0 * torch.randn((T, ld), generator=g, device="cuda")
+    x[:, V:] = float("nan")
+    col = torch.arange(V, device="cuda")
+    live = [(col // 2048) % 8 == 1, (col // 1024) % 2 == 0, col < 2048, col == 1, col >= V - 5, col >= 0]
+    shift = [-100.0, -1000.0, -95.0, -300.0, 200.0, -150.0]
+    lab = torch.zeros(T, device="cuda", dtype=torch.int32)
+    for i in range(T):
+        k = i % 6
+        x[i, :V] += shift[k]
+        x[i, :V][~live[k]] = -float("inf")
+        lab[i] = int(col[live[k]][-1])
+    row = torch.empty(T, device="cuda")
+    dlog = torch.full((T, ld), 7.0, dtype=torch.bfloat16, device="cuda")
+    loss = torch.empty(1, device="cuda")
+    cnt = torch.empty(1, dtype=torch.int32, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    F.fl_k_cross_entropy(T, V, ld, x, lab, row, dlog, loss, cnt, st)
+    torch.cuda.synchronize()
+    xd = x[:, :V].double()
+    lse = torch.logsumexp(xd, 1)
+    want = torch.exp(xd - lse[:, None])
+    want[torch.arange(T, device="cuda"), lab.long()] -= 1.0
+    want /= T
+    # as above: the exponent's argument, of at most 2^11, is rounded to fp32
+    assert not dlog[:, V:].any()
+    assert ((dlog[:, :V].double() - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -12 * want.abs() + 2.0 ** -18 / T).all()
+    want_row = lse - xd.gather(1, lab.long()[:, None])[:, 0]
+    assert ((row.double() - want_row).abs() <= 2.0 ** -21 * (1.0 + want_row.abs() + lse.abs())).all()
+    x[2, 0] = float("nan")  # a row that holds a NaN is NaN, its padding stays zero
+    F.fl_k_cross_entropy(T, V, ld, x, lab, row, dlog, loss, cnt, st)
+    torch.cuda.synchronize()
+    assert dlog[2, :V].isnan().all() and not dlog[:, V:].any() and dlog[[0, 1, 3], :V].isfinite().all()
+
+
 @pytest.mark.parametrize("H,off", [(256, 0), (256, 2), (258, 0), (4096, 4)])
 def test_embedding_scatter_alignment(F, H, off):
     """Vector and element-wise reductions by the alignment of the gradient and the width."""
