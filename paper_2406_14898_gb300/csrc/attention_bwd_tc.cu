@@ -206,8 +206,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   uint64_t* bar_dp = bars + 4;
   uint64_t* bar_mma2 = bars + 5;
   uint64_t* bar_clc = bars + 6;
-  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // the unit taken over
-  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 10);
+  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // [2] the unit taken over, requests alternate
+  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 12);
 
   const int nh = H / HD;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -318,14 +318,15 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   bool ok = true;
   // Units: CTA c walks c, + gridDim.x, ..., or, when the grid has one CTA per unit, the hardware
   // hands them out: the resident CTA takes over the next one that has not started, two units ahead
-  // of its work.
+  // of its work.  A request is written to the answer slot that the one before it left alone: that one
+  // may still be being read, while the slot's own last answer was read before the wait in between.
   const bool handed = (int)gridDim.x == n_units;
   int u_next = blockIdx.x;
   auto take = [&]() {
     if (!handed) return;
     tclc.pend = true;
     __syncwarp();
-    if (elect_one()) clc_request(clc, bar_clc);
+    if (elect_one()) clc_request(clc + (tclc.done & 1), bar_clc);
   };
   auto taken = [&](int& x) {  // the unit taken, or -1
     if (!handed) {
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     }
     ok = track_wait_all(bar_clc, tclc);
     if (!ok && tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-    x = ok ? clc_answer(clc) : -1;
+    x = ok ? clc_answer(clc + ((tclc.done & 1) ^ 1)) : -1;
     return ok;
   };
   Unit w = unit(blockIdx.x), wn = Unit{};
@@ -703,8 +704,8 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   uint64_t* bar_dp = bars + 4;
   uint64_t* bar_mma2 = bars + 5;
   uint64_t* bar_clc = bars + 6;
-  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // the unit taken over
-  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 10);
+  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // [2] the unit taken over, requests alternate
+  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 12);
 
   const int nh = H / HD;
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -791,14 +792,15 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   bool ok = true;
   // Units: CTA c walks c, + gridDim.x, ..., or, when the grid has one CTA per unit, the hardware
   // hands them out: the resident CTA takes over the next one that has not started, two units ahead
-  // of its work.
+  // of its work.  A request is written to the answer slot that the one before it left alone: that one
+  // may still be being read, while the slot's own last answer was read before the wait in between.
   const bool handed = (int)gridDim.x == n_units;
   int u_next = blockIdx.x;
   auto take = [&]() {
     if (!handed) return;
     tclc.pend = true;
     __syncwarp();
-    if (elect_one()) clc_request(clc, bar_clc);
+    if (elect_one()) clc_request(clc + (tclc.done & 1), bar_clc);
   };
   auto taken = [&](int& x) {  // the unit taken, or -1
     if (!handed) {
@@ -808,7 +810,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     }
     ok = track_wait_all(bar_clc, tclc);
     if (!ok && tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-    x = ok ? clc_answer(clc) : -1;
+    x = ok ? clc_answer(clc + ((tclc.done & 1) ^ 1)) : -1;
     return ok;
   };
   Unit w = unit(blockIdx.x), wn = Unit{};
