@@ -175,14 +175,14 @@ FL_DEV void staged_colsum(uint8_t* stage, int rows, float* out, int tid) {
 // dK / dV.  Non-prefix: unit u = (entry u / nh of the 128-row tile list, head u % nh), the
 // entry's tile index i standing for key tile nq - 1 - i (a segment's key tile 0, seen by
 // every query tile, first).
-// PREFIX: unit u = (slice u / nh of the tile list cut into n_split slices, head u % nh),
-// the unit's keys the Lp prefix keys of its head.
+// PREFIX: unit u = (slice u / nh of the tile list cut into slices of `per` tiles, head u % nh),
+// the unit's keys the Lp prefix keys of its head.  Every unit has a query tile.
 template <int HD, bool PREFIX>
 __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     const __grid_constant__ CUtensorMap tm_qkv, const __grid_constant__ CUtensorMap tm_do,
     const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
     const __grid_constant__ CUtensorMap tm_dqkv, int T, int H,
-    const int32_t* __restrict__ cu, const uint32_t* __restrict__ tiles, int n_tiles, int n_units, int n_split,
+    const int32_t* __restrict__ cu, const uint32_t* __restrict__ tiles, int n_tiles, int n_units, int per,
     const float* __restrict__ lse, const float* __restrict__ delta, const float2* __restrict__ rope_tab, float scale,
     float scale_log2, int Lp, bf16* __restrict__ dqkv, float* __restrict__ dpk, float* __restrict__ dpv,
     const int32_t* __restrict__ ctxs, const int32_t* __restrict__ gpos, const int32_t* __restrict__ gpos2,
@@ -226,7 +226,6 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     Unit w;
     w.h = u % nh;
     if constexpr (PREFIX) {
-      const int per = (n_tiles + n_split - 1) / n_split;
       w.it0 = (u / nh) * per;
       w.it_end = min(n_tiles, w.it0 + per);
       w.seg0 = w.L = w.kb = 0;
@@ -348,14 +347,12 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     const float* src = tid < TB ? lse : delta;
     return c < valid ? __ldg(src + (int64_t)x.h * T + row0 + c) : 0.f;
   };
-  float pf = w.it0 < w.it_end ? stat_of(w, w.it0) : 0.f;
+  float pf = stat_of(w, w.it0);
   RopeRow<HD> rrow;
   if (warp == 0) {
-    if (w.it0 < w.it_end) {
-      issue_kv(w);
-      issue_q(w, w.it0, 0);
-      if (w.it0 + 1 < w.it_end) issue_q(w, w.it0 + 1, 1);
-    }
+    issue_kv(w);
+    issue_q(w, w.it0, 0);
+    if (w.it0 + 1 < w.it_end) issue_q(w, w.it0 + 1, 1);
     take();
   }
   int un;
@@ -363,16 +360,15 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   while (ok) {
     const int k = w.kb + r;  // the key inside its segment (or the prefix)
     const bool key_ok = PREFIX ? r < Lp : k < w.L;
-    const bool work = w.it0 < w.it_end;
     // the next unit: its K / V load once this unit's last S^T / dP^T products have read K
     // and V, its first query tile once buffer pair 0 has had its last use here
-    const bool next = un >= 0 && wn.it0 < wn.it_end;
+    const bool next = un >= 0;
     Unit wnn = Unit{};  // the unit after next: taken over while the first score products run,
     int unn = -1;       // read after the first pass
     uint32_t tnn = 0;
-    if (un >= 0 && warp == 0) take();
+    if (next && warp == 0) take();
     // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
-    if (work && !track_wait_all(bar_kv, tkv)) {
+    if (!track_wait_all(bar_kv, tkv)) {
       if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
       ok = false;
       break;
@@ -391,16 +387,14 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       }
       __syncwarp();
     };
-    if (work) {
-      if (!track_wait_all(bar_q, tq0)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
-      if (warp == 0) {
-        tc_fence_after();
-        scores(0);
-      }
+    if (!track_wait_all(bar_q, tq0)) {
+      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
+      ok = false;
+      break;
+    }
+    if (warp == 0) {
+      tc_fence_after();
+      scores(0);
     }
     for (int it = w.it0; it < w.it_end && ok; ++it) {
       const int b = (it - w.it0) & 1;
@@ -471,7 +465,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       };
       if (open) probs(std::false_type{});
       else probs(std::true_type{});
-      if (it == w.it0 && un >= 0) {
+      if (it == w.it0 && next) {
         if (!taken(unn)) break;
         if (unn >= 0) tnn = tile_word(unn);
       }
@@ -569,92 +563,81 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
 
     // ---- every product of the unit is complete: its dK / dV leave while the next unit's
     // tiles load
-    if (warp == 0 && next && !work) {
-      issue_kv(wn);
-      issue_q(wn, wn.it0, 0);
-      if (wn.it0 + 1 < wn.it_end) issue_q(wn, wn.it0 + 1, 1);
-    }
-    if (work) {
-      if constexpr (PREFIX) {
-        // ---- dK * scale and dV added into the fp32 prefix gradients: thread (r, qh) adds
-        // dims qh * HD/2 .. + HD/2 - 1 of prefix key r
+    if constexpr (PREFIX) {
+      // ---- dK * scale and dV added into the fp32 prefix gradients: thread (r, qh) adds
+      // dims qh * HD/2 .. + HD/2 - 1 of prefix key r
 #pragma unroll 1
-        for (int part = 0; part < 2; ++part) {  // 0: dK, 1: dV
-          uint32_t vr[HD / 2];
+      for (int part = 0; part < 2; ++part) {  // 0: dK, 1: dV
+        uint32_t vr[HD / 2];
 #pragma unroll
-          for (int c = 0; c < HD / 2; c += 32)
-            tmem_ld32(t_lane + (part ? 256 : 256 + HD) + qh * (HD / 2) + c,
-                      *reinterpret_cast<uint32_t(*)[32]>(vr + c));
-          tmem_ld_wait();
-          if (key_ok) {
-            const float f = part ? 1.f : scale;
-            float* dst = (part ? dpv : dpk) + (int64_t)r * H + w.h * HD + qh * (HD / 2);
+        for (int c = 0; c < HD / 2; c += 32)
+          tmem_ld32(t_lane + (part ? 256 : 256 + HD) + qh * (HD / 2) + c,
+                    *reinterpret_cast<uint32_t(*)[32]>(vr + c));
+        tmem_ld_wait();
+        if (key_ok) {
+          const float f = part ? 1.f : scale;
+          float* dst = (part ? dpv : dpk) + (int64_t)r * H + w.h * HD + qh * (HD / 2);
 #pragma unroll
-            for (int c = 0; c < HD / 2; c += 4)
-              red_add_v4(dst + c, __uint_as_float(vr[c]) * f, __uint_as_float(vr[c + 1]) * f,
-                         __uint_as_float(vr[c + 2]) * f, __uint_as_float(vr[c + 3]) * f);
+          for (int c = 0; c < HD / 2; c += 4)
+            red_add_v4(dst + c, __uint_as_float(vr[c]) * f, __uint_as_float(vr[c + 1]) * f,
+                       __uint_as_float(vr[c + 2]) * f, __uint_as_float(vr[c + 3]) * f);
+        }
+      }
+    } else {
+      // ---- dV, then dK (scaled, rotated back): thread (r, qh) takes dims qh * HD/2 .. +
+      // HD/2 - 1 of key row r from TMEM and stages the bf16 rows; a tile inside the
+      // segment leaves by bulk tensor stores, a ragged last tile by coalesced 16-byte
+      // stores of its valid rows; the bias column sums are taken from the staged rows
+      // (the values stored)
+#pragma unroll 1
+      for (int pi = 0; pi < 2; ++pi) {
+        const int part = 1 - pi;  // dV, then dK
+        uint8_t* stage = sST;
+        uint32_t vr[HD / 2];
+        float* v = reinterpret_cast<float*>(vr);
+#pragma unroll
+        for (int c = 0; c < HD / 2; c += 32)
+          tmem_ld32(t_lane + (part ? 256 : 256 + HD) + qh * (HD / 2) + c,
+                    *reinterpret_cast<uint32_t(*)[32]>(vr + c));
+        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < HD / 2; ++c) v[c] = __uint_as_float(vr[c]) * (part ? 1.f : scale);
+        if (part == 0 && qh < nreg && key_ok) inverse_rope_row<HD>(v, rrow);  // rotary region qh
+        // the staging tile is free once the previous bulk store has read it
+        if (tid == 0) bulk_wait_read();
+        __syncthreads();
+#pragma unroll
+        for (int c8 = 0; c8 < HD / 16; ++c8)
+          *reinterpret_cast<uint4*>(stage_chunk<HD>(stage, r, qh * (HD / 16) + c8)) =
+              make_uint4(pack_bf16x2(v[8 * c8], v[8 * c8 + 1]), pack_bf16x2(v[8 * c8 + 2], v[8 * c8 + 3]),
+                         pack_bf16x2(v[8 * c8 + 4], v[8 * c8 + 5]), pack_bf16x2(v[8 * c8 + 6], v[8 * c8 + 7]));
+        const int col = (part ? 2 * H : H) + w.h * HD;
+        const bool full = w.kb + TB <= w.L;  // a whole tile of the segment: TMA stores
+        if (full) fence_proxy_async_smem();  // the staged rows, visible to the bulk copies
+        __syncthreads();  // the tile is staged
+        if (full && tid == 0) {
+#pragma unroll
+          for (int x = 0; x < NB; ++x) tma_store_2d(&tm_dqkv, stage + x * (TB * 128), col + 64 * x, w.seg0 + w.kb);
+          bulk_commit();
+        }
+        if (w.db) staged_colsum<HD>(stage, min(TB, w.L - w.kb), w.db + col, tid);
+        if (!full) {
+          // 128 rows x CH chunks: consecutive threads write consecutive chunks of a row
+#pragma unroll
+          for (int i = 0; i < TB * CH / 256; ++i) {
+            const int id = tid + 256 * i, row = id / CH, jc = id % CH;
+            if (w.kb + row < w.L)
+              *reinterpret_cast<uint4*>(dqkv + ((int64_t)w.seg0 + w.kb + row) * 3 * H + col + jc * 8) =
+                  *reinterpret_cast<const uint4*>(stage_chunk<HD>(stage, row, jc));
           }
         }
-      } else {
-        // ---- dV, then dK (scaled, rotated back): thread (r, qh) takes dims qh * HD/2 .. +
-        // HD/2 - 1 of key row r from TMEM and stages the bf16 rows; a tile inside the
-        // segment leaves by bulk tensor stores, a ragged last tile by coalesced 16-byte
-        // stores of its valid rows; the bias column sums are taken from the staged rows
-        // (the values stored)
-#pragma unroll 1
-        for (int pi = 0; pi < 2; ++pi) {
-          const int part = 1 - pi;  // dV, then dK
-          uint8_t* stage = sST;
-          uint32_t vr[HD / 2];
-          float* v = reinterpret_cast<float*>(vr);
-#pragma unroll
-          for (int c = 0; c < HD / 2; c += 32)
-            tmem_ld32(t_lane + (part ? 256 : 256 + HD) + qh * (HD / 2) + c,
-                      *reinterpret_cast<uint32_t(*)[32]>(vr + c));
-          tmem_ld_wait();
-#pragma unroll
-          for (int c = 0; c < HD / 2; ++c) v[c] = __uint_as_float(vr[c]) * (part ? 1.f : scale);
-          if (part == 0 && qh < nreg && key_ok) inverse_rope_row<HD>(v, rrow);  // rotary region qh
-          // the staging tile is free once the previous bulk store has read it
-          if (tid == 0) bulk_wait_read();
-          __syncthreads();
-#pragma unroll
-          for (int c8 = 0; c8 < HD / 16; ++c8)
-            *reinterpret_cast<uint4*>(stage_chunk<HD>(stage, r, qh * (HD / 16) + c8)) =
-                make_uint4(pack_bf16x2(v[8 * c8], v[8 * c8 + 1]), pack_bf16x2(v[8 * c8 + 2], v[8 * c8 + 3]),
-                           pack_bf16x2(v[8 * c8 + 4], v[8 * c8 + 5]), pack_bf16x2(v[8 * c8 + 6], v[8 * c8 + 7]));
-          const int col = (part ? 2 * H : H) + w.h * HD;
-          const bool full = w.kb + TB <= w.L;  // a whole tile of the segment: TMA stores
-          if (full) fence_proxy_async_smem();  // the staged rows, visible to the bulk copies
-          __syncthreads();  // the tile is staged
-          if (full && tid == 0) {
-#pragma unroll
-            for (int x = 0; x < NB; ++x) tma_store_2d(&tm_dqkv, stage + x * (TB * 128), col + 64 * x, w.seg0 + w.kb);
-            bulk_commit();
-          }
-          if (w.db) staged_colsum<HD>(stage, min(TB, w.L - w.kb), w.db + col, tid);
-          if (!full) {
-            // 128 rows x CH chunks: consecutive threads write consecutive chunks of a row
-#pragma unroll
-            for (int i = 0; i < TB * CH / 256; ++i) {
-              const int id = tid + 256 * i, row = id / CH, jc = id % CH;
-              if (w.kb + row < w.L)
-                *reinterpret_cast<uint4*>(dqkv + ((int64_t)w.seg0 + w.kb + row) * 3 * H + col + jc * 8) =
-                    *reinterpret_cast<const uint4*>(stage_chunk<HD>(stage, row, jc));
-            }
-          }
-          __syncthreads();  // the staged rows have been read (the bulk store reads them on)
-        }
+        __syncthreads();  // the staged rows have been read (the bulk store reads them on)
       }
     }
     // the dK / dV columns are loaded before the next unit's products overwrite them
     tc_fence_before();
     __syncthreads();
-    if (un < 0) break;
-    if (!work) {  // no first pass to read the answer after
-      if (!taken(unn)) break;
-      if (unn >= 0) wnn = unit(unn);
-    }
+    if (!next) break;
     w = wn;
     wn = wnn;
     un = unn;
@@ -1049,6 +1032,23 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   }
 }
 
+// A list of n_tiles > 0 tiles cut into at most `want` slices of equal length but the last: the tiles of
+// a slice, and the number of slices, none of them empty.
+constexpr int slice_tiles(int n_tiles, int want) {
+  const int n = want < 1 ? 1 : want < n_tiles ? want : n_tiles;
+  return (n_tiles + n - 1) / n;
+}
+constexpr int slices(int n_tiles, int per) { return (n_tiles + per - 1) / per; }
+constexpr bool slices_hold_tiles(int max_tiles, int max_want) {
+  for (int n = 1; n <= max_tiles; ++n)
+    for (int want = 1; want <= max_want; ++want) {
+      const int per = slice_tiles(n, want), k = slices(n, per);
+      if (k > want || (k - 1) * per >= n || k * per < n) return false;
+    }
+  return true;
+}
+static_assert(slices_hold_tiles(200, 160), "slices");
+
 template <int HD>
 int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float* lse, const float* delta,
                   const int32_t* cu, const uint32_t* tiles, int n_tiles, int max_tiles, const float* rope_tab, void* dqkv,
@@ -1088,11 +1088,9 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
   }
   if (pre.len > 0 && n_tiles > 0) {
     // the prefix keys of each head against slices of the query tiles, about one CTA per SM
-    int nsplit = (fl_sm_count() + nh - 1) / nh;
-    if (nsplit > n_tiles) nsplit = n_tiles;
-    if (nsplit < 1) nsplit = 1;
+    const int per = slice_tiles(n_tiles, (fl_sm_count() + nh - 1) / nh), nsplit = slices(n_tiles, per);
     FL_CUDA_TRY(fl_launch(attn_bwd_dkv_tc_kernel<HD, true>, dim3(nsplit * nh), dim3(256), BwdCfg<HD>::SMEM, st, tq,
-                          tdo, tpk, tpv, tdq, T, H, cu, tiles, n_tiles, nsplit * nh, nsplit, lse, delta, tab, scale,
+                          tdo, tpk, tpv, tdq, T, H, cu, tiles, n_tiles, nsplit * nh, per, lse, delta, tab, scale,
                           scale * LOG2E_B, pre.len, (bf16*)dqkv, pre.dk, pre.dv, glm.ctx, glm.pos, glm.pos2,
                           (float*)nullptr, 0, (int64_t)0, status));
   }

@@ -500,6 +500,34 @@ def test_attention_with_prefix(F, hd, Lp):
     assert rel_inf(f64(gpv), dpvr.reshape(Lp, H)) < 5e-2
 
 
+@pytest.mark.parametrize("nh,hd,seqs", [(16, 64, [70] * 11), (32, 128, [40] * 6), (4, 64, [9] * 39),
+                                        (16, 128, [300, 1, 128, 5, 260, 129, 2])])
+def test_attention_prefix_slices(F, nh, hd, seqs):
+    """Prefix gradients where the query tiles do not divide into a slice per SM (11 tiles for 10
+    slices, 6 for 5, 39 for 38 on 152 SMs), and with more slices times heads than SMs, whose units
+    are handed out while the kernel runs: every tile's share, added once."""
+    Lp, H = 24, nh * hd
+    cu = np.cumsum([0] + seqs).astype(np.int32)
+    T = int(cu[-1])
+    rng = np.random.default_rng(nh + hd)
+    qkv, do = rnd_bf16_f64(rng, (T, 3 * H)), rnd_bf16_f64(rng, (T, H))
+    pk, pv = rnd_bf16_f64(rng, (Lp, H)), rnd_bf16_f64(rng, (Lp, H))
+    dqkv_, dcu, dpk_, dpv_ = dev_bf16(qkv), dev_i32(cu), dev_bf16(pk), dev_bf16(pv)
+    tiles = torch.empty(F.fl_k_attention_tiles(cu) * 2, dtype=torch.int32, device="cuda")
+    o = torch.empty((T, H), dtype=torch.bfloat16, device="cuda")
+    lse, delta = torch.empty((2, nh, T), dtype=torch.float32, device="cuda")
+    F.fl_k_attention_fwd(T, nh, hd, dqkv_, cu, dcu, tiles, o, lse, dpk_, dpv_, Lp)
+    dq = torch.empty((T, 3 * H), dtype=torch.bfloat16, device="cuda")
+    gpk, gpv = torch.zeros((2, Lp, H), dtype=torch.float32, device="cuda")
+    F.fl_k_attention_bwd(T, nh, hd, dqkv_, o, lse, dev_bf16(do), cu, dcu, tiles, delta, None, 0, dq,
+                         dpk_, dpv_, Lp, gpk, gpv)
+    torch.cuda.synchronize()
+    r = lambda x: x.reshape(-1, nh, hd)
+    _, _, _, dpkr, dpvr = O.attention_bwd(r(do), r(qkv[:, :H]), r(qkv[:, H:2 * H]), r(qkv[:, 2 * H:]), cu, r(pk), r(pv))
+    assert rel_inf(f64(gpk), dpkr.reshape(Lp, H)) < 5e-2
+    assert rel_inf(f64(gpv), dpvr.reshape(Lp, H)) < 5e-2
+
+
 @pytest.mark.parametrize("tile", ["auto", "pair"])
 @pytest.mark.parametrize("M,N,K,mn", [(200, 384, 136, 1), (256, 512, 64, 1), (130, 256, 96, 0), (600, 1024, 520, 1)])
 def test_gemm_adamw_epilogue(F, M, N, K, mn, tile):
