@@ -5,10 +5,12 @@
 // Shared layout of both kernels: 128-row tiles; operands arrive by TMA as 64-column
 // 128-byte-swizzled boxes; the score-side products (S, dP or their transposes) sit in
 // TMEM columns [0, 256); the probabilities / score gradients the threads derive from them
-// are stored back into TMEM (bf16, two per 32-bit column) over the values already read,
-// and feed the next products as A operands read from TMEM.  That leaves shared memory to
-// double-buffer the tiles the CTA walks through, so their loads overlap the work on the
-// previous tile.
+// are stored back into TMEM (bf16, two per 32-bit column) and feed the next products as A
+// operands read from TMEM.  That leaves shared memory to double-buffer the tiles the CTA
+// walks through, so their loads overlap the work on the previous tile.  Products of
+// different shapes or accumulators keep no order among themselves: a product is issued
+// while others run only if it writes none of the columns that they read, else after a wait
+// for a commit behind them (PTX orders only those of one shape into one accumulator).
 //
 // Both kernels are persistent: one CTA per SM (226 KB of shared memory at head_dim 128,
 // 512 TMEM columns) walks work units, in a fixed stride or as the hardware hands them out
@@ -28,8 +30,9 @@
 //   threads: P^T = exp2(S^T scale log2e - lse_q log2e) where key r is visible to query q, as
 //            soon as S^T is complete; then, while dV += P^T dO_i -> TMEM [256, 256 + hd) runs,
 //            dS^T = P^T (dP^T - delta_q); both bf16 over the S^T / dP^T values just read;
-//   dK += dS^T Q_i -> TMEM [256 + hd, 256 + 2 hd), with S^T and dP^T of tile i + 1 right behind it
-//            (A from TMEM, dO_i and Q_i as MN-major operands).
+//   dK += dS^T Q_i -> TMEM [256 + hd, 256 + 2 hd) (A from TMEM, dO_i and Q_i as MN-major operands),
+//            with S^T of tile i + 1 right behind it, over the P^T of a dV that is complete by then;
+//            dP^T of tile i + 1, over the dS^T that dK reads, once that S^T, and so dK, is complete.
 // Bound by the latency of that chain, one CTA per SM (cycles of a unit of one tile: loads and
 // scores 2200, P 1100-1800, dS 1200, dK 850, output 4400).  A ninth warp to issue the products
 // (the issuer waits for room in the tensor pipe) left 168 registers a thread and spilled.
@@ -46,8 +49,10 @@
 // segment's own keys), K_j / V_j double-buffered:
 //   S = Q K_j^T -> TMEM [0, 128), dP = dO V_j^T -> TMEM [128, 256);
 //   threads: dS = P (dP - delta_q), P = exp2(S scale log2e - lse_q log2e) on the visible
-//            keys, bf16 over the S values just read;
-//   dQ += dS K_j -> TMEM [256, 256 + hd) (A from TMEM, K_j as an MN-major operand).
+//            keys, bf16 in TMEM [256 + hd, 320 + hd), which the dQ product before, complete with
+//            this tile's S, has read;
+//   dQ += dS K_j -> TMEM [256, 256 + hd) (A from TMEM, K_j as an MN-major operand), S and dP of the
+//            next tile right behind it.
 // Epilogue as in dK / dV: dQ * scale, inverse rotary rotation(s), coalesced bf16 rows, q
 // column sums.
 //
@@ -92,7 +97,7 @@ FL_DEV constexpr uint64_t step_k(int kk) { return (kk >> 2) * (BOX / 16) + (kk &
 FL_DEV uint64_t desc_mn(uint32_t base) { return smem_desc_sw128(base, BOX, 1024); }
 FL_DEV constexpr uint64_t step_mn(int kk) { return kk * 128; }
 
-// TMEM column (relative to the region's start) of the bf16 operand's k-step kk (16
+// dK / dV: TMEM column (relative to the region's start) of the bf16 operand's k-step kk (16
 // columns of the 128-wide product): thread half g = kk / 4 wrote its columns 64 g .. + 63
 // as two groups of 32 values at 64 g + 16 hf (hf = (kk / 2) % 2), 8 columns per k-step.
 FL_DEV uint32_t a_col(int kk) { return (kk >> 2) * 64 + ((kk >> 1) & 1) * 16 + (kk & 1) * 8; }
@@ -200,14 +205,9 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   float* sL = reinterpret_cast<float*>(smem + 7 * TILE);  // [128] lse * log2e of the query tile
   float* sD = sL + TB;                                    // [128] delta of the query tile
   uint64_t* bars = reinterpret_cast<uint64_t*>(sD + TB);
-  uint64_t* bar_kv = bars;
-  uint64_t* bar_q = bars + 1;  // [2]
-  uint64_t* bar_s = bars + 3;
-  uint64_t* bar_dp = bars + 4;
-  uint64_t* bar_mma2 = bars + 5;
-  uint64_t* bar_clc = bars + 6;
-  uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // [2] the unit taken over, requests alternate
-  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 12);
+  enum { B_KV = 0, B_Q = 1 /* and 2 */, B_S = 3, B_DP = 4, B_MMA2 = 5, B_CLC = 6, B_DV = 7, BARS = 8 };
+  uint4* clc = reinterpret_cast<uint4*>(bars + 10);  // [2] the unit taken over, requests alternate
+  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 14);
 
   const int nh = H / HD;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   };
 
   if (tid == 0) {
-    for (int i = 0; i < 7; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < BARS; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
     tma_prefetch_desc(&tm_do);
@@ -279,63 +279,65 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
-  BarTrack tkv, tq0, tq1, ts, tdp, tm2, tclc;
+  BarTracks tr;
+  bool ok = true;
+  // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
+  auto wait_all = [&](int i, int code) {
+    ok = track_wait_all(bars, i, tr);
+    if (!ok && tid == 0) report_status(status, code);
+    return ok;
+  };
   // Copies and products are issued by warp 0 as a whole, one elected lane at work: the
   // instructions' operands stay in uniform registers.
   auto issue_q = [&](const Unit& w, int it, int b) {  // Q_it, dO_it into pair b
     int row0, qpos0, valid;
     qtile(w, it, row0, qpos0, valid);
-    (b ? tq1 : tq0).pend = true;
+    tr.arm(B_Q + b);
     __syncwarp();
     if (!elect_one()) return;
-    mbar_arrive_expect_tx(bar_q + b, 2 * TILE);
+    mbar_arrive_expect_tx(bars + B_Q + b, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
-      tma_load_2d(sQ + b * TILE + x * BOX, &tm_qkv, bar_q + b, w.h * HD + 64 * x, row0);
-      tma_load_2d(sdO + b * TILE + x * BOX, &tm_do, bar_q + b, w.h * HD + 64 * x, row0);
+      tma_load_2d(sQ + b * TILE + x * BOX, &tm_qkv, bars + B_Q + b, w.h * HD + 64 * x, row0);
+      tma_load_2d(sdO + b * TILE + x * BOX, &tm_do, bars + B_Q + b, w.h * HD + 64 * x, row0);
     }
   };
   auto issue_kv = [&](const Unit& w) {  // the unit's K and V
-    tkv.pend = true;
+    tr.arm(B_KV);
     __syncwarp();
     if (!elect_one()) return;
-    mbar_arrive_expect_tx(bar_kv, 2 * TILE);
+    mbar_arrive_expect_tx(bars + B_KV, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
       if constexpr (PREFIX) {
-        tma_load_2d(sK + x * BOX, &tm_pk, bar_kv, w.h * HD + 64 * x, 0);
-        tma_load_2d(sV + x * BOX, &tm_pv, bar_kv, w.h * HD + 64 * x, 0);
+        tma_load_2d(sK + x * BOX, &tm_pk, bars + B_KV, w.h * HD + 64 * x, 0);
+        tma_load_2d(sV + x * BOX, &tm_pv, bars + B_KV, w.h * HD + 64 * x, 0);
       } else {
-        tma_load_2d(sK + x * BOX, &tm_qkv, bar_kv, H + w.h * HD + 64 * x, w.seg0 + w.kb);
-        tma_load_2d(sV + x * BOX, &tm_qkv, bar_kv, 2 * H + w.h * HD + 64 * x, w.seg0 + w.kb);
+        tma_load_2d(sK + x * BOX, &tm_qkv, bars + B_KV, H + w.h * HD + 64 * x, w.seg0 + w.kb);
+        tma_load_2d(sV + x * BOX, &tm_qkv, bars + B_KV, 2 * H + w.h * HD + 64 * x, w.seg0 + w.kb);
       }
     }
   };
 
   constexpr uint32_t IDESC_S = umma_idesc_bf16(TB, TB, false, false);
   constexpr uint32_t IDESC_G = umma_idesc_bf16(TB, HD, false, true);
-  bool ok = true;
   // Units: CTA c walks c, + gridDim.x, ..., or, when the grid has one CTA per unit, the hardware
   // hands them out: the resident CTA takes over the next one that has not started, two units ahead
   // of its work.  A request is written to the answer slot that the one before it left alone: that one
   // may still be being read, while the slot's own last answer was read before the wait in between.
   const bool handed = (int)gridDim.x == n_units;
-  int u_next = blockIdx.x;
   auto take = [&]() {
     if (!handed) return;
-    tclc.pend = true;
+    tr.arm(B_CLC);
     __syncwarp();
-    if (elect_one()) clc_request(clc + (tclc.done & 1), bar_clc);
+    if (elect_one()) clc_request(clc + tr.parity(B_CLC), bars + B_CLC);
   };
-  auto taken = [&](int& x) {  // the unit taken, or -1
+  auto taken = [&](int u, int& x) {  // the unit after unit u, or -1
     if (!handed) {
-      u_next += gridDim.x;
-      x = u_next < n_units ? u_next : -1;
+      x = u + (int)gridDim.x < n_units ? u + gridDim.x : -1;
       return true;
     }
-    ok = track_wait_all(bar_clc, tclc);
-    if (!ok && tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-    x = ok ? clc_answer(clc + ((tclc.done & 1) ^ 1)) : -1;
+    x = wait_all(B_CLC, FL_DEV_TIMEOUT_FULL) ? clc_answer(clc + (tr.parity(B_CLC) ^ 1)) : -1;
     return ok;
   };
   Unit w = unit(blockIdx.x), wn = Unit{};
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     take();
   }
   int un;
-  if (taken(un) && un >= 0) wn = unit(un);
+  if (taken(blockIdx.x, un) && un >= 0) wn = unit(un);
   while (ok) {
     const int k = w.kb + r;  // the key inside its segment (or the prefix)
     const bool key_ok = PREFIX ? r < Lp : k < w.L;
@@ -367,34 +369,24 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     int unn = -1;       // read after the first pass
     uint32_t tnn = 0;
     if (next && warp == 0) take();
-    // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
-    if (!track_wait_all(bar_kv, tkv)) {
-      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-      ok = false;
-      break;
-    }
-    auto scores = [&](int b) {  // warp 0: S^T = K Q^T and dP^T = V dO^T of the tile in pair b
-      ts.pend = tdp.pend = true;
-      if (elect_one()) {
-        const uint64_t ak = desc_k(smem_u32(sK)), av = desc_k(smem_u32(sV)), bq = desc_k(smem_u32(sQ + b * TILE)),
-                       bo = desc_k(smem_u32(sdO + b * TILE));
+    if (!wait_all(B_KV, FL_DEV_TIMEOUT_FULL)) break;
+    // warp 0: S^T = K Q^T (part 0) or dP^T = V dO^T (part 1) of the tile in pair b
+    auto scores = [&](int b, int part) {
+      const uint64_t a = desc_k(smem_u32(part ? sV : sK)), q = desc_k(smem_u32((part ? sdO : sQ) + b * TILE));
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, ak + step_k(kk), bq + step_k(kk), IDESC_S, kk > 0);
-        umma_commit(bar_s);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, av + step_k(kk), bo + step_k(kk), IDESC_S, kk > 0);
-        umma_commit(bar_dp);
-      }
-      __syncwarp();
+      for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128 * part, a + step_k(kk), q + step_k(kk), IDESC_S, kk > 0);
+      umma_commit(bars + (part ? B_DP : B_S));
     };
-    if (!track_wait_all(bar_q, tq0)) {
-      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-      ok = false;
-      break;
-    }
+    if (!wait_all(B_Q, FL_DEV_TIMEOUT_FULL)) break;
     if (warp == 0) {
       tc_fence_after();
-      scores(0);
+      tr.arm(B_S);
+      tr.arm(B_DP);
+      if (elect_one()) {
+        scores(0, 0);
+        scores(0, 1);
+      }
+      __syncwarp();
     }
     for (int it = w.it0; it < w.it_end && ok; ++it) {
       const int b = (it - w.it0) & 1;
@@ -409,15 +401,17 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       // while the products run: the next tile's statistics, the unit after next
       if (!last) pf = stat_of(w, it + 1);
       else if (next) pf = stat_of(wn, wn.it0);
-      if (!track_wait_all(bar_s, ts)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
-        ok = false;
-        break;
-      }
+      if (!wait_all(B_S, FL_DEV_TIMEOUT_ACC_FULL)) break;
       tc_fence_after();
-      // S^T is complete and so is every product issued before it: the other buffer pair is free
-      // for the next tile (the second tile of a unit was loaded at the end of the unit before)
+      // S^T is complete and so is every product issued before it: the dS^T columns are free for the
+      // dP^T of a tile after the first, and the other buffer pair for the next tile (the second tile
+      // of a unit was loaded at the end of the unit before)
       if (warp == 0) {
+        if (it > w.it0) {
+          tr.arm(B_DP);
+          if (elect_one()) scores(b, 1);
+          __syncwarp();
+        }
         if (!last) {
           if (it > w.it0) issue_q(w, it + 1, 1 - b);
         } else if (next && wn.it0 + (1 - b) < wn.it_end) {
@@ -466,16 +460,12 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       if (open) probs(std::false_type{});
       else probs(std::true_type{});
       if (it == w.it0 && next) {
-        if (!taken(unn)) break;
+        if (!taken(un, unn)) break;
         if (unn >= 0) tnn = tile_word(unn);
       }
       tmem_st_wait();
       tc_fence_before();
-      if (!track_wait_all(bar_dp, tdp)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
-        ok = false;
-        break;
-      }
+      if (!wait_all(B_DP, FL_DEV_TIMEOUT_ACC_FULL)) break;
       tc_fence_after();
       auto add_dv = [&]() {
         if (elect_one()) {
@@ -493,7 +483,12 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       if (warp == 0) {
         if (last && next) issue_kv(wn);
         __syncwarp();
-        if (!last) add_dv();
+        if (!last) {
+          tr.arm(B_DV);
+          add_dv();
+          if (elect_one()) umma_commit(bars + B_DV);
+          __syncwarp();
+        }
       }
       // ---- dS^T, written the same way over dP^T
 #pragma unroll
@@ -520,28 +515,31 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       // the next tile's Q and dO have landed (and every thread has written its dS^T)
       if (last) {
         __syncthreads();
-      } else if (!track_wait_all(bar_q + 1 - b, b ? tq0 : tq1)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
-      // ---- dK += dS^T Q, and the next tile's scores behind it (they overwrite P^T and dS^T, which
-      // the products before them in the tensor pipe have read)
+      } else if (!wait_all(B_Q + 1 - b, FL_DEV_TIMEOUT_FULL)) break;
+      // ---- dK += dS^T Q, and the next tile's S^T behind it
       if (warp == 0) {
         tc_fence_after();
-        if (last) tm2.pend = true;
+        if (last) tr.arm(B_MMA2);
         __syncwarp();
         if (last) add_dv();
         if (elect_one()) {
           const uint64_t bq = desc_mn(smem_u32(sQ + b * TILE));
 #pragma unroll
           for (int kk = 0; kk < TB / 16; ++kk)
-            umma_bf16_ts(tmem + 256 + HD, tmem + 128 + a_col(kk), bq + step_mn(kk), IDESC_G, (it > w.it0 || kk > 0) ? 1u : 0u);
-          if (last) umma_commit(bar_mma2);
+            umma_bf16_ts(tmem + 256 + HD, tmem + 128 + a_col(kk), bq + step_mn(kk), IDESC_G,
+                         (it > w.it0 || kk > 0) ? 1u : 0u);
+          if (last) umma_commit(bars + B_MMA2);
         }
         __syncwarp();
-        if (!last) scores(1 - b);
+        // (S^T overwrites the P^T that dV has read)
+        if (!last && mbar_wait_warp(bars + B_DV, tr.parity(B_DV))) {
+          tc_fence_after();
+          tr.arm(B_S);
+          if (elect_one()) scores(1 - b, 0);
+          __syncwarp();
+        }
       }
+      if (!last) tr.waited(B_DV);  // it is complete once the next S^T is
       // (its segment: two dependent loads, while the products run)
       if (it == w.it0 && unn >= 0) wnn = unit_t(unn, tnn);
       if (last) {
@@ -549,11 +547,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
           const int32_t* gp = qh == 0 ? gpos : gpos2;
           rope_load<HD>(rrow, rope_tab + (int64_t)(gp ? __ldg(gp + w.seg0 + k) : k) * E);
         }
-        if (!track_wait_all(bar_mma2, tm2)) {
-          if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
-          ok = false;
-          break;
-        }
+        if (!wait_all(B_MMA2, FL_DEV_TIMEOUT_ACC_EMPTY)) break;
         tc_fence_after();
         // this pair's last use in the unit: the next unit's tile of the pair
         if (warp == 0 && next && wn.it0 + b < wn.it_end) issue_q(wn, wn.it0 + b, b);
@@ -643,15 +637,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     un = unn;
   }
   if (tid == 0) bulk_wait_all();  // this CTA's bulk stores are complete before it leaves
-  if (!ok && tid == 0) {  // a wait gave up: let what this CTA armed land before leaving
-    track_drain(bar_kv, tkv);
-    track_drain(bar_q, tq0);
-    track_drain(bar_q + 1, tq1);
-    track_drain(bar_s, ts);
-    track_drain(bar_dp, tdp);
-    track_drain(bar_mma2, tm2);
-    track_drain(bar_clc, tclc);
-  }
+  if (!ok && tid == 0) track_drain(bars, BARS, tr);  // a wait gave up: let what this CTA armed land before leaving
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -681,12 +667,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   uint8_t* sV = smem + 4 * TILE;  // [2]
   uint8_t* sST = smem + 6 * TILE;  // staging of the bf16 output rows
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 7 * TILE + 2 * TB * 4);
-  uint64_t* bar_qdo = bars;
-  uint64_t* bar_kv = bars + 1;  // [2]
-  uint64_t* bar_s = bars + 3;
-  uint64_t* bar_dp = bars + 4;
-  uint64_t* bar_mma2 = bars + 5;
-  uint64_t* bar_clc = bars + 6;
+  enum { B_QDO = 0, B_KV = 1 /* and 2 */, B_S = 3, B_DP = 4, B_MMA2 = 5, B_CLC = 6, BARS = 7 };
   uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // [2] the unit taken over, requests alternate
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 12);
 
@@ -724,7 +705,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   };
 
   if (tid == 0) {
-    for (int i = 0; i < 7; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < BARS; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
     tma_prefetch_desc(&tm_do);
@@ -739,61 +720,64 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(quarter * 32) << 16);
 
-  BarTrack tqdo, tkv0, tkv1, ts, tdp, tm2, tclc;
+  BarTracks tr;
+  bool ok = true;
+  // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
+  auto wait_all = [&](int i, int code) {
+    ok = track_wait_all(bars, i, tr);
+    if (!ok && tid == 0) report_status(status, code);
+    return ok;
+  };
   // Copies and products are issued by warp 0 as a whole, as in the dK / dV kernel.
   auto issue_kv = [&](const Unit& w, int j, int b) {  // K_j, V_j into pair b
-    (b ? tkv1 : tkv0).pend = true;
+    tr.arm(B_KV + b);
     __syncwarp();
     if (!elect_one()) return;
-    mbar_arrive_expect_tx(bar_kv + b, 2 * TILE);
+    mbar_arrive_expect_tx(bars + B_KV + b, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
       if (j < npt) {
-        tma_load_2d(sK + b * TILE + x * BOX, &tm_pk, bar_kv + b, w.h * HD + 64 * x, 0);
-        tma_load_2d(sV + b * TILE + x * BOX, &tm_pv, bar_kv + b, w.h * HD + 64 * x, 0);
+        tma_load_2d(sK + b * TILE + x * BOX, &tm_pk, bars + B_KV + b, w.h * HD + 64 * x, 0);
+        tma_load_2d(sV + b * TILE + x * BOX, &tm_pv, bars + B_KV + b, w.h * HD + 64 * x, 0);
       } else {
         const int row = w.seg0 + (j - npt) * TB;
-        tma_load_2d(sK + b * TILE + x * BOX, &tm_qkv, bar_kv + b, H + w.h * HD + 64 * x, row);
-        tma_load_2d(sV + b * TILE + x * BOX, &tm_qkv, bar_kv + b, 2 * H + w.h * HD + 64 * x, row);
+        tma_load_2d(sK + b * TILE + x * BOX, &tm_qkv, bars + B_KV + b, H + w.h * HD + 64 * x, row);
+        tma_load_2d(sV + b * TILE + x * BOX, &tm_qkv, bars + B_KV + b, 2 * H + w.h * HD + 64 * x, row);
       }
     }
   };
   auto issue_qdo = [&](const Unit& w) {  // the unit's Q and dO
-    tqdo.pend = true;
+    tr.arm(B_QDO);
     __syncwarp();
     if (!elect_one()) return;
-    mbar_arrive_expect_tx(bar_qdo, 2 * TILE);
+    mbar_arrive_expect_tx(bars + B_QDO, 2 * TILE);
 #pragma unroll
     for (int x = 0; x < NB; ++x) {
-      tma_load_2d(sQ + x * BOX, &tm_qkv, bar_qdo, w.h * HD + 64 * x, w.seg0 + w.q0);
-      tma_load_2d(sdO + x * BOX, &tm_do, bar_qdo, w.h * HD + 64 * x, w.seg0 + w.q0);
+      tma_load_2d(sQ + x * BOX, &tm_qkv, bars + B_QDO, w.h * HD + 64 * x, w.seg0 + w.q0);
+      tma_load_2d(sdO + x * BOX, &tm_do, bars + B_QDO, w.h * HD + 64 * x, w.seg0 + w.q0);
     }
   };
 
+  constexpr uint32_t T_DS = 256 + HD;  // dS (64 columns)
   constexpr uint32_t IDESC_S = umma_idesc_bf16(TB, TB, false, false);
   constexpr uint32_t IDESC_G = umma_idesc_bf16(TB, HD, false, true);
-  bool ok = true;
   // Units: CTA c walks c, + gridDim.x, ..., or, when the grid has one CTA per unit, the hardware
   // hands them out: the resident CTA takes over the next one that has not started, two units ahead
   // of its work.  A request is written to the answer slot that the one before it left alone: that one
   // may still be being read, while the slot's own last answer was read before the wait in between.
   const bool handed = (int)gridDim.x == n_units;
-  int u_next = blockIdx.x;
   auto take = [&]() {
     if (!handed) return;
-    tclc.pend = true;
+    tr.arm(B_CLC);
     __syncwarp();
-    if (elect_one()) clc_request(clc + (tclc.done & 1), bar_clc);
+    if (elect_one()) clc_request(clc + tr.parity(B_CLC), bars + B_CLC);
   };
-  auto taken = [&](int& x) {  // the unit taken, or -1
+  auto taken = [&](int u, int& x) {  // the unit after unit u, or -1
     if (!handed) {
-      u_next += gridDim.x;
-      x = u_next < n_units ? u_next : -1;
+      x = u + (int)gridDim.x < n_units ? u + gridDim.x : -1;
       return true;
     }
-    ok = track_wait_all(bar_clc, tclc);
-    if (!ok && tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-    x = ok ? clc_answer(clc + ((tclc.done & 1) ^ 1)) : -1;
+    x = wait_all(B_CLC, FL_DEV_TIMEOUT_FULL) ? clc_answer(clc + (tr.parity(B_CLC) ^ 1)) : -1;
     return ok;
   };
   Unit w = unit(blockIdx.x), wn = Unit{};
@@ -807,7 +791,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     take();
   }
   int un;
-  if (taken(un) && un >= 0) wn = unit(un);
+  if (taken(blockIdx.x, un) && un >= 0) wn = unit(un);
   while (ok) {
     const int q = w.q0 + r;
     const bool q_ok = q < w.L;
@@ -819,31 +803,23 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     int unn = -1;
     uint32_t tnn = 0;
     if (next && warp == 0) take();
-    // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
-    if (!track_wait_all(bar_qdo, tqdo)) {
-      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-      ok = false;
-      break;
-    }
+    if (!wait_all(B_QDO, FL_DEV_TIMEOUT_FULL)) break;
     auto scores = [&](int b) {  // warp 0: S = Q K^T and dP = dO V^T of the tile in pair b
-      ts.pend = tdp.pend = true;
+      tr.arm(B_S);
+      tr.arm(B_DP);
       if (elect_one()) {
         const uint64_t aq = desc_k(smem_u32(sQ)), ao = desc_k(smem_u32(sdO)), bk = desc_k(smem_u32(sK + b * TILE)),
                        bv = desc_k(smem_u32(sV + b * TILE));
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, aq + step_k(kk), bk + step_k(kk), IDESC_S, kk > 0);
-        umma_commit(bar_s);
+        umma_commit(bars + B_S);
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128, ao + step_k(kk), bv + step_k(kk), IDESC_S, kk > 0);
-        umma_commit(bar_dp);
+        umma_commit(bars + B_DP);
       }
       __syncwarp();
     };
-    if (!track_wait_all(bar_kv, tkv0)) {
-      if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-      ok = false;
-      break;
-    }
+    if (!wait_all(B_KV, FL_DEV_TIMEOUT_FULL)) break;
     if (warp == 0) {
       tc_fence_after();
       scores(0);
@@ -851,11 +827,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     for (int j = 0; j < w.n_kv && ok; ++j) {
       const int b = j & 1;
       const bool last = j + 1 == w.n_kv;
-      if (!track_wait_all(bar_s, ts)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
-        ok = false;
-        break;
-      }
+      if (!wait_all(B_S, FL_DEV_TIMEOUT_ACC_FULL)) break;
       tc_fence_after();
       // S is complete and so is every product issued before it: the other buffer pair is free for
       // the next tile (the second tile of a unit was loaded at the end of the unit before)
@@ -888,18 +860,14 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
       if (open) probs(std::false_type{});
       else probs(std::true_type{});
       if (j == 0 && next) {
-        if (!taken(unn)) break;
+        if (!taken(un, unn)) break;
         if (unn >= 0) tnn = tiles[unn / nh];
       }
       tc_fence_before();
-      if (!track_wait_all(bar_dp, tdp)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
-        ok = false;
-        break;
-      }
+      if (!wait_all(B_DP, FL_DEV_TIMEOUT_ACC_FULL)) break;
       tc_fence_after();
       if (warp == 0 && next && last) issue_qdo(wn);
-      // ---- dS, written (bf16 pairs) into the 16 S columns at 64 kh + 16 hf
+      // ---- dS, written (bf16 pairs) into the 16 columns at 32 kh + 16 hf of its own
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         uint32_t dr[32];
@@ -910,30 +878,25 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
         for (int c2 = 0; c2 < 16; ++c2)
           dd[c2] = pack_bf16x2(p[32 * hf + 2 * c2] * (__uint_as_float(dr[2 * c2]) - dl),
                                p[32 * hf + 2 * c2 + 1] * (__uint_as_float(dr[2 * c2 + 1]) - dl));
-        tmem_st16(t_lane + kh * 64 + 16 * hf, dd);
+        tmem_st16(t_lane + T_DS + kh * 32 + 16 * hf, dd);
       }
       tmem_st_wait();
       tc_fence_before();
       // the next tile's K and V have landed (and every thread has written its dS)
       if (last) {
         __syncthreads();
-      } else if (!track_wait_all(bar_kv + 1 - b, b ? tkv0 : tkv1)) {
-        if (tid == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
-        ok = false;
-        break;
-      }
-      // ---- dQ += dS K_j (A from TMEM), and the next tile's scores behind it (they overwrite dS,
-      // which the product before them in the tensor pipe has read)
+      } else if (!wait_all(B_KV + 1 - b, FL_DEV_TIMEOUT_FULL)) break;
+      // ---- dQ += dS K_j (A from TMEM), and the next tile's scores behind it
       if (warp == 0) {
         tc_fence_after();
-        if (last) tm2.pend = true;
+        if (last) tr.arm(B_MMA2);
         __syncwarp();
         if (elect_one()) {
           const uint64_t bk = desc_mn(smem_u32(sK + b * TILE));
 #pragma unroll
           for (int kk = 0; kk < TB / 16; ++kk)
-            umma_bf16_ts(tmem + 256, tmem + a_col(kk), bk + step_mn(kk), IDESC_G, (j > 0 || kk > 0) ? 1u : 0u);
-          if (last) umma_commit(bar_mma2);
+            umma_bf16_ts(tmem + 256, tmem + T_DS + 8 * kk, bk + step_mn(kk), IDESC_G, (j > 0 || kk > 0) ? 1u : 0u);
+          if (last) umma_commit(bars + B_MMA2);
         }
         __syncwarp();
         if (!last) scores(1 - b);
@@ -945,11 +908,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
           const int32_t* gp = kh == 0 ? gpos : gpos2;
           rope_load<HD>(rrow, rope_tab + (int64_t)(gp ? __ldg(gp + w.seg0 + q) : q) * E);
         }
-        if (!track_wait_all(bar_mma2, tm2)) {
-          if (tid == 0) report_status(status, FL_DEV_TIMEOUT_ACC_EMPTY);
-          ok = false;
-          break;
-        }
+        if (!wait_all(B_MMA2, FL_DEV_TIMEOUT_ACC_EMPTY)) break;
         tc_fence_after();
         // this pair's last use in the unit: the next unit's tile of the pair
         if (warp == 0 && next && b < wn.n_kv) issue_kv(wn, b, b);
@@ -1015,15 +974,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     dl = dln;
   }
   if (tid == 0) bulk_wait_all();  // this CTA's bulk stores are complete before it leaves
-  if (!ok && tid == 0) {  // a wait gave up: let what this CTA armed land before leaving
-    track_drain(bar_qdo, tqdo);
-    track_drain(bar_kv, tkv0);
-    track_drain(bar_kv + 1, tkv1);
-    track_drain(bar_s, ts);
-    track_drain(bar_dp, tdp);
-    track_drain(bar_mma2, tm2);
-    track_drain(bar_clc, tclc);
-  }
+  if (!ok && tid == 0) track_drain(bars, BARS, tr);  // a wait gave up: let what this CTA armed land before leaving
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {

@@ -8,11 +8,11 @@
 //   TMA: K_j and V_j (128 rows x head_dim, 64-column 128-byte-swizzled boxes; Q once),
 //        each on its own barrier;
 //   S = Q K_j^T     -> TMEM columns [0, 128)   (tcgen05.mma, both operands in shared memory),
-//        issued right behind the P V of the tile before it; once it is complete, so is that
-//        P V, and K_(j+1) (after a unit's last tile the next unit's Q and K) and V_j are loaded;
+//        issued once the P V of the tile before it has read a P there; once S is complete, K_(j+1)
+//        (after a unit's last tile the next unit's Q and K) and V_j are loaded;
 //   softmax: the thread's S row (masked max, exp2, row sum); P (bf16, two per 32-bit
-//        column) is stored back into the first 64 columns of S; the O row is rescaled when
-//        the running max moved;
+//        column) is stored back into the first 64 columns of S (head_dim 64: into the last 64 of
+//        the CTA's); the O row is rescaled when the running max moved;
 //   O += P V_j      -> TMEM columns [128, 128 + head_dim) (A = P read from TMEM, V_j as an
 //        MN-major operand).
 // The next unit's first scores run while a unit's output is written.
@@ -68,6 +68,8 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
     const uint32_t* __restrict__ tiles, int n_units, bf16* __restrict__ O, float* __restrict__ lse,
     float scale_log2, int Lp, const int32_t* __restrict__ ctxs, int* status) {
   constexpr int NB = FwdCfg<HD>::NB, TILE = FwdCfg<HD>::TILE;
+  // P's 64 columns: the last ones at head_dim 64, the first of S at 128, where O fills the others
+  constexpr uint32_t T_P = HD == 64 ? 192 : 0;
   pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
   pdl_trigger();
   extern __shared__ uint8_t smem_raw[];
@@ -76,11 +78,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   uint8_t* sK = smem + TILE;
   uint8_t* sV = smem + 2 * TILE;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 3 * TILE);
-  uint64_t* bar_q = bars;
-  uint64_t* bar_k = bars + 1;
-  uint64_t* bar_v = bars + 2;
-  uint64_t* bar_s = bars + 3;
-  uint64_t* bar_pv = bars + 4;
+  enum { B_Q = 0, B_K = 1, B_V = 2, B_S = 3, B_PV = 4, BARS = 5 };
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int npt = Lp > 0 ? 1 : 0;  // at most one prefix tile (Lp <= 128)
@@ -105,7 +103,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   auto unit = [&](int u) { return unit_t(u, tiles[u / n_heads]); };
 
   if (tid == 0) {
-    for (int i = 0; i < 5; ++i) mbar_init(bars + i, 1);
+    for (int i = 0; i < BARS; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_qkv);
   }
@@ -118,16 +116,16 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   tc_fence_after();
   const uint32_t tmem = *holder;
   const uint32_t t_lane = tmem + (uint32_t(warp * 32) << 16);  // this warp's TMEM lanes
-  const uint32_t t_s = t_lane, t_o = t_lane + 128;
+  const uint32_t t_s = t_lane, t_o = t_lane + 128, t_p = t_lane + T_P;
 
-  BarTrack tq, tk, tv, ts, tpv;
+  BarTracks tr;
   // Copies and products are issued by warp 0 as a whole, one elected lane at work: the
   // instructions' operands stay in uniform registers.
   // the key (part 0) or value (part 1) tile j of unit w into its buffer
   auto issue = [&](const Unit& w, int j, int part) {
     uint8_t* dst = part ? sV : sK;
-    uint64_t* bar = part ? bar_v : bar_k;
-    (part ? tv : tk).pend = true;
+    uint64_t* bar = bars + (part ? B_V : B_K);
+    tr.arm(part ? B_V : B_K);
     __syncwarp();
     if (!elect_one()) return;
     mbar_arrive_expect_tx(bar, TILE);
@@ -143,35 +141,35 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
     }
   };
   auto issue_q = [&](const Unit& w) {
-    tq.pend = true;
+    tr.arm(B_Q);
     __syncwarp();
     if (!elect_one()) return;
-    mbar_arrive_expect_tx(bar_q, TILE);
+    mbar_arrive_expect_tx(bars + B_Q, TILE);
 #pragma unroll
-    for (int b = 0; b < NB; ++b) tma_load_2d(sQ + b * BOX, &tm_qkv, bar_q, w.h * HD + 64 * b, w.seg0 + w.q0);
+    for (int b = 0; b < NB; ++b) tma_load_2d(sQ + b * BOX, &tm_qkv, bars + B_Q, w.h * HD + 64 * b, w.seg0 + w.q0);
   };
 
   constexpr uint32_t IDESC_S = umma_idesc_bf16(TB, TB, false, false);
   constexpr uint32_t IDESC_PV = umma_idesc_bf16(TB, HD, false, true);
   auto score = [&]() {  // warp 0: S = Q K^T of the tiles in place
     tc_fence_after();
-    ts.pend = true;
+    tr.arm(B_S);
     __syncwarp();
     if (elect_one()) {
       const uint64_t aq = desc_kmajor(smem_u32(sQ)), bk = desc_kmajor(smem_u32(sK));
 #pragma unroll
       for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem, aq + step_kmajor(kk), bk + step_kmajor(kk), IDESC_S, kk > 0);
-      umma_commit(bar_s);
+      umma_commit(bars + B_S);
     }
     __syncwarp();
   };
   // every wait's outcome is agreed on by the whole CTA, so that all threads leave together
-  auto wait_all = [&](uint64_t* bar, BarTrack& t, int code) {
-    const bool good = track_wait_all(bar, t);
-    if (!good && tid == 0) report_status(status, code);
-    return good;
-  };
   bool ok = true;
+  auto wait_all = [&](int i, int code) {
+    ok = track_wait_all(bars, i, tr);
+    if (!ok && tid == 0) report_status(status, code);
+    return ok;
+  };
   int u = blockIdx.x;
   Unit w = u < n_units ? unit(u) : Unit{};
   Unit wn = u + (int)gridDim.x < n_units ? unit(u + gridDim.x) : Unit{};
@@ -181,7 +179,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
       issue(w, 0, 0);
       issue(w, 0, 1);
     }
-    ok = wait_all(bar_q, tq, FL_DEV_TIMEOUT_FULL) && wait_all(bar_k, tk, FL_DEV_TIMEOUT_FULL);
+    wait_all(B_Q, FL_DEV_TIMEOUT_FULL) && wait_all(B_K, FL_DEV_TIMEOUT_FULL);
     if (ok && warp == 0) score();
   }
   while (u < n_units && ok) {  // the unit's first scores have been issued
@@ -197,7 +195,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
       if (j == 0 && unn < n_units) tnn = tiles[unn / n_heads];
       // ---- S_j is complete, and so is the P V before it: K_j (after the last tile Q too) and
       // V_(j-1) have been read
-      if (!(ok = wait_all(bar_s, ts, FL_DEV_TIMEOUT_ACC_FULL))) break;
+      if (!wait_all(B_S, FL_DEV_TIMEOUT_ACC_FULL)) break;
       tc_fence_after();
       if (warp == 0) {
         if (j > 0) issue(w, j, 1);
@@ -239,8 +237,8 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
         lt += p0 + p1;
         r[c] = pack_bf16x2(p0, p1);
       }
-      tmem_st32(t_s, *reinterpret_cast<uint32_t(*)[32]>(r));
-      tmem_st32(t_s + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
+      tmem_st32(t_p, *reinterpret_cast<uint32_t(*)[32]>(r));
+      tmem_st32(t_p + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
       l_run = l_run * corr + lt;
       m_run = m_new;
       // ---- rescale the O rows when a row max moved (not before the first P V); TMEM
@@ -259,30 +257,32 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
       if (j == 0 && unn < n_units) wnn = unit_t(unn, tnn);
       tmem_st_wait();
       tc_fence_before();
-      if (!(ok = wait_all(bar_v, tv, FL_DEV_TIMEOUT_FULL))) break;
+      if (!wait_all(B_V, FL_DEV_TIMEOUT_FULL)) break;
       // ---- O += P V_j
       if (warp == 0) {
         tc_fence_after();
-        if (last) tpv.pend = true;
+        tr.arm(B_PV);
         __syncwarp();
         if (elect_one()) {
           const uint64_t bv = desc_mnmajor(smem_u32(sV));
 #pragma unroll
           for (int kk = 0; kk < TB / 16; ++kk)
-            umma_bf16_ts(tmem + 128, tmem + kk * 8, bv + step_mnmajor(kk), IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u);
-          if (last) umma_commit(bar_pv);
+            umma_bf16_ts(tmem + 128, tmem + T_P + kk * 8, bv + step_mnmajor(kk), IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(bars + B_PV);
         }
         __syncwarp();
       }
-      // ---- the next scores behind it in the tensor pipe (they overwrite P, which it has read):
-      // this unit's next tile, or the next unit's first, whose product runs under this epilogue
+      // ---- the next scores: this unit's next tile, or the next unit's first, whose product runs
+      // under this epilogue.  Where they overwrite the P that P V reads the issuing warp waits for P V
+      // first: PTX orders products only among those of one shape and accumulator
       if (!last || next) {
-        if (last && !(ok = wait_all(bar_q, tq, FL_DEV_TIMEOUT_FULL))) break;
-        if (!(ok = wait_all(bar_k, tk, FL_DEV_TIMEOUT_FULL))) break;
-        if (warp == 0) score();
+        if (last && !wait_all(B_Q, FL_DEV_TIMEOUT_FULL)) break;
+        if (!wait_all(B_K, FL_DEV_TIMEOUT_FULL)) break;
+        if (warp == 0 && (T_P != 0 || mbar_wait_warp(bars + B_PV, tr.parity(B_PV)))) score();
       }
+      if (!last) tr.waited(B_PV);  // it is complete once the next S is
     }
-    if (!ok || !(ok = wait_all(bar_pv, tpv, FL_DEV_TIMEOUT_ACC_EMPTY))) break;
+    if (!ok || !wait_all(B_PV, FL_DEV_TIMEOUT_ACC_EMPTY)) break;
     tc_fence_after();
     if (warp == 0 && next) issue(wn, 0, 1);  // the unit's last V has been read
     // ---- O / l and the log-sum-exp (every lane reads TMEM, all of the row at once; rows
@@ -318,13 +318,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
     w = wn;
     wn = wnn;
   }
-  if (!ok && tid == 0) {  // a wait gave up: let what this CTA armed land before leaving
-    track_drain(bar_q, tq);
-    track_drain(bar_k, tk);
-    track_drain(bar_v, tv);
-    track_drain(bar_s, ts);
-    track_drain(bar_pv, tpv);
-  }
+  if (!ok && tid == 0) track_drain(bars, BARS, tr);  // a wait gave up: let what this CTA armed land before leaving
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {

@@ -37,8 +37,26 @@ def test_launch_control_answers_alternate():
         slots = int(re.search(r"holder = reinterpret_cast<uint32_t\*>\(bars \+ (\d+)\)", body).group(1)) - \
             int(re.search(r"clc = reinterpret_cast<uint4\*>\(bars \+ (\d+)\)", body).group(1))
         assert slots == 4  # two answers of 16 bytes
-        # `done` counts the answers waited for: n when request n is made, n + 1 when its answer is read
-        assert re.findall(r"clc_request\((.*), bar_clc\)", body) == ["clc + (tclc.done & 1)"]
-        assert re.findall(r"clc_answer\((.*)\) : -1", body) == ["clc + ((tclc.done & 1) ^ 1)"]
-        taken = body[body.index("auto taken"):]
-        assert taken.index("track_wait_all(bar_clc, tclc)") < taken.index("clc_answer")
+        # the parity of the answers waited for: n % 2 when request n is made, (n + 1) % 2 when its answer is read
+        assert re.findall(r"clc_request\((.*), bars \+ B_CLC\)", body) == ["clc + tr.parity(B_CLC)"]
+        assert re.findall(r"wait_all\(B_CLC, .*?\) \? clc_answer\((.*)\) : -1", body) == ["clc + (tr.parity(B_CLC) ^ 1)"]
+
+
+def test_products_wait_for_the_readers_of_their_columns():
+    """Attention: a score product whose TMEM columns hold an operand of a product in flight is issued
+    behind a wait for it (PTX orders only products of one shape and accumulator).  Forward: the next
+    S over the P that P V reads; backward: S^T over the P^T that dV reads, dP^T over the dS^T that
+    dK reads (behind the next S^T, committed after dK); dQ's dS has columns of its own."""
+    fwd = _kernel(_code("attention_tc.cu"), "attn_fwd_tc_kernel")
+    p_over_s = re.search(r"T_P = HD == 64 \? 192 : 0;", fwd)
+    assert p_over_s and "if (warp == 0 && (T_P != 0 || mbar_wait_warp(bars + B_PV, tr.parity(B_PV)))) score();" in fwd
+    src = _code("attention_bwd_tc.cu")
+    dkv = _kernel(src, "attn_bwd_dkv_tc_kernel")
+    loop = dkv[dkv.index("for (int it = w.it0"):]
+    # in the loop: dP^T behind the CTA-wide wait for S^T, S^T behind the wait for dV
+    assert loop.index("wait_all(B_S,") < loop.index("scores(b, 1)") < loop.index("scores(1 - b, 0)")
+    assert loop.index("mbar_wait_warp(bars + B_DV, tr.parity(B_DV))") < loop.index("scores(1 - b, 0)")
+    assert len(re.findall(r"\bscores\(", loop)) == 2
+    dq = _kernel(src, "attn_bwd_dq_tc_kernel")
+    assert "T_DS = 256 + HD;" in dq
+    assert re.findall(r"umma_bf16_ts\(tmem \+ 256, (.*?), bk", dq) == ["tmem + T_DS + 8 * kk"]
