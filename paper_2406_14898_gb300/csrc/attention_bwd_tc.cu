@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   float* sL = reinterpret_cast<float*>(smem + 7 * TILE);  // [128] lse * log2e of the query tile
   float* sD = sL + TB;                                    // [128] delta of the query tile
   uint64_t* bars = reinterpret_cast<uint64_t*>(sD + TB);
-  enum { B_KV = 0, B_Q = 1 /* and 2 */, B_S = 3, B_DP = 4, B_MMA2 = 5, B_CLC = 6, B_DV = 7, BARS = 8 };
+  enum { B_KV = 0, B_Q = 1 /* and 2 */, B_S = 3, B_DP = 4, B_MMA2 = 5, B_CLC = 6, B_END = 7, B_DV = 8, BARS = 9 };
   uint4* clc = reinterpret_cast<uint4*>(bars + 10);  // [2] the unit taken over, requests alternate
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 14);
 
@@ -637,7 +637,11 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     un = unn;
   }
   if (tid == 0) bulk_wait_all();  // this CTA's bulk stores are complete before it leaves
-  if (!ok && tid == 0) track_drain(bars, BARS, tr);  // a wait gave up: let what this CTA armed land before leaving
+  if (!ok && warp == 0) {  // a wait gave up: let what this CTA issued and armed end before leaving
+    if (elect_one()) umma_commit(bars + B_END);
+    mbar_wait_warp(bars + B_END, 0);
+  }
+  if (!ok && tid == 0) track_drain(bars, BARS, tr);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -667,7 +671,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
   uint8_t* sV = smem + 4 * TILE;  // [2]
   uint8_t* sST = smem + 6 * TILE;  // staging of the bf16 output rows
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 7 * TILE + 2 * TB * 4);
-  enum { B_QDO = 0, B_KV = 1 /* and 2 */, B_S = 3, B_DP = 4, B_MMA2 = 5, B_CLC = 6, BARS = 7 };
+  enum { B_QDO = 0, B_KV = 1 /* and 2 */, B_S = 3, B_DP = 4, B_MMA2 = 5, B_CLC = 6, B_END = 7, BARS = 8 };
   uint4* clc = reinterpret_cast<uint4*>(bars + 8);  // [2] the unit taken over, requests alternate
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 12);
 
@@ -974,7 +978,11 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dq_tc_kernel(
     dl = dln;
   }
   if (tid == 0) bulk_wait_all();  // this CTA's bulk stores are complete before it leaves
-  if (!ok && tid == 0) track_drain(bars, BARS, tr);  // a wait gave up: let what this CTA armed land before leaving
+  if (!ok && warp == 0) {  // a wait gave up: let what this CTA issued and armed end before leaving
+    if (elect_one()) umma_commit(bars + B_END);
+    mbar_wait_warp(bars + B_END, 0);
+  }
+  if (!ok && tid == 0) track_drain(bars, BARS, tr);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {

@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   uint8_t* sK = smem + TILE;
   uint8_t* sV = smem + 2 * TILE;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 3 * TILE);
-  enum { B_Q = 0, B_K = 1, B_V = 2, B_S = 3, B_PV = 4, BARS = 5 };
+  enum { B_Q = 0, B_K = 1, B_V = 2, B_S = 3, B_PV = 4, B_END = 5, BARS = 6 };
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 6);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int npt = Lp > 0 ? 1 : 0;  // at most one prefix tile (Lp <= 128)
@@ -318,7 +318,11 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
     w = wn;
     wn = wnn;
   }
-  if (!ok && tid == 0) track_drain(bars, BARS, tr);  // a wait gave up: let what this CTA armed land before leaving
+  if (!ok && warp == 0) {  // a wait gave up: let what this CTA issued and armed end before leaving
+    if (elect_one()) umma_commit(bars + B_END);
+    mbar_wait_warp(bars + B_END, 0);
+  }
+  if (!ok && tid == 0) track_drain(bars, BARS, tr);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {

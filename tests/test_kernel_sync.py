@@ -60,3 +60,15 @@ def test_products_wait_for_the_readers_of_their_columns():
     dq = _kernel(src, "attn_bwd_dq_tc_kernel")
     assert "T_DS = 256 + HD;" in dq
     assert re.findall(r"umma_bf16_ts\(tmem \+ 256, (.*?), bk", dq) == ["tmem + T_DS + 8 * kk"]
+
+
+def test_given_up_waits_end_behind_every_product():
+    """Attention: when a wait gave up, the issuing warp commits once more and waits for it before the
+    CTA frees its TMEM, so that no product (committed before or not) is still at work on it."""
+    kernels = [("attention_tc.cu", "attn_fwd_tc_kernel"), ("attention_bwd_tc.cu", "attn_bwd_dkv_tc_kernel"),
+               ("attention_bwd_tc.cu", "attn_bwd_dq_tc_kernel")]
+    for name, kernel in kernels:
+        body = _kernel(_code(name), kernel)
+        end = re.search(r"if \(!ok && warp == 0\) \{\s*if \(elect_one\(\)\) umma_commit\(bars \+ B_END\);\s*"
+                        r"mbar_wait_warp\(bars \+ B_END, 0\);\s*\}", body)
+        assert end and max(m.start() for m in re.finditer(r"umma_bf16", body)) < end.start() < body.index("tmem_dealloc")
