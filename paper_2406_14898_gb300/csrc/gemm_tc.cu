@@ -188,6 +188,7 @@ Epi make_epi(const fl_gemm_args* a) {
   e.b1 = a->beta1;
   e.b2 = a->beta2;
   e.eps = a->eps;
+  e.den_scale = a->eps < 0x1p-100f ? 0x1p40f : 1.f;  // the square root alone is 0 or at least 2^-75
   e.wd = a->weight_decay;
   e.inv_bc1 = a->inv_bc1;
   e.inv_bc2 = a->inv_bc2;

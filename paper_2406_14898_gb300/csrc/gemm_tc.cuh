@@ -144,6 +144,7 @@ struct Epi {
   const float *ln_mean, *ln_rstd, *ln_gamma, *ln_beta;  // residual = LayerNorm(aux) when ln_mean
   float *adam_m, *adam_v;
   float lr, b1, b2, eps, wd, inv_bc1, inv_bc2;
+  float den_scale;  // power of two that keeps the AdamW denominator in div_nr's range
   float* colsum;  // GELU_BWD: column sums of D added here (bias gradient of the up-projection)
   // launch of several problems: element offsets of problem r's pointers from problem 0's
   // (entry 0 unused, always 0): D, aux, aux_out, bias / colsum, the per-row arrays (pos,
@@ -197,7 +198,8 @@ FL_DEV void st_quad(__nv_bfloat16* p, float4 v) {
 FL_DEV void adamw_update(const Epi& e, float g, float& w, float& m, float& v) {
   m = e.b1 * m + (1.f - e.b1) * g;
   v = e.b2 * v + (1.f - e.b2) * g * g;
-  w = w - e.lr * (div_nr(m * e.inv_bc1, sqrt_nr(v * e.inv_bc2) + e.eps) + e.wd * w);
+  const float d = (sqrt_nr(v * e.inv_bc2) + e.eps) * e.den_scale;
+  w = w - e.lr * (div_nr(m * e.inv_bc1, d) * e.den_scale + e.wd * w);
 }
 
 // Entry r of a per-problem offset array (constant indices only: no local copy of the

@@ -644,6 +644,36 @@ def test_gemm_fp32_gradient_bit_identical(F, M, N, K):
                 assert torch.equal(D[:, :, N:], D0[:, :, N:])
 
 
+@pytest.mark.parametrize("K", [64, 3072])
+@pytest.mark.parametrize("eps", [0.0, 1e-44, 1e-40, 1e-30])
+def test_gemm_adamw_epilogue_tiny_eps(F, K, eps):
+    """Denominators down to nothing: rows with a zero gradient and zero moments keep their weights
+    with any eps above 0 (0 / 0 without one), rows with an infinite one move by what the separate
+    kernel says, as do the others (two ulps of the update)."""
+    M, N = 256, 512
+    g = torch.Generator(device="cuda").manual_seed(K)
+    A = torch.randn((K, M), generator=g, device="cuda").bfloat16()
+    A[:, 16:48] = 0
+    A[:, 48:50] *= 1e-25                     # the squares underflow
+    B = torch.randn((K, N), generator=g, device="cuda").bfloat16()
+    w0 = 0.05 * torch.randn((M, N), generator=g, device="cuda")
+    m0 = torch.zeros((M, N), device="cuda")
+    m0[60, :8] = float("inf")
+    lr, b1, b2, wd = 1e-3, 0.9, 0.999, 0.01
+    grad = torch.zeros((M, N), device="cuda")
+    F.gemm(M, N, K, A, M, 1, B, N, 1, grad, N, epilogue=F.FL_EPI_STORE_F32)
+    wr, mr, vr, wbr = w0.clone(), m0.clone(), torch.zeros_like(w0), torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    F.fl_k_adamw(M * N, wr, grad.clone(), mr, vr, wbr, lr, b1, b2, eps, wd, 0.1, 0.001)
+    w, m, v, wb = w0.clone(), m0.clone(), torch.zeros_like(w0), torch.empty_like(wbr)
+    F.gemm(M, N, K, A, M, 1, B, N, 1, w, N, epilogue=F.FL_EPI_ADAMW, adam_m=m, adam_v=v, aux_out=wb, ld_aux_out=N,
+           lr=lr, beta1=b1, beta2=b2, eps=eps, weight_decay=wd, inv_bc1=1 / 0.1, inv_bc2=1 / 0.001)
+    torch.cuda.synchronize()
+    assert torch.equal(w.isnan(), wr.isnan()) and torch.equal(w.isinf(), wr.isinf())
+    assert bool(w[16:48].isnan().any()) == (eps == 0.0)
+    ok = wr.isfinite()
+    assert ((w - wr).abs()[ok] <= 2.0 ** -22 * ((w0 - wr).abs() + w0.abs())[ok]).all()
+
+
 @pytest.mark.parametrize("K", [8, 2048, 3064, 3072, 3080])
 def test_gemm_adamw_epilogue_against_exact(F, K):
     """The fused update on both sides of the contraction length where its epilogue changes,
