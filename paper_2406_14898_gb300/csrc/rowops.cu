@@ -523,7 +523,7 @@ struct CopyReg {
   }
 };
 
-// blockIdx.y = table entry, then one row of blocks for the zeros.  A thread has four groups in
+// blockIdx.y = table entry; the zeros are shared by the whole grid.  A thread has four groups in
 // flight when it scatters (3072 x 4096 fp32 -> bf16 15.6 -> 11.5 us, bf16 13.5 -> 8.3 on twice the
 // CTAs) and one when it gathers, which its fp32 stores bound (15.6 us against 18 with four).
 constexpr bool copy_scatters(int mode) { return mode == COPY_SCATTER_BF16 || mode == COPY_SCATTER_F32; }
@@ -532,23 +532,21 @@ FL_DEV void copy_clients(const CopyTable& tab) {
   constexpr int COPY_NV = copy_scatters(MODE) ? 4 : 1;
   const int e = blockIdx.y;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
-  if (e < tab.n) {
-    const int64_t n8 = tab.n8[e], off = tab.off8[e];
-    uint4* client = reinterpret_cast<uint4*>(tab.client[e]);
-    for (int64_t i0 = tid; i0 < n8; i0 += COPY_NV * nth) {
-      CopyReg<MODE> r[COPY_NV];
+  const int64_t n8 = tab.n8[e], off = tab.off8[e];
+  uint4* client = reinterpret_cast<uint4*>(tab.client[e]);
+  for (int64_t i0 = tid; i0 < n8; i0 += COPY_NV * nth) {
+    CopyReg<MODE> r[COPY_NV];
 #pragma unroll
-      for (int k = 0; k < COPY_NV; ++k)
-        if (i0 + k * nth < n8) r[k].load(tab, client, off, i0 + k * nth);
+    for (int k = 0; k < COPY_NV; ++k)
+      if (i0 + k * nth < n8) r[k].load(tab, client, off, i0 + k * nth);
 #pragma unroll
-      for (int k = 0; k < COPY_NV; ++k)
-        if (i0 + k * nth < n8) r[k].store(tab, client, off, i0 + k * nth);
-    }
-  } else if (e == tab.n) {
-    for (int z = 0; z < tab.n_zero; ++z)
-      for (int64_t i = tid; i < tab.zero_n / 4; i += nth)
-        reinterpret_cast<float4*>(tab.zero[z])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < COPY_NV; ++k)
+      if (i0 + k * nth < n8) r[k].store(tab, client, off, i0 + k * nth);
   }
+  const int64_t gtid = e * nth + tid, gnth = gridDim.y * nth;
+  for (int z = 0; z < tab.n_zero; ++z)
+    for (int64_t i = gtid; i < tab.zero_n / 4; i += gnth)
+      reinterpret_cast<float4*>(tab.zero[z])[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 template <int MODE>
 __global__ void __launch_bounds__(256) copy_clients_kernel(CopyTable tab) {
@@ -583,14 +581,15 @@ FL_DEV void write_meta(const MetaArgs& a, const MetaOut& o, int64_t tid, int64_t
     if (o.pos2) o.pos2[t] = p2;
   }
 }
-// The forward's first launch: the clients' states gathered (blockIdx.y < tab.n) and the call's
-// metadata written (the last row of blocks).
+// The forward's first launch: the clients' states gathered and the call's metadata written, by the
+// whole grid.
 __global__ void __launch_bounds__(256) gather_meta_kernel(const __grid_constant__ CopyTable tab,
                                                           const __grid_constant__ MetaArgs a, MetaOut o) {
   pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
   pdl_trigger();
-  if (blockIdx.y + 1 < gridDim.y) copy_clients<COPY_GATHER_F32>(tab);
-  else write_meta(a, o, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+  copy_clients<COPY_GATHER_F32>(tab);
+  const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+  write_meta(a, o, blockIdx.y * nth + blockIdx.x * (int64_t)blockDim.x + threadIdx.x, gridDim.y * nth);
 }
 
 // ------------------------------------------------------------------ seeded init
@@ -746,17 +745,19 @@ int fl_launch_adamw(int64_t n, float* w, float* g, float* m, float* v, void* w_b
 
 int fl_launch_copy_clients(const CopyTable& tab, cudaStream_t st, const MetaArgs* meta, const MetaOut* out) {
   if (tab.n <= 0) return FL_OK;
-  int64_t maxn = 0;
+  // a thread per unit of the longest entry, or of an entry's share of the zeros or the metadata, up to
+  // a few CTAs per SM over all entries
+  int64_t maxn = ((tab.n_zero > 0 ? tab.n_zero * (tab.zero_n / 4) : meta ? meta->cu[meta->S] : 0) + tab.n - 1) / tab.n;
   for (int e = 0; e < tab.n; ++e) maxn = tab.n8[e] > maxn ? tab.n8[e] : maxn;
   int gx = (int)((maxn + 255) / 256);
   const int cap = ((copy_scatters(tab.mode) ? 4 : 2) * sm_count() + tab.n - 1) / tab.n + 1;
   if (gx > cap) gx = cap;
   if (gx < 1) gx = 1;
   if (meta) {  // CopyTable and MetaArgs together stay below the 32 KB of kernel parameters
-    FL_CUDA_TRY(fl_launch(gather_meta_kernel, dim3(gx, tab.n + 1), dim3(256), 0, st, tab, *meta, *out));
+    FL_CUDA_TRY(fl_launch(gather_meta_kernel, dim3(gx, tab.n), dim3(256), 0, st, tab, *meta, *out));
     return FL_OK;
   }
-  const dim3 grid(gx, tab.n + (tab.n_zero > 0 ? 1 : 0));
+  const dim3 grid(gx, tab.n);
   switch (tab.mode) {
     case COPY_GATHER_BF16: FL_CUDA_TRY(fl_launch(copy_clients_kernel<COPY_GATHER_BF16>, grid, dim3(256), 0, st, tab)); break;
     case COPY_SCATTER_BF16: FL_CUDA_TRY(fl_launch(copy_clients_kernel<COPY_SCATTER_BF16>, grid, dim3(256), 0, st, tab)); break;

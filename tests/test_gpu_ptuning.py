@@ -75,3 +75,35 @@ def test_ptuning_parity(F, freeze, fused):
             else:
                 check_updated_weights(w, ref.params[b][t].reshape(-1), w0, gref[b][t], cfg.lr, (b, t))
     srv.close()
+
+
+@pytest.mark.parametrize("lens", [(1,) * 70, (3,), (130,) + (2,) * 63])
+def test_gather_clears_and_packs_with_any_grid(F, lens):
+    """The launches that gather the clients also write the packing metadata and clear the bias,
+    LayerNorm and prefix gradients, whatever grid the clients' rows ask for (many short ones, a
+    single tiny one, more than one launch holds): the states equal one client at a time, and the
+    gradients after a step equal those from before it (no update at a zero learning rate)."""
+    cfg = syn.CONFIGS["tiny"].with_(n_blocks=2, client_batch=1, seq_lens=lens, prefix_len=128)
+    srv = F.Server(F.make_cfg(cfg, cfg.tokens), cfg.seed)
+    g = torch.Generator(device="cuda").manual_seed(len(lens))
+    draw = lambda n: torch.randn((1, n, cfg.hidden), generator=g, device="cuda").bfloat16()
+    st, go = [draw(n) for n in lens], [draw(n) for n in lens]
+    vecs = [t for t in range(14) if t not in (F.FL_T_WQKV, F.FL_T_WDENSE, F.FL_T_WUP, F.FL_T_WDOWN)]
+    seen = []
+    for _ in range(2):
+        outs, gi = [torch.empty_like(x) for x in st], [torch.empty_like(x) for x in st]
+        srv.forward(st, lens, outs)
+        srv.backward(go, gi)
+        srv.sync()
+        seen.append([srv.get_grad(b, t) for b in range(2) for t in vecs])
+        srv.step(0.0)
+    for a, b in zip(*seen):  # sums over atomics: equal up to their order
+        np.testing.assert_allclose(a, b, rtol=0, atol=1e-5 * max(1e-30, np.abs(a).max()))
+    for k in {0, len(lens) // 2, len(lens) - 1}:
+        one = torch.empty_like(st[k])
+        srv.forward([st[k]], lens[k:k + 1], [one])
+        srv.backward([go[k]], [torch.empty_like(st[k])])
+        srv.sync()
+        assert torch.equal(one.view(torch.int16), outs[k].view(torch.int16)), k
+        srv.step(0.0)
+    srv.close()
