@@ -36,9 +36,8 @@
 // Bound by the latency of that chain, one CTA per SM (cycles of a unit of one tile: loads and
 // scores 2200, P 1100-1800, dS 1200, dK 850, output 4400).  A ninth warp to issue the products
 // (the issuer waits for room in the tensor pipe) left 168 registers a thread and spilled.
-// Against both passes in one behind a common barrier: segments of several tiles gain (4 x 2048 tokens
-// 809 -> 646 us), segments of one tile lose, in this kernel alone (64 x 128 tokens 197 -> 205 us for
-// the whole backward, 64 x 64 172 -> 180).
+// Against both passes in one behind a common barrier, segments of several tiles gain (4 x 2048 tokens
+// 809 -> 643 us); where every segment is one tile the one pass stays (ONE).
 // Epilogue: dK * scale, the inverse rotary rotation(s), bf16 rows of dqkv and the k / v
 // column sums for the QKV bias gradient; the prefix variant (PREFIX: the unit's keys are
 // the prefix of its head, its query tiles a slice of the call's tile list) adds dK * scale
@@ -182,7 +181,11 @@ FL_DEV void staged_colsum(uint8_t* stage, int rows, float* out, int tid) {
 // every query tile, first).
 // PREFIX: unit u = (slice u / nh of the tile list cut into slices of `per` tiles, head u % nh),
 // the unit's keys the Lp prefix keys of its head.  Every unit has a query tile.
-template <int HD, bool PREFIX>
+// ONE (not PREFIX): every segment, and so every unit, is one tile.  P^T and dS^T are then made in one
+// pass behind one wait: the split passes, which units of several tiles gain from, cost more than
+// they hide (whole backward, split / one pass: 64 x 128 tokens 209 / 198 us, 64 x 64 181 / 168, 12 x 100
+// 54 / 52).
+template <int HD, bool PREFIX, bool ONE>
 __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     const __grid_constant__ CUtensorMap tm_qkv, const __grid_constant__ CUtensorMap tm_do,
     const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
@@ -218,8 +221,14 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
   // a unit: its head, keys (segment start and length, first key kb), the last context key
   // of the segment (GLM; -1 when causal), its query tiles [it0, it_end), and the QKV bias
   // gradient of the segment's replica
-  struct Unit {
-    int h, seg0, L, kb, clast, it0, it_end;
+  struct Tiles {
+    int kb, it0, it_end;
+  };
+  struct OneTile {
+    enum { kb = 0, it0 = 0, it_end = 1 };
+  };
+  struct Unit : std::conditional_t<ONE, OneTile, Tiles> {
+    int h, seg0, L, clast;
     float* db;
   };
   auto unit_t = [&](int u, uint32_t t) {
@@ -235,12 +244,14 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       const int s = int(t >> 16), idx = int(t & 0xFFFFu);
       w.seg0 = cu[s];
       w.L = cu[s + 1] - w.seg0;
-      const int nq = (w.L + TB - 1) / TB;
-      const int kt = nq - 1 - idx;
-      w.kb = kt * TB;
       w.clast = (ctxs ? min(max(ctxs[s], 0), w.L) : 0) - 1;
-      w.it0 = w.kb <= w.clast ? 0 : kt;  // a tile holding context keys is seen by every query
-      w.it_end = nq;
+      if constexpr (!ONE) {
+        const int nq = (w.L + TB - 1) / TB;
+        const int kt = nq - 1 - idx;
+        w.kb = kt * TB;
+        w.it0 = w.kb <= w.clast ? 0 : kt;  // a tile holding context keys is seen by every query
+        w.it_end = nq;
+      }
       w.db = dbias ? dbias + (dbias_segs > 0 ? (int64_t)(s / dbias_segs) * dbias_rstride : 0) : nullptr;
     }
     return w;
@@ -375,12 +386,12 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       const uint64_t a = desc_k(smem_u32(part ? sV : sK)), q = desc_k(smem_u32((part ? sdO : sQ) + b * TILE));
 #pragma unroll
       for (int kk = 0; kk < HD / 16; ++kk) umma_bf16(tmem + 128 * part, a + step_k(kk), q + step_k(kk), IDESC_S, kk > 0);
-      umma_commit(bars + (part ? B_DP : B_S));
+      if (part || !ONE) umma_commit(bars + (part ? B_DP : B_S));
     };
     if (!wait_all(B_Q, FL_DEV_TIMEOUT_FULL)) break;
     if (warp == 0) {
       tc_fence_after();
-      tr.arm(B_S);
+      if (!ONE) tr.arm(B_S);
       tr.arm(B_DP);
       if (elect_one()) {
         scores(0, 0);
@@ -390,7 +401,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
     }
     for (int it = w.it0; it < w.it_end && ok; ++it) {
       const int b = (it - w.it0) & 1;
-      const bool last = it + 1 == w.it_end;
+      const bool last = ONE || it + 1 == w.it_end;
       int row0, qpos0, valid;
       qtile(w, it, row0, qpos0, valid);
       {  // lse and delta of the query tile (rows past its segment are never visible)
@@ -401,7 +412,7 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
       // while the products run: the next tile's statistics, the unit after next
       if (!last) pf = stat_of(w, it + 1);
       else if (next) pf = stat_of(wn, wn.it0);
-      if (!wait_all(B_S, FL_DEV_TIMEOUT_ACC_FULL)) break;
+      if (!wait_all(ONE ? B_DP : B_S, FL_DEV_TIMEOUT_ACC_FULL)) break;
       tc_fence_after();
       // S^T is complete and so is every product issued before it: the dS^T columns are free for the
       // dP^T of a tile after the first, and the other buffer pair for the next tile (the second tile
@@ -428,45 +439,6 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         qlim = key_ok ? min(w.L, q0 + 64) : q0;
         qfirst = k <= w.clast ? q0 : max(q0, k);
       }
-      // every key of the warp visible to all 64 queries: no masks
-      const bool open = __all_sync(0xffffffffu, qfirst <= q0 && qlim >= q0 + 64);
-      // ---- P^T of key row r for queries qh * 64 .. + 63, in two groups of 32, kept in registers
-      // and written (bf16 pairs) into the 16 columns at 64 qh + 16 hf of the S^T just read
-      float p[64];
-      auto probs = [&](auto masked) {
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          uint32_t sr[32];
-          tmem_ld32(t_lane + qh * 64 + 32 * hf, sr);
-          tmem_ld_wait();
-          const float4* L4 = reinterpret_cast<const float4*>(sL + qh * 64 + 32 * hf);
-          uint32_t pp[16];
-#pragma unroll
-          for (int c4 = 0; c4 < 8; ++c4) {
-            const float4 l4 = L4[c4];
-            const float lq[4] = {l4.x, l4.y, l4.z, l4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int c = 4 * c4 + e, q = q0 + 32 * hf + c;
-              const float pv = exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lq[e]));
-              p[32 * hf + c] = !masked.value || (q >= qfirst && q < qlim) ? pv : 0.f;
-            }
-            pp[2 * c4] = pack_bf16x2(p[32 * hf + 4 * c4], p[32 * hf + 4 * c4 + 1]);
-            pp[2 * c4 + 1] = pack_bf16x2(p[32 * hf + 4 * c4 + 2], p[32 * hf + 4 * c4 + 3]);
-          }
-          tmem_st16(t_lane + qh * 64 + 16 * hf, pp);
-        }
-      };
-      if (open) probs(std::false_type{});
-      else probs(std::true_type{});
-      if (it == w.it0 && next) {
-        if (!taken(un, unn)) break;
-        if (unn >= 0) tnn = tile_word(unn);
-      }
-      tmem_st_wait();
-      tc_fence_before();
-      if (!wait_all(B_DP, FL_DEV_TIMEOUT_ACC_FULL)) break;
-      tc_fence_after();
       auto add_dv = [&]() {
         if (elect_one()) {
           const uint64_t bo = desc_mn(smem_u32(sdO + b * TILE));
@@ -476,39 +448,116 @@ __global__ void __launch_bounds__(256, 1) attn_bwd_dkv_tc_kernel(
         }
         __syncwarp();
       };
-      // ---- dV += P^T dO (A from TMEM) while dS^T is made; the unit's last reader of K and V is done.
-      // A unit's last tile has no later products to make room for, and the issuing warp's dS^T would
-      // be what the others wait for: its dV goes with dK.  32 x 256 tokens 234 -> 228 us, 64 x 128 211 ->
-      // 205, 16 x 512 295 -> 288, segments of 67 to 2048 335 -> 329 (late on every tile: 234, 210, 296, 340).
-      if (warp == 0) {
-        if (last && next) issue_kv(wn);
-        __syncwarp();
-        if (!last) {
-          tr.arm(B_DV);
-          add_dv();
-          if (elect_one()) umma_commit(bars + B_DV);
+      if constexpr (ONE) {
+        // ---- P^T and dS^T of key row r, in two groups of 32 queries, each written (bf16 pairs) into the
+        // 16 columns at 64 qh + 16 hf of the values it has just read
+        if (warp == 0 && next) issue_kv(wn);  // the unit's last reader of K and V is done
+#pragma unroll 1
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t sr[32], dr[32];
+          tmem_ld32(t_lane + qh * 64 + 32 * hf, sr);
+          tmem_ld32(t_lane + 128 + qh * 64 + 32 * hf, dr);
+          tmem_ld_wait();
+          const float4* L4 = reinterpret_cast<const float4*>(sL + qh * 64 + 32 * hf);
+          const float4* D4 = reinterpret_cast<const float4*>(sD + qh * 64 + 32 * hf);
+          uint32_t pp[16], dd[16];
+#pragma unroll
+          for (int c4 = 0; c4 < 8; ++c4) {
+            const float4 l4 = L4[c4], d4 = D4[c4];
+            const float lq[4] = {l4.x, l4.y, l4.z, l4.w}, dq[4] = {d4.x, d4.y, d4.z, d4.w};
+            float p[4], ds[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int c = 4 * c4 + e, q = q0 + 32 * hf + c;
+              p[e] = q >= qfirst && q < qlim ? exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lq[e])) : 0.f;
+              ds[e] = p[e] * (__uint_as_float(dr[c]) - dq[e]);
+            }
+            pp[2 * c4] = pack_bf16x2(p[0], p[1]);
+            pp[2 * c4 + 1] = pack_bf16x2(p[2], p[3]);
+            dd[2 * c4] = pack_bf16x2(ds[0], ds[1]);
+            dd[2 * c4 + 1] = pack_bf16x2(ds[2], ds[3]);
+          }
+          tmem_st16(t_lane + qh * 64 + 16 * hf, pp);
+          tmem_st16(t_lane + 128 + qh * 64 + 16 * hf, dd);
+        }
+        if (next) {
+          if (!taken(un, unn)) break;
+          if (unn >= 0) tnn = tile_word(unn);
+        }
+      } else {
+        // every key of the warp visible to all 64 queries: no masks
+        const bool open = __all_sync(0xffffffffu, qfirst <= q0 && qlim >= q0 + 64);
+        // ---- P^T of key row r for queries qh * 64 .. + 63, in two groups of 32, kept in registers
+        // and written (bf16 pairs) into the 16 columns at 64 qh + 16 hf of the S^T just read
+        float p[64];
+        auto probs = [&](auto masked) {
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t sr[32];
+            tmem_ld32(t_lane + qh * 64 + 32 * hf, sr);
+            tmem_ld_wait();
+            const float4* L4 = reinterpret_cast<const float4*>(sL + qh * 64 + 32 * hf);
+            uint32_t pp[16];
+#pragma unroll
+            for (int c4 = 0; c4 < 8; ++c4) {
+              const float4 l4 = L4[c4];
+              const float lq[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const int c = 4 * c4 + e, q = q0 + 32 * hf + c;
+                const float pv = exp2_hw(fmaf(__uint_as_float(sr[c]), scale_log2, -lq[e]));
+                p[32 * hf + c] = !masked.value || (q >= qfirst && q < qlim) ? pv : 0.f;
+              }
+              pp[2 * c4] = pack_bf16x2(p[32 * hf + 4 * c4], p[32 * hf + 4 * c4 + 1]);
+              pp[2 * c4 + 1] = pack_bf16x2(p[32 * hf + 4 * c4 + 2], p[32 * hf + 4 * c4 + 3]);
+            }
+            tmem_st16(t_lane + qh * 64 + 16 * hf, pp);
+          }
+        };
+        if (open) probs(std::false_type{});
+        else probs(std::true_type{});
+        if (it == w.it0 && next) {
+          if (!taken(un, unn)) break;
+          if (unn >= 0) tnn = tile_word(unn);
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        if (!wait_all(B_DP, FL_DEV_TIMEOUT_ACC_FULL)) break;
+        tc_fence_after();
+        // ---- dV += P^T dO (A from TMEM) while dS^T is made; the unit's last reader of K and V is done.
+        // A unit's last tile has no later products to make room for, and the issuing warp's dS^T would
+        // be what the others wait for: its dV goes with dK.  32 x 256 tokens 234 -> 228 us, 16 x 512 295 ->
+        // 288, segments of 67 to 2048 335 -> 329 (late on every tile: 234, 296, 340).
+        if (warp == 0) {
+          if (last && next) issue_kv(wn);
           __syncwarp();
+          if (!last) {
+            tr.arm(B_DV);
+            add_dv();
+            if (elect_one()) umma_commit(bars + B_DV);
+            __syncwarp();
+          }
         }
-      }
-      // ---- dS^T, written the same way over dP^T
+        // ---- dS^T, written the same way over dP^T
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        uint32_t dr[32];
-        tmem_ld32(t_lane + 128 + qh * 64 + 32 * hf, dr);
-        tmem_ld_wait();
-        const float4* D4 = reinterpret_cast<const float4*>(sD + qh * 64 + 32 * hf);
-        uint32_t dd[16];
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t dr[32];
+          tmem_ld32(t_lane + 128 + qh * 64 + 32 * hf, dr);
+          tmem_ld_wait();
+          const float4* D4 = reinterpret_cast<const float4*>(sD + qh * 64 + 32 * hf);
+          uint32_t dd[16];
 #pragma unroll
-        for (int c4 = 0; c4 < 8; ++c4) {
-          const float4 d4 = D4[c4];
-          const float dq[4] = {d4.x, d4.y, d4.z, d4.w};
-          float ds[4];
+          for (int c4 = 0; c4 < 8; ++c4) {
+            const float4 d4 = D4[c4];
+            const float dq[4] = {d4.x, d4.y, d4.z, d4.w};
+            float ds[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) ds[e] = p[32 * hf + 4 * c4 + e] * (__uint_as_float(dr[4 * c4 + e]) - dq[e]);
-          dd[2 * c4] = pack_bf16x2(ds[0], ds[1]);
-          dd[2 * c4 + 1] = pack_bf16x2(ds[2], ds[3]);
+            for (int e = 0; e < 4; ++e) ds[e] = p[32 * hf + 4 * c4 + e] * (__uint_as_float(dr[4 * c4 + e]) - dq[e]);
+            dd[2 * c4] = pack_bf16x2(ds[0], ds[1]);
+            dd[2 * c4 + 1] = pack_bf16x2(ds[2], ds[3]);
+          }
+          tmem_st16(t_lane + 128 + qh * 64 + 16 * hf, dd);
         }
-        tmem_st16(t_lane + 128 + qh * 64 + 16 * hf, dd);
       }
       tmem_st_wait();
       tc_fence_before();
@@ -1014,8 +1063,9 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
                   const AttnPrefix& pre, const AttnGlm& glm, float* dbias, int* status, cudaStream_t st,
                   int dbias_segs, int64_t dbias_rstride) {
   FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dq_tc_kernel<HD>, BwdCfg<HD>::SMEM));
-  FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dkv_tc_kernel<HD, false>, BwdCfg<HD>::SMEM));
-  FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dkv_tc_kernel<HD, true>, BwdCfg<HD>::SMEM));
+  FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dkv_tc_kernel<HD, false, false>, BwdCfg<HD>::SMEM));
+  FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dkv_tc_kernel<HD, false, true>, BwdCfg<HD>::SMEM));
+  FL_CUDA_TRY(fl_func_smem((const void*)attn_bwd_dkv_tc_kernel<HD, true, false>, BwdCfg<HD>::SMEM));
   const int H = nh * HD;
   CUtensorMap tq, tdo, tpk, tpv, tdq;
   if (int rc = fl_gemm::make_map(&tq, qkv, (uint64_t)3 * H, (uint64_t)T, 3 * (int64_t)H, 128)) return rc;
@@ -1033,14 +1083,15 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
   // One CTA is resident per SM (512 TMEM columns).  Units of different cost (segments of three
   // tiles and more: a unit walks 1 .. that many) are handed out as CTAs finish: segments of 67 to
   // 2048 tokens 362 -> 331 us, 4 x 512 106 -> 98, 8 x 1024 422 -> 411; a fixed walk is enough for
-  // even ones and spares them the requests: 40 x 190 tokens 262 against 273 us, 64 x 64 181 / 183.
+  // even ones and spares them the requests: 40 x 190 tokens 262 against 273 us.
   const int n_units = n_tiles * nh, sms = fl_sm_count();
   const int grid = max_tiles >= 3 || n_units < sms ? n_units : sms;
   if (n_units > 0) {
     FL_CUDA_TRY(fl_launch(attn_bwd_dq_tc_kernel<HD>, dim3(grid), dim3(256), BwdCfg<HD>::SMEM, st, tq, tdo, tpk, tpv,
                           tdq, T, H, cu, tiles, n_units, lse, delta, tab, scale, scale * LOG2E_B, pre.len, (bf16*)dqkv,
                           glm.ctx, glm.pos, glm.pos2, dbias, dbias_segs, dbias_rstride, status));
-    FL_CUDA_TRY(fl_launch(attn_bwd_dkv_tc_kernel<HD, false>, dim3(grid), dim3(256), BwdCfg<HD>::SMEM, st, tq, tdo,
+    const auto dkv = max_tiles == 1 ? attn_bwd_dkv_tc_kernel<HD, false, true> : attn_bwd_dkv_tc_kernel<HD, false, false>;
+    FL_CUDA_TRY(fl_launch(dkv, dim3(grid), dim3(256), BwdCfg<HD>::SMEM, st, tq, tdo,
                           tpk, tpv, tdq, T, H, cu, tiles, n_tiles, n_units, 0, lse, delta, tab, scale, scale * LOG2E_B, 0,
                           (bf16*)dqkv, (float*)nullptr, (float*)nullptr, glm.ctx, glm.pos, glm.pos2, dbias,
                           dbias_segs, dbias_rstride, status));
@@ -1048,7 +1099,7 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
   if (pre.len > 0 && n_tiles > 0) {
     // the prefix keys of each head against slices of the query tiles, about one CTA per SM
     const int per = slice_tiles(n_tiles, (fl_sm_count() + nh - 1) / nh), nsplit = slices(n_tiles, per);
-    FL_CUDA_TRY(fl_launch(attn_bwd_dkv_tc_kernel<HD, true>, dim3(nsplit * nh), dim3(256), BwdCfg<HD>::SMEM, st, tq,
+    FL_CUDA_TRY(fl_launch(attn_bwd_dkv_tc_kernel<HD, true, false>, dim3(nsplit * nh), dim3(256), BwdCfg<HD>::SMEM, st, tq,
                           tdo, tpk, tpv, tdq, T, H, cu, tiles, n_tiles, nsplit * nh, per, lse, delta, tab, scale,
                           scale * LOG2E_B, pre.len, (bf16*)dqkv, pre.dk, pre.dv, glm.ctx, glm.pos, glm.pos2,
                           (float*)nullptr, 0, (int64_t)0, status));

@@ -405,10 +405,11 @@ def test_attention_bwd_many_units(F, hd):
 
 
 @pytest.mark.parametrize("hd", [64, 128])
-@pytest.mark.parametrize("seqs", [[256] * 10 + [1, 130], [256] * 6 + [1, 300, 130, 700]])
+@pytest.mark.parametrize("seqs", [[256] * 10 + [1, 130], [256] * 6 + [1, 300, 130, 700], [128] * 11 + [1, 77, 64]])
 def test_attention_bwd_unit_order(F, hd, seqs):
     """Units taken in a fixed stride (two tiles per segment at most) or handed out while the
-    kernel runs (three and more), several per SM: the bits of every segment alone."""
+    kernel runs (three and more), several per SM, probabilities and score gradients made in two
+    passes or (one tile per segment, as short ones alone) in one: the bits of every segment alone."""
     nh = 16
     H, rd = nh * hd, hd // 2
     g = torch.Generator(device="cuda").manual_seed(hd + len(seqs))

@@ -54,7 +54,7 @@ def test_products_wait_for_the_readers_of_their_columns():
     dkv = _kernel(src, "attn_bwd_dkv_tc_kernel")
     loop = dkv[dkv.index("for (int it = w.it0"):]
     # in the loop: dP^T behind the CTA-wide wait for S^T, S^T behind the wait for dV
-    assert loop.index("wait_all(B_S,") < loop.index("scores(b, 1)") < loop.index("scores(1 - b, 0)")
+    assert loop.index("wait_all(ONE ? B_DP : B_S,") < loop.index("scores(b, 1)") < loop.index("scores(1 - b, 0)")
     assert loop.index("mbar_wait_warp(bars + B_DV, tr.parity(B_DV))") < loop.index("scores(1 - b, 0)")
     assert len(re.findall(r"\bscores\(", loop)) == 2
     dq = _kernel(src, "attn_bwd_dq_tc_kernel")
