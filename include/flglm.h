@@ -83,7 +83,7 @@ typedef struct {
                              * gradient GEMMs when the pending call has at least this many
                              * tokens, else it runs the backward and then fl_server_step;
                              * 0 -> the library's choice (fused at every token count where a
-                             * block holds 2^24 matrix weights or more, as measured on GB300);
+                             * block holds 2^23 matrix weights or more, as measured on GB300);
                              * 1 -> always fused */
   int32_t n_replicas;       /* server-hierarchical strategy (§3.3) on one GPU: 0 or 1 = one
                              * server; 2..4 = that many replicas in one handle, each with its

@@ -111,10 +111,12 @@ namespace {
 // Matrix weights per block from which fl_server_backward_step fuses the AdamW update into the
 // weight-gradient GEMMs (at every token count), unless cfg.fused_step_min_tokens says otherwise.
 // Measured on GB300, one block, fused / separate step: H 4096 (201M weights) 1.45 / 1.61 ms at 128
-// tokens, 1.79 / 2.02 at 1024, 3.21 / 3.58 at 3072; H 2048 (50M) 563 / 590, 673 / 719, 1237 / 1296
-// us; H 1024 (12.6M) 302 / 303, 348 / 350, 567 / 565; H 512 203 / 196; H 256 184 / 170 (a small
-// weight's update costs less than the longer epilogue).
-constexpr int64_t FL_FUSED_STEP_MIN_WEIGHTS = int64_t(1) << 24;
+// tokens, 1.79 / 2.02 at 1024, 3.21 / 3.58 at 3072; H 2048 (50M) 535 / 579 us at 512, 1321 / 1446 at
+// 4608, 3932 / 4114 at 16384; H 1024 (12.6M) 228 / 229 at 64, 269 / 268 at 512, 554 / 553 at 3072, 671 /
+// 683 at 4608, 1023 / 1055 at 8192, 1818 / 1862 at 16384; H 512 (3.1M) 172 / 168 at 512, 383 / 377 at
+// 4608, 1012 / 1016 at 16384; H 256 156 / 141, 276 / 250, 712 / 648 (a small weight's update costs less
+// than the longer epilogue).
+constexpr int64_t FL_FUSED_STEP_MIN_WEIGHTS = int64_t(1) << 23;
 
 constexpr uint64_t GOLDEN = 0x9E3779B97F4A7C15ull;
 uint64_t mix64_host(uint64_t z) {

@@ -206,6 +206,26 @@ def test_backward_step_below_the_fusion_crossover(F):
     b.close()
 
 
+def test_backward_step_default_at_hidden_1024(F):
+    """Hidden 1024 (12.6M matrix weights per block): what the library picks by itself against the
+    separate update, over two steps (up to the rounding of the atomic bias sums)."""
+    cfg = syn.CONFIGS["tiny"].with_(hidden=1024, n_heads=16, ffn_hidden=4096, client_batch=1, seq_lens=(300, 77))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    states = [torch.randn((1, n, 1024), generator=g, device="cuda").bfloat16() for n in cfg.seq_lens]
+    grads = [(1e-3 * torch.randn((1, n, 1024), generator=g, device="cuda")).bfloat16() for n in cfg.seq_lens]
+    a, b = (make_server(F, cfg, fused_step_min_tokens=n) for n in (0, 1 << 30))
+    for _ in range(2):
+        for srv in (a, b):
+            outs, gi = [torch.empty_like(x) for x in states], [torch.empty_like(x) for x in states]
+            srv.forward(states, cfg.seq_lens, outs)
+            srv.backward_step(grads, gi, 1e-3)
+            srv.sync()
+    for t in range(12):
+        assert rel_inf(a.get_param(0, t), b.get_param(0, t)) < 1e-5, t
+    a.close()
+    b.close()
+
+
 def test_ragged_small_parity(F):
     cfg = syn.CONFIGS["tiny"].with_(n_blocks=2, client_batch=1, seq_lens=(1, 17, 64, 65, 130, 3))
     parity_case(F, cfg)
