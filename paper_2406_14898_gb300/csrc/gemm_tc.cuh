@@ -440,8 +440,8 @@ FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int wa
   uint32_t cs_par = 0;  // parity of the column sums' barriers
   for (int tile = t0; tile < num_tiles; tile += step, ++local) {
     const int acc = local & 1;
-    if (!mbar_wait(&acc_full[acc], (local >> 1) & 1)) {
-      report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+    if (!mbar_wait_warp(&acc_full[acc], (local >> 1) & 1)) {
+      if (lane == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
       return;
     }
     tc_fence_after();
@@ -501,8 +501,8 @@ FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int wa
         uint64_t* written = cs_bars + 2 * ((warp - 2) >> 2);
         if (lane == 0) mbar_arrive(written);
         if (wi == 0) {
-          if (!mbar_wait(written, cs_par)) {
-            report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+          if (!mbar_wait_warp(written, cs_par)) {
+            if (lane == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
             return;
           }
           if (h == 0) {
@@ -516,8 +516,8 @@ FL_DEV void epilogue_loop(const Epi& e, float* stage, uint32_t tmem_base, int wa
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(written + 1);
-        } else if (!mbar_wait(written + 1, cs_par)) {
-          report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
+        } else if (!mbar_wait_warp(written + 1, cs_par)) {
+          if (lane == 0) report_status(status, FL_DEV_TIMEOUT_ACC_FULL);
           return;
         }
         cs_par ^= 1;

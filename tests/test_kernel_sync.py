@@ -72,3 +72,13 @@ def test_given_up_waits_end_behind_every_product():
         end = re.search(r"if \(!ok && warp == 0\) \{\s*if \(elect_one\(\)\) umma_commit\(bars \+ B_END\);\s*"
                         r"mbar_wait_warp\(bars \+ B_END, 0\);\s*\}", body)
         assert end and max(m.start() for m in re.finditer(r"umma_bf16", body)) < end.start() < body.index("tmem_dealloc")
+
+
+def test_warp_wide_loops_agree_on_an_expired_wait():
+    """GEMM epilogues: their loops hold warp-wide TMEM reads, so a wait that gives up does so for the
+    whole warp; a lane alone must not leave the loop."""
+    src = _code("gemm_tc.cuh")
+    for name in ("epilogue_loop", "adamw_epilogue", "f32_epilogue"):
+        body = _kernel(src, name)
+        waits = re.findall(r"if \(!(.*?mbar_wait\w*)\(", body)
+        assert waits and all(w in ("mbar_wait_warp", "__all_sync(0xffffffffu, mbar_wait") for w in waits), name
