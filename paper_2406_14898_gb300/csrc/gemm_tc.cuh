@@ -956,10 +956,9 @@ __global__ void __launch_bounds__(EpiCfg<FAM, BN>::THREADS, 1)
 constexpr int PAIR_BM = 256;
 template <int PBN, int FAM>
 struct CfgPair {
-  static constexpr int KSUB = 1;
   static constexpr int A_BYTES = 128 * BK * 2;        // this CTA's 128 rows of A
   static constexpr int B_BYTES = (PBN / 2) * BK * 2;  // this CTA's columns of B
-  static constexpr int STAGE_BYTES = KSUB * (A_BYTES + B_BYTES);
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = ring_stages(STAGE_BYTES, EpiCfg<FAM, PBN>::BYTES);
   static constexpr int TMEM_COLS = 2 * PBN;  // double-buffered accumulator
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EpiCfg<FAM, PBN>::BYTES + BAR_BYTES + 1024 /*align*/;
@@ -971,11 +970,11 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ GemmMaps<FAM> maps, Epi epi, int M, int N, int K, int batch, Raster raster,
                      int* status) {
   using C = CfgPair<PBN, FAM>;
-  constexpr int STAGES = C::STAGES, KSUB = C::KSUB;
+  constexpr int STAGES = C::STAGES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + STAGES * KSUB * C::A_BYTES;
+  uint8_t* sB = smem + STAGES * C::A_BYTES;
   uint8_t* epi_smem = smem + STAGES * C::STAGE_BYTES;
   uint64_t* bars = reinterpret_cast<uint64_t*>(epi_smem + EpiCfg<FAM, PBN>::BYTES);
   uint64_t* full = bars;
@@ -1038,7 +1037,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
       const CUtensorMap* tmA = &maps.a[r];
       const CUtensorMap* tmB = &maps.b[r];
       const int m0 = mb * PAIR_BM + int(rank) * 128, n0 = nb * PBN + int(rank) * (PBN / 2);
-      for (int kb = 0; kb < num_k; kb += KSUB) {
+      for (int kb = 0; kb < num_k; ++kb) {
         if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
           if (lane == 0) report_status(status, FL_DEV_TIMEOUT_EMPTY);
           ok = false;
@@ -1047,23 +1046,20 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
         if (elect_one()) {
           if (leader) mbar_arrive_expect_tx(&full[stage], 2 * C::STAGE_BYTES);
           const uint32_t fb = full0 + 8u * stage;
+          const int k0 = kb * BK;
+          uint8_t* a_dst = sA + stage * C::A_BYTES;
+          uint8_t* b_dst = sB + stage * C::B_BYTES;
+          if (!A_MN) {
+            tma_load_2d_pair(a_dst, tmA, fb, k0, m0);
+          } else {
+            tma_load_2d_pair(a_dst, tmA, fb, m0, k0);
+            tma_load_2d_pair(a_dst + 64 * BK * 2, tmA, fb, m0 + 64, k0);
+          }
+          if (!B_MN) {
+            tma_load_2d_pair(b_dst, tmB, fb, k0, n0);
+          } else {
 #pragma unroll
-          for (int q = 0; q < KSUB; ++q) {  // a k-block past K reads zeros
-            const int k0 = (kb + q) * BK;
-            uint8_t* a_dst = sA + (stage * KSUB + q) * C::A_BYTES;
-            uint8_t* b_dst = sB + (stage * KSUB + q) * C::B_BYTES;
-            if (!A_MN) {
-              tma_load_2d_pair(a_dst, tmA, fb, k0, m0);
-            } else {
-              tma_load_2d_pair(a_dst, tmA, fb, m0, k0);
-              tma_load_2d_pair(a_dst + 64 * BK * 2, tmA, fb, m0 + 64, k0);
-            }
-            if (!B_MN) {
-              tma_load_2d_pair(b_dst, tmB, fb, k0, n0);
-            } else {
-#pragma unroll
-              for (int j = 0; j < PBN / 128; ++j) tma_load_2d_pair(b_dst + j * 64 * BK * 2, tmB, fb, n0 + 64 * j, k0);
-            }
+            for (int j = 0; j < PBN / 128; ++j) tma_load_2d_pair(b_dst + j * 64 * BK * 2, tmB, fb, n0 + 64 * j, k0);
           }
         }
         __syncwarp();
@@ -1097,7 +1093,7 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * PBN;
-        for (int kb = 0; kb < num_k; kb += KSUB) {
+        for (int kb = 0; kb < num_k; ++kb) {
           if (!mbar_wait_warp(&full[stage], phase)) {
             if (lane == 0) report_status(status, FL_DEV_TIMEOUT_FULL);
             ok = false;
@@ -1105,18 +1101,14 @@ __global__ void __launch_bounds__(EpiCfg<FAM, PBN>::THREADS, 1)
           }
           tc_fence_after();
           if (elect_one()) {
+            const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + stage * C::A_BYTES));
+            const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + stage * C::B_BYTES));
 #pragma unroll
-            for (int q = 0; q < KSUB; ++q) {
-              if (KSUB > 1 && kb + q >= num_k) break;
-              const uint64_t ad = stage_desc<A_MN>(smem_u32(sA + (stage * KSUB + q) * C::A_BYTES));
-              const uint64_t bd = stage_desc<B_MN>(smem_u32(sB + (stage * KSUB + q) * C::B_BYTES));
-#pragma unroll
-              for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                umma_bf16_pair(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC,
-                               (kb | q | kk) != 0 ? 1u : 0u);
-            }
+            for (int kk = 0; kk < BK / UMMA_K; ++kk)
+              umma_bf16_pair(d_tmem, ad + kk * kstep_desc<A_MN>(), bd + kk * kstep_desc<B_MN>(), IDESC,
+                             (kb | kk) != 0 ? 1u : 0u);
             umma_commit_pair(&empty[stage], 3);
-            if (kb + KSUB >= num_k) umma_commit_pair(&acc_full[acc], 3);
+            if (kb + 1 == num_k) umma_commit_pair(&acc_full[acc], 3);
           }
           __syncwarp();
           if (++stage == STAGES) {
