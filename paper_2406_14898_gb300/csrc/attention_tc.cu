@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
   constexpr int NB = FwdCfg<HD>::NB, TILE = FwdCfg<HD>::TILE;
   // P's 64 columns: the last ones at head_dim 64, the first of S at 128, where O fills the others
   constexpr uint32_t T_P = HD == 64 ? 192 : 0;
+  constexpr bool pv_waited = T_P == 0;  // the next S is issued behind a wait for P V
   pdl_wait();  // the previous kernel on the stream has completed (see fl_launch)
   pdl_trigger();
   extern __shared__ uint8_t smem_raw[];
@@ -261,14 +262,14 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
       // ---- O += P V_j
       if (warp == 0) {
         tc_fence_after();
-        tr.arm(B_PV);
+        if (pv_waited || last) tr.arm(B_PV);
         __syncwarp();
         if (elect_one()) {
           const uint64_t bv = desc_mnmajor(smem_u32(sV));
 #pragma unroll
           for (int kk = 0; kk < TB / 16; ++kk)
             umma_bf16_ts(tmem + 128, tmem + T_P + kk * 8, bv + step_mnmajor(kk), IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(bars + B_PV);
+          if (pv_waited || last) umma_commit(bars + B_PV);
         }
         __syncwarp();
       }
@@ -278,9 +279,9 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(
       if (!last || next) {
         if (last && !wait_all(B_Q, FL_DEV_TIMEOUT_FULL)) break;
         if (!wait_all(B_K, FL_DEV_TIMEOUT_FULL)) break;
-        if (warp == 0 && (T_P != 0 || mbar_wait_warp(bars + B_PV, tr.parity(B_PV)))) score();
+        if (warp == 0 && (!pv_waited || mbar_wait_warp(bars + B_PV, tr.parity(B_PV)))) score();
       }
-      if (!last) tr.waited(B_PV);  // it is complete once the next S is
+      if (pv_waited && !last) tr.waited(B_PV);  // it is complete once the next S is
     }
     if (!ok || !wait_all(B_PV, FL_DEV_TIMEOUT_ACC_EMPTY)) break;
     tc_fence_after();

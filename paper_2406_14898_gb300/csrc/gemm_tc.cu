@@ -204,9 +204,10 @@ bool d_is_f32(const fl_gemm_args* a) {
 // The tile shape with the least estimated time: waves of tiles, each as long as its main loop
 // or its epilogue, and the fill and last epilogue.  Measured on GB300 (ns per 64-deep k-block
 // of a CTA or pair with one tile at a time; us for the fixed part): 256 x 256 on a pair 295 and
-// 9.7, 256 x 128 on a pair 230 and 5.4, 128 x 128 262 and 6.1, 128 x 64 180 and 5.0 (the fixed
-// parts of the narrow tiles set so that H 256 steps take 128 x 64: 119 us, 135 on pairs).  So one
-// wave of narrow tiles over all SMs beats a wide tile on a few of them: 4096 columns, K = 16384
+// 9.7, 256 x 128 on a pair 230 and 5.4, 128 x 128 262 and 6.1, 128 x 64 180 and 5.0 (the two narrow
+// tiles' fixed parts chosen by the H 256 step, which takes 119 us on 128 x 64 and 137 where the pair
+// tile's 5.4 is set to 4.0; alone with operands in L2, K 256 .. 4096, they measure 5.0 and 4.6, the
+// others 6.3 and 4.6, the k-blocks 263, 170, 230 and 150 ns).  So one wave of narrow tiles over all SMs beats a wide tile on a few of them: 4096 columns, K = 16384
 // take 85 / 63 / 73 / 51 us (in that order) at 77 rows, 87 / 65 / 75 / 96 at 512; and wide tiles
 // win once they fill the device: 170 / 224 / 271 / 319 us at 2048 rows.
 int pick_shape(const fl_gemm_args* a, int batch, int fam, int pairs) {

@@ -26,7 +26,7 @@ def F():
 
 def make_server(F, cfg, max_tokens=None, seed=None, fused_step_min_tokens=1):
     """fused_step_min_tokens=1: fl_server_backward_step always takes the fused path (the
-    test shapes are far below the library's crossover)."""
+    test blocks hold far fewer weights than the library fuses by itself)."""
     mt = max_tokens or cfg.tokens
     return F.Server(F.make_cfg(cfg, mt, fused_step_min_tokens=fused_step_min_tokens),
                     cfg.seed if seed is None else seed)
@@ -184,7 +184,7 @@ def test_fused_step_equals_backward_then_step(F):
 
 
 def test_backward_step_below_the_fusion_crossover(F):
-    """With the library's default crossover a small call takes backward + step inside
+    """By default a block of few weights takes backward + step inside
     fl_server_backward_step; two steps of it give the weights of the forced fused path
     (up to the rounding of the atomic bias sums)."""
     cfg = syn.CONFIGS["tiny"].with_(n_blocks=2, seq_lens=(64, 40))

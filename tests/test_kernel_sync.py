@@ -49,7 +49,8 @@ def test_products_wait_for_the_readers_of_their_columns():
     dK reads (behind the next S^T, committed after dK); dQ's dS has columns of its own."""
     fwd = _kernel(_code("attention_tc.cu"), "attn_fwd_tc_kernel")
     p_over_s = re.search(r"T_P = HD == 64 \? 192 : 0;", fwd)
-    assert p_over_s and "if (warp == 0 && (T_P != 0 || mbar_wait_warp(bars + B_PV, tr.parity(B_PV)))) score();" in fwd
+    assert p_over_s and "pv_waited = T_P == 0;" in fwd
+    assert "if (warp == 0 && (!pv_waited || mbar_wait_warp(bars + B_PV, tr.parity(B_PV)))) score();" in fwd
     src = _code("attention_bwd_tc.cu")
     dkv = _kernel(src, "attn_bwd_dkv_tc_kernel")
     loop = dkv[dkv.index("for (int it = w.it0"):]
