@@ -95,8 +95,9 @@ typedef struct {
                                                [rotary_dim, 2*rotary_dim) of each q/k head then turn
                                                by pos2 (2D rotary; needs rotary_dim = head_dim/2) */
   int32_t tile;                             /* FL_TILE_*: tile shape, FL_TILE_AUTO (0) lets the library
-                                               pick (256-column tiles on CTA pairs unless smaller tiles
-                                               leave clearly fewer SMs idle in the last wave) */
+                                               pick the one of least estimated time, among these and
+                                               narrow ones (128 x 64, 256 x 128 on a pair);
+                                               every tile sums over K in the same order */
   float* colsum;                            /* FL_EPI_GELU_BWD only, or NULL: colsum[n] += sum over m of
                                                D[m,n] (fp32, before rounding; fp32 atomics, so the
                                                order of the additions is not fixed); 16-byte aligned */

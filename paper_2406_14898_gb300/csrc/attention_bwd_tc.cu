@@ -1082,7 +1082,7 @@ int launch_bwd_tc(int T, int nh, const void* qkv, const void* dout, const float*
   const float2* tab = reinterpret_cast<const float2*>(rope_tab);
   // One CTA is resident per SM (512 TMEM columns).  Units of different cost (segments of three
   // tiles and more: a unit walks 1 .. that many) are handed out as CTAs finish: segments of 67 to
-  // 2048 tokens 362 -> 331 us, 4 x 512 106 -> 98, 8 x 1024 422 -> 411; a fixed walk is enough for
+  // 2048 tokens 362 -> 332 us, 4 x 512 106 -> 99, 8 x 1024 422 -> 414; a fixed walk is enough for
   // even ones and spares them the requests: 40 x 190 tokens 262 against 273 us.
   const int n_units = n_tiles * nh, sms = fl_sm_count();
   const int grid = max_tiles >= 3 || n_units < sms ? n_units : sms;

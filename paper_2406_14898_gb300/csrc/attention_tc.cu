@@ -19,7 +19,7 @@
 // Shared memory: three tiles (96 KB at head_dim 128); 256 TMEM columns: two CTAs per SM
 // overlap each other's copies and softmax.  Bound at 256-token segments by HBM (8 H bytes per
 // token), at long ones by the softmax threads: 32 x 256 tokens x
-// 32 heads 72 -> 65 us, 4.2 TB/s; 4 x 2048 tokens 249 -> 196 us, 700 TFLOP/s (before: loads only
+// 32 heads 72 -> 65 us, 4.2 TB/s; 4 x 2048 tokens 249 -> 197 us, 697 TFLOP/s (before: loads only
 // after a unit's last product, every product waited for, 16-byte stores of half sectors).
 // Every mbarrier wait is bounded (2 s): on expiry the CTA records a status code and leaves its
 // remaining work undone.
